@@ -200,8 +200,6 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 }
 
 // ---------------------------------------------------------------- cross-TU entry points
-int hd_knn_impl(hd_ctx* ctx, const void* Xd, int64_t n, int32_t d, int dtype, const void* Qd,
-                int64_t nq, int32_t k, int exclude_self, int32_t* idx_d, float* sim_d);
 int hd_graph_from_lists(hd_ctx* ctx, int64_t n, int32_t k, const int32_t* idx_d, const float* sim_d,
                         float gamma, int sym, hd_graph** out);
 int hd_normalize_graph(hd_ctx* ctx, hd_graph* g);
