@@ -49,113 +49,6 @@ int hd_make_tmap_2d(CUtensorMap* map, const void* base, int elem_bytes, uint64_t
 
 constexpr int KMAX = 64;  // neighbours per list
 
-// ------------------------------------------------------------------ list insertion
-// Insert (s, id) into a row's list kept sorted by (-s, id).  Returns new k-th score.
-__device__ __noinline__ float list_insert_ordered(float* ls, int32_t* li, int k, float s, int32_t id) {
-    int p = k - 1;
-    while (p > 0 && (ls[p - 1] < s || (ls[p - 1] == s && li[p - 1] > id))) {
-        ls[p] = ls[p - 1];
-        li[p] = li[p - 1];
-        --p;
-    }
-    ls[p] = s;
-    li[p] = id;
-    return ls[k - 1];
-}
-
-// ------------------------------------------------------------------ fp32 CUDA-core kNN
-namespace {
-constexpr int FB = 64;   // queries and database rows per tile
-constexpr int FK = 16;   // depth chunk
-}
-
-__global__ void __launch_bounds__(256) k_knn_f32(const float* __restrict__ X, int64_t n, int d,
-                                                 const float* __restrict__ Q, int64_t nq, int k, int excl,
-                                                 int32_t* __restrict__ idx_out, float* __restrict__ sim_out) {
-    __shared__ float As[FK][FB + 4];
-    __shared__ float Bs[FK][FB + 4];
-    __shared__ float ls[FB][KMAX];
-    __shared__ int32_t li[FB][KMAX];
-    __shared__ float cs[FB][FB];
-    __shared__ int32_t cidx[FB][FB];
-    __shared__ int cnt[FB];
-    __shared__ float tau[FB];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int64_t q0 = (int64_t)blockIdx.x * FB;
-    for (int t = tid; t < FB * KMAX; t += 256) {
-        ls[t / KMAX][t % KMAX] = -INFINITY;
-        li[t / KMAX][t % KMAX] = -1;
-    }
-    if (tid < FB) {
-        cnt[tid] = 0;
-        tau[tid] = -INFINITY;
-    }
-    __syncthreads();
-    for (int64_t t0 = 0; t0 < n; t0 += FB) {
-        float acc[4][4] = {};
-        for (int kc = 0; kc < d; kc += FK) {
-            for (int e = tid; e < FB * FK; e += 256) {
-                int r = e / FK, c = e % FK;
-                int64_t qr = q0 + r, xr = t0 + r;
-                As[c][r] = (qr < nq && kc + c < d) ? Q[qr * d + kc + c] : 0.0f;
-                Bs[c][r] = (xr < n && kc + c < d) ? X[xr * d + kc + c] : 0.0f;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int c = 0; c < FK; ++c) {
-                float a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    a[i] = As[c][ty * 4 + i];
-                    b[i] = Bs[c][tx * 4 + i];
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            int r = ty * 4 + i;
-            int64_t qr = q0 + r;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                int64_t id = t0 + tx * 4 + j;
-                float s = acc[i][j];
-                if (qr < nq && id < n && !(excl && id == qr) && s > tau[r]) {
-                    int p = atomicAdd(&cnt[r], 1);
-                    cs[r][p] = s;
-                    cidx[r][p] = (int32_t)id;
-                }
-            }
-        }
-        __syncthreads();
-        if (tid < FB) {
-            int r = tid;
-            float th = tau[r];
-            for (int c = 0; c < cnt[r]; ++c) {
-                float s = cs[r][c];
-                int32_t id = cidx[r][c];
-                if (s > ls[r][k - 1] || (s == ls[r][k - 1] && id < li[r][k - 1]))
-                    th = list_insert_ordered(&ls[r][0], &li[r][0], k, s, id);
-            }
-            tau[r] = th;
-            cnt[r] = 0;
-        }
-        __syncthreads();
-    }
-    for (int t = tid; t < FB * k; t += 256) {
-        int r = t / k, c = t % k;
-        int64_t qr = q0 + r;
-        if (qr < nq) {
-            idx_out[qr * k + c] = li[r][c];
-            sim_out[qr * k + c] = ls[r][c];
-        }
-    }
-}
-
 // ------------------------------------------------------------------ top-k selection
 // A (similarity, id) pair is one 64-bit key, ordered like the lists (larger
 // similarity first, then smaller id); 0 is the empty entry, below every real
@@ -252,12 +145,233 @@ __global__ void __launch_bounds__(256) k_knn_merge(const uint64_t* __restrict__ 
     }
 }
 
+// ------------------------------------------------------------------ search arguments
+// A work item is one block of queries against one segment of the database: all
+// of it when there are enough query blocks to fill the GPU, else a share, the
+// per-segment lists meeting in k_knn_merge.  Items are numbered with the query
+// block fastest, so the blocks of one wave read the same database tiles.
+struct KnnArgs {
+    int64_t n, nq;
+    int d, k, excl;
+    int nwork;         // query blocks
+    int nseg, tps;     // database segments and tiles per segment
+    uint64_t* lists;   // [gridDim.x][rows of a query block][64] running lists
+    uint64_t* part;    // [nseg][nq][k] per-segment results (nseg > 1)
+    int32_t* idx_out;  // [nq][k] (nseg == 1)
+    float* sim_out;
+};
+
+// the final list of a row: the result itself, or the segment's part of it
+__device__ __forceinline__ void knn_store(const KnnArgs& a, int seg, int64_t row, const uint64_t* list, int lane) {
+    for (int c = lane; c < a.k; c += 32) {
+        const uint64_t key = list[c];
+        if (a.nseg > 1) {
+            a.part[((int64_t)seg * a.nq + row) * a.k + c] = key;
+        } else {
+            a.idx_out[row * a.k + c] = key_id(key);
+            a.sim_out[row * a.k + c] = key_sim(key);
+        }
+    }
+}
+
+// ------------------------------------------------------------------ fp32 kNN on CUDA cores
+// Exact fp32 products: every similarity is one chain of fused multiply-adds in
+// the order of the dimensions, whatever the tile.  16 x 16 threads hold a tile
+// of 16 TM queries x 128 database rows, TM x 8 per thread; two consecutive
+// database rows share a packed multiply-add.  16 dimensions at a time go
+// through double-buffered shared memory, loaded into registers one step ahead.
+// TM = 8 when there are more than 64 queries; fewer queries take the smallest
+// tile that holds them, so that no product is formed for padding.
+//
+// Bound: the FP32 pipe (127 ms of fused multiply-adds for the lists of 100,000 x
+// 512; 221 ms for the whole graph, from 407 ms with a 64 x 64 tile, 4 x 4 per
+// thread, and one thread inserting per row; 64 queries against 100,000 x 512:
+// 0.40 ms, from 101.5 ms on one SM).  Candidates above a row's threshold are
+// appended to 64 slots of shared memory (32 columns of a row at a time), merged
+// as in k_knn_tc.
+namespace knnf {
+constexpr int BN = 128;      // database rows per tile
+constexpr int FK = 16;       // dimensions per step
+constexpr int BLD = BN + 4;  // leading dimension of the transposed tiles (16-byte rows)
+template <int TM>
+struct Cfg {
+    static constexpr int BM = 16 * TM;
+    static constexpr int ALD = BM + 4;
+    static constexpr int AV = (BM * FK / 4 + 255) / 256;  // float4 loads per thread and step
+    static constexpr size_t SMEM = 2 * (size_t)FK * (ALD + BLD) * 4 + (size_t)BM * KBUF_LD * 8 + BM * 8;
+};
+
+// four dimensions of one row (zero past the end)
+__device__ __forceinline__ float4 load4(const float* p, int64_t row, int64_t rows, int d, int c, bool vec) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row >= rows || c >= d) return v;
+    const float* q = p + row * d + c;
+    if (vec) return __ldg(reinterpret_cast<const float4*>(q));
+    v.x = __ldg(q);
+    if (c + 1 < d) v.y = __ldg(q + 1);
+    if (c + 2 < d) v.z = __ldg(q + 2);
+    if (c + 3 < d) v.w = __ldg(q + 3);
+    return v;
+}
+__device__ __forceinline__ void put4(float* t, int ld, int c, int r, float4 v) {
+    t[c * ld + r] = v.x;
+    t[(c + 1) * ld + r] = v.y;
+    t[(c + 2) * ld + r] = v.z;
+    t[(c + 3) * ld + r] = v.w;
+}
+// the tile row of a thread's i-th query: groups of four rows, 64 apart
+template <int TM>
+__device__ __forceinline__ int tile_row(int ty, int i) {
+    return TM >= 4 ? (i >> 2) * 64 + ty * 4 + (i & 3) : ty * TM + i;
+}
+__device__ __forceinline__ int tile_col(int tx, int j) { return (j >> 2) * 64 + tx * 4 + (j & 3); }
+}  // namespace knnf
+
+template <int TM>
+__global__ void __launch_bounds__(256, 2)
+    k_knn_f32(const float* __restrict__ X, const float* __restrict__ Q, const KnnArgs a, const int vec) {
+    using namespace knnf;
+    using C = Cfg<TM>;
+    constexpr int BM = C::BM, ALD = C::ALD, AV = C::AV;
+    extern __shared__ __align__(16) uint8_t smem_f[];
+    float* As = reinterpret_cast<float*>(smem_f);           // [2][FK][ALD]
+    float* Bs = As + 2 * FK * ALD;                          // [2][FK][BLD]
+    uint64_t* bufs = reinterpret_cast<uint64_t*>(Bs + 2 * FK * BLD);  // [BM][KBUF_LD]
+    float* tau = reinterpret_cast<float*>(bufs + BM * KBUF_LD);       // [BM]
+    int* cnt = reinterpret_cast<int*>(tau + BM);                      // [BM]
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, warp = tid >> 5, lane = tid & 31;
+    const int ntile = (int)((a.n + BN - 1) / BN), nk = (a.d + FK - 1) / FK, nitem = a.nwork * a.nseg;
+    uint64_t* lists = a.lists + (int64_t)blockIdx.x * BM * 64;
+
+    for (int item = blockIdx.x; item < nitem; item += gridDim.x) {
+        const int w = item % a.nwork, seg = item / a.nwork, t0 = seg * a.tps, t1 = min(ntile, t0 + a.tps);
+        const int64_t q0 = (int64_t)w * BM;
+        for (int r = warp; r < BM; r += 8) {
+            lists[r * 64 + lane] = 0ull;
+            lists[r * 64 + lane + 32] = 0ull;
+        }
+        if (tid < BM) {
+            tau[tid] = q0 + tid < a.nq ? -INFINITY : INFINITY;  // a row past the last query takes nothing
+            cnt[tid] = 0;
+        }
+        float4 ar[AV], br[2];
+        auto fetch = [&](int t, int kc) {
+#pragma unroll
+            for (int u = 0; u < AV; ++u) {
+                const int e = tid + u * 256;
+                if (BM * FK / 4 >= 256 || e < BM * FK / 4) ar[u] = load4(Q, q0 + (e >> 2), a.nq, a.d, kc * FK + (e & 3) * 4, vec);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int e = tid + u * 256;
+                br[u] = load4(X, (int64_t)t * BN + (e >> 2), a.n, a.d, kc * FK + (e & 3) * 4, vec);
+            }
+        };
+        auto stash = [&](int b) {
+#pragma unroll
+            for (int u = 0; u < AV; ++u) {
+                const int e = tid + u * 256;
+                if (BM * FK / 4 >= 256 || e < BM * FK / 4) put4(As + b * FK * ALD, ALD, (e & 3) * 4, e >> 2, ar[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int e = tid + u * 256;
+                put4(Bs + b * FK * BLD, BLD, (e & 3) * 4, e >> 2, br[u]);
+            }
+        };
+        fetch(t0, 0);
+        stash(0);
+        __syncthreads();
+        int b = 0;
+        for (int t = t0; t < t1; ++t) {
+            unsigned long long acc[TM][4];  // pairs of fp32: columns 2 jp and 2 jp + 1
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+            for (int kc = 0; kc < nk; ++kc, b ^= 1) {
+                const bool more = kc + 1 < nk || t + 1 < t1;
+                if (more) fetch(kc + 1 < nk ? t : t + 1, kc + 1 < nk ? kc + 1 : 0);
+                const float* at = As + b * FK * ALD;
+                const float* bt = Bs + b * FK * BLD + tx * 4;
+#pragma unroll
+                for (int c = 0; c < FK; ++c) {
+                    const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bt + c * BLD);
+                    const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(bt + c * BLD + 64);
+                    float av[TM];
+#pragma unroll
+                    for (int i = 0; i < TM; i += 4) {
+                        const float* p = at + c * ALD + tile_row<TM>(ty, i);
+                        if constexpr (TM >= 4) {
+                            const float4 v = *reinterpret_cast<const float4*>(p);
+                            av[i] = v.x;
+                            av[i + 1] = v.y;
+                            av[i + 2] = v.z;
+                            av[i + 3] = v.w;
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < TM; ++u) av[u] = p[u];
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) {
+                        unsigned long long aa;
+                        asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(av[i]));
+                        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][0]) : "l"(aa), "l"(b0.x));
+                        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][1]) : "l"(aa), "l"(b0.y));
+                        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][2]) : "l"(aa), "l"(b1.x));
+                        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][3]) : "l"(aa), "l"(b1.y));
+                    }
+                }
+                if (more) stash(b ^ 1);
+                __syncthreads();
+            }
+            // ---- candidates of this tile, 32 columns of every row at a time
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                int most = 0;
+                const int64_t id0 = (int64_t)t * BN + tile_col(tx, 2 * j);
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    const int r = tile_row<TM>(ty, i);
+                    const float th = tau[r];
+                    float v[2];
+                    asm("mov.b64 {%0, %1}, %2;" : "=f"(v[0]), "=f"(v[1]) : "l"(acc[i][j]));
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        if (v[u] > th && id0 + u < a.n && !(a.excl && id0 + u == q0 + r)) {
+                            const int p = atomicAdd(&cnt[r], 1);
+                            bufs[r * KBUF_LD + p] = knn_key(v[u], id0 + u);
+                            most = max(most, p + 1);
+                        }
+                }
+                if (__syncthreads_or(most > KBUF - 32)) {
+                    for (int r = warp; r < BM; r += 8) {
+                        const int rc = cnt[r];
+                        __syncwarp();
+                        if (rc <= KBUF - 32) continue;
+                        const float th = knn_flush(lists + r * 64, bufs + r * KBUF_LD, rc, a.k, lane);
+                        if (lane == 0) {
+                            tau[r] = th;
+                            cnt[r] = 0;
+                        }
+                    }
+                    __syncthreads();
+                }
+            }
+        }
+        __syncthreads();
+        for (int r = warp; r < BM; r += 8) {
+            if (q0 + r >= a.nq) break;
+            if (cnt[r] > 0) knn_flush(lists + r * 64, bufs + r * KBUF_LD, cnt[r], a.k, lane);
+            knn_store(a, seg, q0 + r, lists + r * 64, lane);
+        }
+        __syncthreads();
+    }
+}
+
 // ------------------------------------------------------------------ bf16 tcgen05 kNN
-// A work item is 128 queries against one segment of the database (tps tiles of
-// 256 rows): all of it when there are enough query blocks to fill the GPU,
-// else a share, the per-segment lists meeting in k_knn_merge.  Items are
-// numbered with the query block fastest, so the CTAs of one wave read the same
-// database tiles.
+// 128 queries x 256 database rows per tile, items as above.
 //
 // Bound: the tensor cores when there are many queries, the stream of the
 // database when there are few (64 queries against 1M x 2048: 0.80 ms for the
@@ -279,30 +393,6 @@ constexpr int BUF_BYTES = BM * KBUF_LD * 8;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + BUF_BYTES + 1024 + 256;
 constexpr int THREADS = 192;
 }  // namespace knntc
-
-struct KnnArgs {
-    int64_t n, nq;
-    int d, k, excl;
-    int nwork;         // query blocks
-    int nseg, tps;     // database segments and tiles per segment
-    uint64_t* lists;   // [gridDim.x][128][64] running lists
-    uint64_t* part;    // [nseg][nq][k] per-segment results (nseg > 1)
-    int32_t* idx_out;  // [nq][k] (nseg == 1)
-    float* sim_out;
-};
-
-// the final list of a row: the result itself, or the segment's part of it
-__device__ __forceinline__ void knn_store(const KnnArgs& a, int seg, int64_t row, const uint64_t* list, int lane) {
-    for (int c = lane; c < a.k; c += 32) {
-        const uint64_t key = list[c];
-        if (a.nseg > 1) {
-            a.part[((int64_t)seg * a.nq + row) * a.k + c] = key;
-        } else {
-            a.idx_out[row * a.k + c] = key_id(key);
-            a.sim_out[row * a.k + c] = key_sim(key);
-        }
-    }
-}
 
 __global__ void __launch_bounds__(knntc::THREADS, 1)
     k_knn_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmX, const KnnArgs a,
@@ -529,15 +619,20 @@ static KnnPlan knn_plan(int64_t nq, int64_t ntile, int bm, int slots, int k, int
     p.grid = (int)std::min<int64_t>((int64_t)p.nwork * p.nseg, slots);
     return p;
 }
-static KnnPlan knn_plan_tc(const hd_ctx* ctx, int64_t n, int64_t nq, int k) {
+// queries per thread of the fp32 kernel: the smallest tile that holds them all
+static int knn_f32_tm(int64_t nq) { return nq <= 16 ? 1 : nq <= 32 ? 2 : nq <= 64 ? 4 : 8; }
+static int knn_bm(int64_t nq, int dtype) { return dtype == HD_F32 ? 16 * knn_f32_tm(nq) : knntc::BM; }
+static KnnPlan knn_plan_for(const hd_ctx* ctx, int64_t n, int64_t nq, int k, int dtype) {
+    if (dtype == HD_F32)
+        return knn_plan(nq, (n + knnf::BN - 1) / knnf::BN, knn_bm(nq, dtype), 2 * ctx->num_sms, k, 2);
     return knn_plan(nq, (n + knntc::BN - 1) / knntc::BN, knntc::BM, ctx->num_sms, k, 4);
 }
 
 // Workspace bytes hd_knn_impl needs for a search (its `scratch`).
 static size_t knn_scratch_bytes(const hd_ctx* ctx, int64_t n, int64_t nq, int32_t k, int dtype) {
-    if (dtype != HD_BF16 || k < 1 || k > KMAX || nq <= 0 || n <= 0) return 256;
-    const KnnPlan p = knn_plan_tc(ctx, n, nq, k);
-    return ws_size((size_t)p.grid * knntc::BM * 64 * 8) + (p.nseg > 1 ? ws_size((size_t)p.nseg * nq * k * 8) : 0);
+    if (k < 1 || k > KMAX || nq <= 0 || n <= 0) return 256;
+    const KnnPlan p = knn_plan_for(ctx, n, nq, k, dtype);
+    return ws_size((size_t)p.grid * knn_bm(nq, dtype) * 64 * 8) + (p.nseg > 1 ? ws_size((size_t)p.nseg * nq * k * 8) : 0);
 }
 
 // Enqueue a search on the context's stream; `scratch` holds knn_scratch_bytes.
@@ -547,23 +642,10 @@ static int hd_knn_impl(hd_ctx* ctx, const void* Xd, int64_t n, int32_t d, int dt
     ctx->h_poll[1] = 0;
     if (k < 1 || k > KMAX) return hd_fail(ctx, HD_ERR_INVALID_ARG, "k=%d outside [1, %d]", k, KMAX);
     if (nq <= 0 || n <= 0) return HD_OK;
-    if (dtype == HD_F32) {
-        k_knn_f32<<<ceil_div(nq, FB), 256, 0, ctx->stream>>>((const float*)Xd, n, d, (const float*)Qd, nq, k,
-                                                             exclude_self, idx_d, sim_d);
-        HD_CHECK_LAUNCH(ctx);
-        return HD_OK;
-    }
-    if (dtype != HD_BF16) return hd_fail(ctx, HD_ERR_INVALID_ARG, "dtype %d", dtype);
-    if (d % 8) return hd_fail(ctx, HD_ERR_INVALID_ARG, "bf16 descriptors need d %% 8 == 0 (d=%d)", d);
-    using namespace knntc;
-    CUtensorMap tq, tx;
-    if (hd_make_tmap_2d(&tq, Qd, 2, nq, d, d, BM, BK, 1) || hd_make_tmap_2d(&tx, Xd, 2, n, d, d, BN, BK, 1))
-        return hd_fail(ctx, HD_ERR_CUDA, "cuTensorMapEncodeTiled failed");
-    static uint64_t attr = 0;
-    if (hd_first_on_device(attr, ctx->device)) {
-        HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    }
-    const KnnPlan p = knn_plan_tc(ctx, n, nq, k);
+    if (dtype != HD_F32 && dtype != HD_BF16) return hd_fail(ctx, HD_ERR_INVALID_ARG, "dtype %d", dtype);
+    if (dtype == HD_BF16 && d % 8)
+        return hd_fail(ctx, HD_ERR_INVALID_ARG, "bf16 descriptors need d %% 8 == 0 (d=%d)", d);
+    const KnnPlan p = knn_plan_for(ctx, n, nq, k, dtype);
     KnnArgs a;
     a.n = n;
     a.nq = nq;
@@ -574,19 +656,47 @@ static int hd_knn_impl(hd_ctx* ctx, const void* Xd, int64_t n, int32_t d, int dt
     a.nseg = p.nseg;
     a.tps = p.tps;
     WsCarver cv(scratch);
-    a.lists = cv.take<uint64_t>((size_t)p.grid * BM * 64);
+    a.lists = cv.take<uint64_t>((size_t)p.grid * knn_bm(nq, dtype) * 64);
     a.part = p.nseg > 1 ? cv.take<uint64_t>((size_t)p.nseg * nq * k) : nullptr;
     a.idx_out = idx_d;
     a.sim_out = sim_d;
-    HD_CUDA(ctx, cudaMemsetAsync(ctx->d_flags + 1, 0, sizeof(int), ctx->stream));
     HD_PROF(ctx, "knn");
-    k_knn_tc<<<p.grid, THREADS, SMEM_BYTES, ctx->stream>>>(tq, tx, a, ctx->d_flags + 1);
-    HD_CHECK_LAUNCH(ctx);
+    if (dtype == HD_F32) {
+        // float4 loads need 16-byte rows
+        const int vec = d % 4 == 0 && ((uintptr_t)Xd & 15) == 0 && ((uintptr_t)Qd & 15) == 0;
+        static uint64_t attr_f = 0;
+        if (hd_first_on_device(attr_f, ctx->device)) {
+            HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knnf::Cfg<1>::SMEM));
+            HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knnf::Cfg<2>::SMEM));
+            HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_f32<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knnf::Cfg<4>::SMEM));
+            HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knnf::Cfg<8>::SMEM));
+        }
+        const float *X = (const float*)Xd, *Q = (const float*)Qd;
+        switch (knn_f32_tm(nq)) {
+            case 1: k_knn_f32<1><<<p.grid, 256, knnf::Cfg<1>::SMEM, ctx->stream>>>(X, Q, a, vec); break;
+            case 2: k_knn_f32<2><<<p.grid, 256, knnf::Cfg<2>::SMEM, ctx->stream>>>(X, Q, a, vec); break;
+            case 4: k_knn_f32<4><<<p.grid, 256, knnf::Cfg<4>::SMEM, ctx->stream>>>(X, Q, a, vec); break;
+            default: k_knn_f32<8><<<p.grid, 256, knnf::Cfg<8>::SMEM, ctx->stream>>>(X, Q, a, vec); break;
+        }
+        HD_CHECK_LAUNCH(ctx);
+    } else {
+        using namespace knntc;
+        CUtensorMap tq, tx;
+        if (hd_make_tmap_2d(&tq, Qd, 2, nq, d, d, BM, BK, 1) || hd_make_tmap_2d(&tx, Xd, 2, n, d, d, BN, BK, 1))
+            return hd_fail(ctx, HD_ERR_CUDA, "cuTensorMapEncodeTiled failed");
+        static uint64_t attr = 0;
+        if (hd_first_on_device(attr, ctx->device)) {
+            HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+        }
+        HD_CUDA(ctx, cudaMemsetAsync(ctx->d_flags + 1, 0, sizeof(int), ctx->stream));
+        k_knn_tc<<<p.grid, THREADS, SMEM_BYTES, ctx->stream>>>(tq, tx, a, ctx->d_flags + 1);
+        HD_CHECK_LAUNCH(ctx);
+        HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll + 1, ctx->d_flags + 1, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    }
     if (p.nseg > 1) {
         k_knn_merge<<<(unsigned)nq, 256, 0, ctx->stream>>>(a.part, p.nseg, nq, k, idx_d, sim_d);
         HD_CHECK_LAUNCH(ctx);
     }
-    HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll + 1, ctx->d_flags + 1, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     return HD_OK;
 }
 
