@@ -150,7 +150,7 @@ int hd_observe(hd_ctx* ctx, const void* X, int64_t n, int32_t d, int dtype, cons
                float* y_val);
 
 int hd_graph_info(const hd_graph* g, int64_t* n, int64_t* nnz);
-/* The SpMM launch shape the library measured for this graph at padded batch
+/* The SpMM launch shape the library chose for this graph at padded batch
  * width Bp (B rounded up to 4) during an earlier solve: *slab = columns per
  * row group (4..128), *segments = node-range passes.  HD_ERR_INVALID_ARG if no
  * solve with that width has run on the graph yet. */

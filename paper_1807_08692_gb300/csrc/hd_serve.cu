@@ -116,7 +116,7 @@ struct Lane {
     Refill rf;              // device pointers of the staging below (E.refill points here)
     int32_t slots = 0;
     int32_t slot_base = 0;  // reported slot number of column 0
-    int S_full = 4;         // SpMM slab width measured for the whole lane
+    int S_full = 4;         // SpMM slab width for the whole lane
     void* dev = nullptr;
     hd_ctx* ctx = nullptr;
     // staging for the next step: device arrays and their pinned host sources
@@ -250,8 +250,8 @@ static int lane_open(hd_ctx* ctx, const hd_graph* g, const hd_eig* eig, double a
     E.st = cv.take<ColState>(Bp);
     E.num_active = cv.take<int>(16);
     E.err = E.num_active + 1;
-    E.vl = vec_launch(ctx, n, Bp, tune_slab(ctx, g, Bp, E.P, E.Q));
-    L.S_full = E.vl.S;
+    E.vl = vec_launch(ctx, n, Bp);
+    E.slab = L.S_full = spmm_slab(g, Bp);
     L.d_idx = cv.take<int32_t>((size_t)Bp * Kmax);
     L.d_sc = cv.take<float>((size_t)Bp * Kmax);
     L.d_off = cv.take<int32_t>(Bp + 1);
@@ -400,6 +400,14 @@ static int lane_stage(hd_server* s, Lane& L) {
     return HD_OK;
 }
 
+// The SpMM in slabs of S columns; the element-wise kernels take the same width
+// where it is one of theirs (a power of two that divides the lane).
+static void lane_slab(Engine& E, int S) {
+    E.slab = S;
+    const int v = (S & (S - 1)) == 0 && E.Bp % S == 0 ? S : 0;
+    E.vl = vec_launch(E.ctx, E.n, E.Bp, v);
+}
+
 // `iters` CG iterations of lane L; staged requests may be taken at the last
 // one's scalar step; then retirement: the rankings of the requests that
 // stopped, copied to the host.
@@ -430,7 +438,7 @@ static int lane_step(hd_server* s, Lane& L, int32_t iters) {
     E.lr.live = live;
     L.rf.live = live;
     // the narrowest slab that holds every column that can be occupied (at most
-    // the width measured for the full lane): a lightly loaded lane gathers less
+    // the width of the full lane): a lightly loaded lane gathers less
     // per SpMM row.  Results do not depend on it: the reductions are chunked by
     // rows, and every slab width sums a row's entries in the same order.
     int S = L.S_full;
@@ -439,7 +447,7 @@ static int lane_step(hd_server* s, Lane& L, int32_t iters) {
             S = c;
             break;
         }
-    if (S != E.vl.S) E.vl = vec_launch(ctx, E.n, Bp, S);
+    lane_slab(E, S);
     HD_CUDA(ctx, cudaMemsetAsync(L.rf.assign, 0xff, Bp * sizeof(int32_t), ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(L.d_ctl, 0, 2 * sizeof(int), ctx->stream));
     for (int t = 0; t < iters; ++t) {
@@ -534,13 +542,14 @@ static int lane_step(hd_server* s, Lane& L, int32_t iters) {
 static int lane_warm(hd_server* s, Lane& L) {
     hd_ctx* ctx = s->ctx;
     Engine& E = L.E;
+    int rc;
     for (int c : {4, 8, 16, 32, 64, 128}) {
-        if (c > L.S_full || E.Bp % c) continue;
-        E.vl = vec_launch(ctx, E.n, E.Bp, c);
-        int rc = engine_iteration(E, refill_cb, &L);
-        if (rc) return rc;
+        if (c >= L.S_full || E.Bp % c) continue;
+        lane_slab(E, c);
+        if ((rc = engine_iteration(E, refill_cb, &L))) return rc;
     }
-    E.vl = vec_launch(ctx, E.n, E.Bp, L.S_full);
+    lane_slab(E, L.S_full);
+    if ((rc = engine_iteration(E, refill_cb, &L))) return rc;
     std::vector<int32_t> K0(E.Bp, 0);
     return hd_rank_impl(ctx, E.X, E.n, E.Bp, E.Bp, K0.data(), s->Kmax, 0, L.d_idx, L.d_sc);
 }

@@ -30,6 +30,9 @@
 __device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 __device__ __forceinline__ float4 ld4v(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+// the same for a result that the next kernel reads as a stream: first to leave
+// L2, so that it does not push out the rows being gathered
+__device__ __forceinline__ void st4s(float* p, float4 v) { __stcs(reinterpret_cast<float4*>(p), v); }
 
 // ------------------------------------------------------------------ kernels
 // R[:, j] += y_j (one thread per column: duplicates summed in input order).
@@ -55,12 +58,15 @@ __global__ void k_scatter_y(const int32_t* y_ptr, const int32_t* y_idx, const fl
 
 // True when some column of this block's S-column slab is active; with
 // st == nullptr every slab works.
-template <int S>
-__device__ __forceinline__ bool slab_has_work(const ColState* st) {
+__device__ __forceinline__ bool columns_have_work(const ColState* st, int first, int last) {
     if (!st) return true;
     int w = 0;
-    if (threadIdx.x < S) w = st[blockIdx.y * S + threadIdx.x].active;
+    if (first + (int)threadIdx.x < last) w = st[first + threadIdx.x].active;
     return __syncthreads_or(w) != 0;
+}
+template <int S>
+__device__ __forceinline__ bool slab_has_work(const ColState* st) {
+    return columns_have_work(st, blockIdx.y * S, blockIdx.y * S + S);
 }
 
 #define FMA4(acc_, wt_, vec_)                  \
@@ -153,79 +159,159 @@ __device__ __forceinline__ void spmm_rows_pair4(const int32_t* rp, const int32_t
     }
 }
 
-// Q = c1 P - c2 W P for the S-column slab blockIdx.y: S/4 threads per row, each
-// over all of the row's entries (chains as above), 8 gathers in flight.  The
-// P^T Q partials of CG come from k_dot below: kept out of this kernel, its
-// register count allows eight 256-thread blocks per SM, and the extra warps
-// keep more of the random row gathers in flight (measured on the 1M-node graph:
-// 1.58 ms + 0.08 ms for the separate pass against 2.06 ms with the partials
-// fused).  The summation order is the same at every slab width.
-// `skip` (may be null): the launch returns at once when *skip is not 0.
-template <int S>
-__global__ void __launch_bounds__(256, 8) k_spmm(const int32_t* rp, const int32_t* ci, const float* wv, const float* P,
-                                              float* Q, int64_t n, int32_t ld, float c1, float c2,
-                                              const ColState* st, const int* skip = nullptr) {
-    constexpr int L = S / 4;
-    constexpr int RPB = 256 / L;
+// 4-column slabs of Q = c1 P - c2 W P.  `skip` (may be null): the launch
+// returns at once when *skip is not 0.
+__global__ void __launch_bounds__(256, 8) k_spmm4(const int32_t* rp, const int32_t* ci, const float* wv, const float* P,
+                                                  float* Q, int64_t n, int32_t ld, float c1, float c2,
+                                                  const ColState* st, const int* skip) {
     if (skip && *skip) return;
-    if (!slab_has_work<S>(st)) return;
-    if constexpr (S == 4) {
-        spmm_rows_pair4(rp, ci, wv, P, Q, n, ld, c1, c2);
-        return;
+    if (!slab_has_work<4>(st)) return;
+    spmm_rows_pair4(rp, ci, wv, P, Q, n, ld, c1, c2);
+}
+
+// ---- the row gathers shared by the wider SpMM kernels
+// A group of L lanes owns a row; each lane moves 16 bytes of every gathered
+// row.  Bound: the random gathers (DRAM when the gathered block exceeds L2).
+// What keeps them in flight is eight gathers per lane and the next eight
+// (index, weight) pairs already on their way: the first G lanes of a group load
+// one pair each and the group reads them by shuffle, two registers where
+// private copies took sixteen.  At 64 registers (32 warps per SM) a 1M x 64
+// product runs in 1.18 ms (7.2 GB of DRAM traffic, 6.1 TB/s) against 1.58 ms for
+// a kernel of 32 registers and 64 warps, whose eight gathers the compiler had
+// to issue a few at a time; 72 registers and 28 warps take 1.24 ms, 80 and 24
+// 1.42 ms.  Sixteen lanes gather 256 bytes per row and prefer 28 warps.
+constexpr int spmm_blocks(int lanes) { return lanes == 8 ? 8 : 7; }  // blocks of 128 threads per SM
+struct RowLanes {
+    int L, g, gb;      // lanes per row, this lane's place in its group, the group's first lane
+    unsigned mask;     // lanes of the group
+    unsigned row, step;  // first row of the group and the stride to its next
+    bool idle;         // a lane past the last whole group of its warp
+};
+template <int LC>
+__device__ __forceinline__ RowLanes row_lanes(int L_) {
+    RowLanes r;
+    r.L = LC ? LC : L_;
+    const int lane = threadIdx.x & 31, per = 32 / r.L, gi = lane / r.L;
+    r.gb = gi * r.L;
+    r.g = LC ? lane & (LC - 1) : lane - r.gb;
+    r.mask = (r.L == 32 ? 0xffffffffu : (1u << r.L) - 1u) << r.gb;
+    r.idle = gi >= per;
+    const unsigned rpb = (blockDim.x >> 5) * per;
+    r.row = blockIdx.x * rpb + (threadIdx.x >> 5) * per + gi;
+    r.step = gridDim.x * rpb;
+    return r;
+}
+// Entries b .. e of one row: full chunks of 8 through acc(u, w, v), u the place
+// in the chunk, the rest through tail(w, v), each in entry order; load(j)
+// gathers row j.  The lanes of a group run it together.
+template <int LC, class T>
+__device__ __forceinline__ T from_lane(const RowLanes& r, T x, int u) {  // lane u of the group
+    return LC ? __shfl_sync(r.mask, x, u, LC) : __shfl_sync(r.mask, x, r.gb + u);
+}
+template <int LC, int G, class V, class LD, class AC, class TL>
+__device__ __forceinline__ void row_entries(const int32_t* __restrict__ ci, const float* __restrict__ wv, unsigned b,
+                                            unsigned e, const RowLanes& r, LD load, AC acc, TL tail) {
+    constexpr int NI = 8 / G;
+    int32_t jj[NI];
+    float ww[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const unsigned q = b + i * G + r.g;
+        jj[i] = 0;
+        ww[i] = 0.f;
+        if (r.g < G && q < e) {
+            jj[i] = __ldg(ci + q);
+            ww[i] = __ldg(wv + q);
+        }
     }
-    const int g = (threadIdx.x & 31) % L;
-    const int col = blockIdx.y * S + 4 * g;
-    for (int64_t row = (int64_t)blockIdx.x * RPB + threadIdx.x / L; row < n; row += (int64_t)gridDim.x * RPB) {
-        const int32_t b = rp[row], e = rp[row + 1];
+    const unsigned full = b + ((e - b) & ~7u);
+    for (unsigned t = b; t < full; t += 8) {
+        int32_t nj[NI];
+        float nw[NI];
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            const unsigned q = t + 8 + i * G + r.g;
+            nj[i] = 0;
+            nw[i] = 0.f;
+            if (r.g < G && q < e) {
+                nj[i] = __ldg(ci + q);
+                nw[i] = __ldg(wv + q);
+            }
+        }
+        V v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = load(from_lane<LC>(r, jj[u / G], u % G));
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc(u, from_lane<LC>(r, ww[u / G], u % G), v[u]);
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            jj[i] = nj[i];
+            ww[i] = nw[i];
+        }
+    }
+    const unsigned m = e - full;
+    if (m) {
+        V v[7];
+#pragma unroll
+        for (int u = 0; u < 7; ++u) {
+            const int32_t j = from_lane<LC>(r, jj[u / G], u % G);
+            v[u] = V{};  // keeps the loads predicated, all in flight before the first sum
+            if (u < m) v[u] = load(j);
+        }
+#pragma unroll
+        for (int u = 0; u < 7; ++u) {
+            const float w = from_lane<LC>(r, ww[u / G], u % G);
+            if (u < m) tail(w, v[u]);
+        }
+    }
+}
+
+// Q = c1 P - c2 W P, L lanes x 4 columns per slab blockIdx.y (LC > 0: L = LC at
+// compile time, whole slabs only; G = min(L, 8) or the next smaller power of two).  The sums are
+// the two chains of spmm_rows_pair4, the same at every slab width; the lanes of
+// a ragged last slab past the last column repeat it and write nothing.  The
+// P^T Q partials of CG come from k_dot below: fused in here they cost more
+// registers, hence gathers in flight, than the extra pass.
+template <int LC, int G>
+__global__ void __launch_bounds__(128, spmm_blocks(LC)) k_spmm(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                                 const float* __restrict__ wv, const float* __restrict__ P,
+                                                 float* __restrict__ Q, unsigned n, int32_t ld, int L_, float c1,
+                                                 float c2, const ColState* st, const int* skip) {
+    if (skip && *skip) return;
+    const int Lq = LC ? LC : L_;
+    if (!columns_have_work(st, blockIdx.y * 4 * Lq, min(ld, (int)(blockIdx.y + 1) * 4 * Lq))) return;
+    const RowLanes r = row_lanes<LC>(L_);
+    if (r.idle) return;
+    const int quad = blockIdx.y * Lq + r.g, nq = ld >> 2;
+    const bool own_col = LC || quad < nq;
+    const int col = 4 * (own_col ? quad : nq - 1);
+    const float* Pc = P + col;
+    auto load = [&](int32_t j) { return ld4(Pc + (int64_t)j * ld); };
+    for (unsigned row = r.row; row < n; row += r.step) {
+        const unsigned b = __ldg(rp + row), e = __ldg(rp + row + 1);
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
         float4 s2 = make_float4(0.f, 0.f, 0.f, 0.f);
-        int32_t t = b;
-        for (; t + 8 <= e; t += 8) {
-            int32_t j[8];
-            float w[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                j[u] = __ldg(ci + t + u);
-                w[u] = __ldg(wv + t + u);
-            }
-            float4 v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = ld4(P + (int64_t)j[u] * ld + col);
-#pragma unroll
-            for (int u = 0; u < 8; u += 2) {
-                FMA4(s, w[u], v[u]);
-                FMA4(s2, w[u + 1], v[u + 1]);
-            }
-        }
-        // the last e - t < 8 entries, four gathers issued before their
-        // multiply-adds, which still run one entry after another
-        for (; t < e; t += 4) {
-            const int m = e - t;
-            float4 v[4];
-            float w[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                w[u] = u < m ? __ldg(wv + t + u) : 0.f;
-                v[u] = u < m ? ld4(P + (int64_t)__ldg(ci + t + u) * ld + col) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (u < m) {
-                    FMA4(s, w[u], v[u]);
+        row_entries<LC, G, float4>(
+            ci, wv, b, e, r, load,
+            [&](int u, float w, const float4& v) {
+                if (u & 1) {
+                    FMA4(s2, w, v);
+                } else {
+                    FMA4(s, w, v);
                 }
-            }
-        }
+            },
+            [&](float w, const float4& v) { FMA4(s, w, v); });
         s.x += s2.x;
         s.y += s2.y;
         s.z += s2.z;
         s.w += s2.w;
-        const float4 own = ld4(P + row * ld + col);
+        const float4 own = ld4(Pc + (int64_t)row * ld);
         float4 q;
         q.x = c1 * own.x - c2 * s.x;
         q.y = c1 * own.y - c2 * s.y;
         q.z = c1 * own.z - c2 * s.z;
         q.w = c1 * own.w - c2 * s.w;
-        st4(Q + row * ld + col, q);
+        if (own_col) st4s(Q + (int64_t)row * ld + col, q);
     }
 }
 
@@ -233,14 +319,15 @@ __global__ void __launch_bounds__(256, 8) k_spmm(const int32_t* rp, const int32_
 // lanes per row, lane e summing entries b + e, b + e + 4, ... in order (four
 // loads in flight), the four sums meeting as (v0 + v2) + (v1 + v3).  The
 // row's index / weight reads are coalesced and eight rows gather per warp:
-// 0.24 ms on the 1M-node benchmark graph against 0.28 ms for k_spmm<4> (two
+// 0.24 ms on the 1M-node benchmark graph against 0.28 ms for k_spmm4 (two
 // lanes per row), 0.38 ms for a thread per row and 0.32 ms for a warp per row.
 // Its sums run in another order than k_spmm's, so the server, whose results
 // must not depend on the lane width, keeps k_spmm.
 constexpr int N4_ROWS = 64;  // rows per 256-thread block
 __global__ void __launch_bounds__(256, 8) k_spmm_n4(const int32_t* rp, const int32_t* ci, const float* wv,
                                                     const float* P, float* Q, int64_t n, float c1, float c2,
-                                                    const ColState* st) {
+                                                    const ColState* st, const int* skip) {
+    if (skip && *skip) return;
     if (!slab_has_work<4>(st)) return;
     const int lane = threadIdx.x & 31, e = lane & 3;
     // rows advance warp-uniformly (the shuffles need every lane); a lane past
@@ -376,64 +463,49 @@ __global__ void __launch_bounds__(256) k_to_half(const float* __restrict__ P, in
         }                                                                         \
     }
 
-// Q = c1 P - c2 W P with the W P gathers from the fp16 copy (S columns per
-// slab, 8 per lane: a row's slab is S 2 bytes); the sums are fp32, unscaled by
-// the column's power of two at the end.  Runs when *use_half is set.
-template <int S>
-__global__ void __launch_bounds__(256, 4) k_spmm_h(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+// Q = c1 P - c2 W P with the W P gathers from the fp16 copy (L lanes x 8
+// columns per slab: a row's slab of 64 columns is one 128-byte line); the sums
+// are fp32, unscaled by the column's power of two at the end.  Runs when
+// *use_half is set.  0.75 ms for a 1M x 64 product (0.82 ms with private index
+// copies); 0.06 ms against 0.16 ms for 100,000 x 40, which took 8-column slabs.
+template <int LC, int G>
+__global__ void __launch_bounds__(128, 7) k_spmm_h(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                    const float* __restrict__ wv, const __half* __restrict__ P16,
                                                    const unsigned* __restrict__ mx, const float* __restrict__ P,
-                                                   float* __restrict__ Q, int64_t n, int32_t ld, float c1, float c2,
-                                                   const ColState* st, const int* __restrict__ use_half) {
-    constexpr int L = S / 8;
-    constexpr int RPB = 256 / L;
+                                                   float* __restrict__ Q, unsigned n, int32_t ld, int L_, float c1,
+                                                   float c2, const ColState* st, const int* __restrict__ use_half) {
     if (!*use_half) return;
-    if (!slab_has_work<S>(st)) return;
-    const int g = (threadIdx.x & 31) % L;
-    const int col = blockIdx.y * S + 8 * g;
+    const int Lq = LC ? LC : L_;
+    const int first = blockIdx.y * 8 * Lq, last = min(ld, first + 8 * Lq);
+    // up to 256 columns of a slab against 128 threads
+    if (!columns_have_work(st, first, min(last, first + 128)) && !columns_have_work(st, first + 128, last)) return;
+    const RowLanes r = row_lanes<LC>(L_);
+    if (r.idle) return;
+    const int oct = blockIdx.y * Lq + r.g, no = ld >> 3;
+    const bool own_col = LC || oct < no;
+    const int col = 8 * (own_col ? oct : no - 1);
     float inv[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) inv[c] = half_scale(mx[col + c], true);
-    for (int64_t row = (int64_t)blockIdx.x * RPB + threadIdx.x / L; row < n; row += (int64_t)gridDim.x * RPB) {
-        const int32_t b = rp[row], e = rp[row + 1];
+    const __half* Pc = P16 + col;
+    auto load = [&](int32_t j) { return __ldg(reinterpret_cast<const uint4*>(Pc + (int64_t)j * ld)); };
+    for (unsigned row = r.row; row < n; row += r.step) {
+        const unsigned b = __ldg(rp + row), e = __ldg(rp + row + 1);
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        int32_t t = b;
-        for (; t + 8 <= e; t += 8) {
-            int32_t j[8];
-            float w[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                j[u] = __ldg(ci + t + u);
-                w[u] = __ldg(wv + t + u);
-            }
-            uint4 v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = __ldg(reinterpret_cast<const uint4*>(P16 + (int64_t)j[u] * ld + col));
-#pragma unroll
-            for (int u = 0; u < 8; ++u) FMA8H(acc, w[u], v[u]);
-        }
-        for (; t < e; t += 4) {
-            const int m = e - t;
-            uint4 v[4];
-            float w[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                w[u] = u < m ? __ldg(wv + t + u) : 0.f;
-                v[u] = u < m ? __ldg(reinterpret_cast<const uint4*>(P16 + (int64_t)__ldg(ci + t + u) * ld + col))
-                             : make_uint4(0u, 0u, 0u, 0u);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (u < m) FMA8H(acc, w[u], v[u]);
-            }
-        }
-        const float4 o0 = ld4(P + row * ld + col), o1 = ld4(P + row * ld + col + 4);
+        row_entries<LC, G, uint4>(
+            ci, wv, b, e, r, load, [&](int, float w, const uint4& v) { FMA8H(acc, w, v); },
+            [&](float w, const uint4& v) { FMA8H(acc, w, v); });
+        const float* po = P + (int64_t)row * ld + col;
+        const float4 o0 = ld4(po), o1 = ld4(po + 4);
         const float own[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
         float q[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) q[c] = c1 * own[c] - c2 * (acc[c] * inv[c]);
-        st4(Q + row * ld + col, make_float4(q[0], q[1], q[2], q[3]));
-        st4(Q + row * ld + col + 4, make_float4(q[4], q[5], q[6], q[7]));
+        if (own_col) {
+            float* qo = Q + (int64_t)row * ld + col;
+            st4s(qo, make_float4(q[0], q[1], q[2], q[3]));
+            st4s(qo + 4, make_float4(q[4], q[5], q[6], q[7]));
+        }
     }
 }
 
@@ -473,56 +545,38 @@ __device__ __forceinline__ float neg_operator(float c1, float x, float c2, float
     return -__fadd_rn(d, tail);
 }
 
-// Q = -(c1 X - c2 W X) for the S-column slab blockIdx.y, W X in two words.
+// Q = -(c1 X - c2 W X), W X in two words, lanes and slabs as in k_spmm.
 // Runs when *pick is 1 (see k_resid_pick).
-template <int S>
-__global__ void __launch_bounds__(256, 4) k_resid(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+template <int LC, int G>
+__global__ void __launch_bounds__(128, 6) k_resid(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                   const float* __restrict__ wv, const float* __restrict__ X,
-                                                  float* __restrict__ Q, int64_t n, int32_t ld, float c1, float c2,
-                                                  const int* __restrict__ pick) {
-    constexpr int L = S / 4;
-    constexpr int RPB = 256 / L;
+                                                  float* __restrict__ Q, unsigned n, int32_t ld, int L_, float c1,
+                                                  float c2, const int* __restrict__ pick) {
     if (*pick != 1) return;
-    const int g = (threadIdx.x & 31) % L;
-    const int col = blockIdx.y * S + 4 * g;
-    for (int64_t row = (int64_t)blockIdx.x * RPB + threadIdx.x / L; row < n; row += (int64_t)gridDim.x * RPB) {
-        const int32_t b = rp[row], e = rp[row + 1];
+    const RowLanes r = row_lanes<LC>(L_);
+    if (r.idle) return;
+    const int quad = blockIdx.y * r.L + r.g, nq = ld >> 2;
+    const bool own_col = LC || quad < nq;
+    const int col = 4 * (own_col ? quad : nq - 1);
+    const float* Xc = X + col;
+    auto load = [&](int32_t j) { return ld4(Xc + (int64_t)j * ld); };
+    for (unsigned row = r.row; row < n; row += r.step) {
+        const unsigned b = __ldg(rp + row), e = __ldg(rp + row + 1);
         float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-        int32_t t = b;
-        for (; t + 4 <= e; t += 4) {
-            int32_t j[4];
-            float w[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                j[u] = __ldg(ci + t + u);
-                w[u] = __ldg(wv + t + u);
-            }
-            float4 v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = ld4(X + (int64_t)j[u] * ld + col);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                df_fma(hi[0], lo[0], w[u], v[u].x);
-                df_fma(hi[1], lo[1], w[u], v[u].y);
-                df_fma(hi[2], lo[2], w[u], v[u].z);
-                df_fma(hi[3], lo[3], w[u], v[u].w);
-            }
-        }
-        for (; t < e; ++t) {
-            const float w0 = __ldg(wv + t);
-            const float4 v0 = ld4(X + (int64_t)__ldg(ci + t) * ld + col);
-            df_fma(hi[0], lo[0], w0, v0.x);
-            df_fma(hi[1], lo[1], w0, v0.y);
-            df_fma(hi[2], lo[2], w0, v0.z);
-            df_fma(hi[3], lo[3], w0, v0.w);
-        }
-        const float4 own = ld4(X + row * ld + col);
+        auto add = [&](float w, const float4& v) {
+            df_fma(hi[0], lo[0], w, v.x);
+            df_fma(hi[1], lo[1], w, v.y);
+            df_fma(hi[2], lo[2], w, v.z);
+            df_fma(hi[3], lo[3], w, v.w);
+        };
+        row_entries<LC, G, float4>(ci, wv, b, e, r, load, [&](int, float w, const float4& v) { add(w, v); }, add);
+        const float4 own = ld4(Xc + (int64_t)row * ld);
         float4 q;
         q.x = neg_operator(c1, own.x, c2, hi[0], lo[0]);
         q.y = neg_operator(c1, own.y, c2, hi[1], lo[1]);
         q.z = neg_operator(c1, own.z, c2, hi[2], lo[2]);
         q.w = neg_operator(c1, own.w, c2, hi[3], lo[3]);
-        st4(Q + row * ld + col, q);
+        if (own_col) st4s(Q + (int64_t)row * ld + col, q);
     }
 }
 
@@ -1527,51 +1581,71 @@ VecLaunch vec_launch(hd_ctx* ctx, int64_t n, int32_t Bp, int S) {
         default: { constexpr int SS = 128; __VA_ARGS__; } break;  \
     }
 
-int tune_slab(hd_ctx* ctx, const hd_graph* g, int32_t Bp, const float* P, float* Q) {
-    auto it = g->slab_cache.find(Bp);
-    if (it != g->slab_cache.end()) return it->second;
-    if (getenv("HD_SLAB")) return g->slab_cache[Bp] = pick_slab(Bp);
-    int best = pick_slab(Bp);
-    float best_ms = 1e30f;
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    for (int S : {8, 16, 32, 64, 128}) {
-        if (Bp % S || (S == 8 && Bp > 8 && g->n < 4096)) continue;
-        VecLaunch v = vec_launch(ctx, g->n, Bp, S);
-        dim3 grid(v.nblk, v.slabs);
-        float tot = 0.f;
-        for (int rep = 0; rep < 3; ++rep) {
-            cudaEventRecord(e0, ctx->stream);
-            HD_DISPATCH_S(S, (k_spmm<SS><<<grid, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, P, Q, g->n, Bp,
-                                                                         1.f, 1.f, nullptr)));
-            cudaEventRecord(e1, ctx->stream);
-            cudaEventSynchronize(e1);
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (rep) tot += ms;
-        }
-        ctx->launches += 3;
-        if (tot < best_ms * 0.97f) {
-            best_ms = tot;
-            best = S;
-        }
+// Lanes per row of the SpMM over `cols` columns in groups of `per` (4 fp32 or 8
+// fp16 columns per lane; `big`: the gathered block exceeds what L2 holds).
+// Whole 128-byte lines, one per row and pass (8 lanes), when the width allows:
+// a 64-column pass over a block larger than L2 reads 1.3 times the DRAM bytes
+// (1M nodes, 64 columns: 1.18 ms against 1.50 ms).  16 lanes when the block fits
+// in L2 (100,000 x 64: 0.082 ms against 0.086 ms), and from 256 columns on, where
+// the 128-byte lines of one pass lie 1 KB apart (1M x 256: 6.1 ms against 6.7).
+// Other widths take the whole row at once up to 16 lanes, else the fewest even
+// parts of at most 16: 100,000 x 40 runs in 0.067 ms with 10 lanes, 0.12 ms in
+// two passes of 9 and 0.174 ms in five of 2.
+static int spmm_lanes(int32_t cols, int per, bool big) {
+    const int nl = cols / per;
+    if (nl % 8 == 0) return per == 4 && nl % 16 == 0 && (!big || nl >= 64) ? 16 : 8;
+    return ceil_div(nl, ceil_div(nl, 16));
+}
+static bool spmm_exceeds_l2(int64_t n, int32_t Bp, int bytes) { return n * Bp * bytes > (int64_t)64 << 20; }
+
+// Column-slab width of the SpMM (4 x lanes per row); recorded per graph and
+// batch width for hd_graph_tuning.  HD_SLAB caps it.
+int spmm_slab(const hd_graph* g, int32_t Bp) {
+    const int S = getenv("HD_SLAB") ? pick_slab(Bp) : 4 * spmm_lanes(Bp, 4, spmm_exceeds_l2(g->n, Bp, 4));
+    g->slab_cache[Bp] = S;
+    return S;
+}
+
+// LC = L where L is a power of two that divides the width, else LC = 0
+#define HD_DISPATCH_L(L, width, ...)                                                  \
+    switch ((width) % (L) ? 0 : (L)) {                                                \
+        case 2: { constexpr int LC = 2, G = 2; __VA_ARGS__; } break;                  \
+        case 4: { constexpr int LC = 4, G = 4; __VA_ARGS__; } break;                  \
+        case 8: { constexpr int LC = 8, G = 8; __VA_ARGS__; } break;                  \
+        case 16: { constexpr int LC = 16, G = 8; __VA_ARGS__; } break;                \
+        case 32: { constexpr int LC = 32, G = 8; __VA_ARGS__; } break;                \
+        default:                                                                      \
+            if (L > 8) { constexpr int LC = 0, G = 8; __VA_ARGS__; }                  \
+            else if (L > 4) { constexpr int LC = 0, G = 4; __VA_ARGS__; }             \
+            else if (L > 1) { constexpr int LC = 0, G = 2; __VA_ARGS__; }             \
+            else { constexpr int LC = 0, G = 1; __VA_ARGS__; }                        \
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    cudaGetLastError();
-    g->slab_cache[Bp] = best;
-    return best;
+// blocks of 128 threads: 32 / L rows per warp, `per_sm` resident blocks per SM
+static dim3 spmm_grid(hd_ctx* ctx, int64_t n, int32_t cols, int per, int L, int per_sm) {
+    const int rpb = 4 * (32 / L);
+    return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, rpb), (int64_t)ctx->num_sms * per_sm)),
+                (unsigned)ceil_div(cols / per, L));
+}
+// Q = c1 P - c2 W P in slabs of S columns
+static int spmm_launch(hd_ctx* ctx, const hd_graph* g, const float* P, float* Q, int32_t ld, int S, float c1, float c2,
+                       const ColState* st, const int* skip) {
+    if (S == 4) {
+        const VecLaunch v = vec_launch(ctx, g->n, ld, 4);
+        k_spmm4<<<dim3(v.nblk, v.slabs), 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, P, Q, g->n, ld, c1, c2, st,
+                                                                skip);
+    } else {
+        const int L = S / 4;
+        const dim3 grid = spmm_grid(ctx, g->n, ld, 4, L, spmm_blocks(L));
+        HD_DISPATCH_L(L, ld / 4, (k_spmm<LC, G><<<grid, 128, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, P, Q, (unsigned)g->n,
+                                                                        ld, L, c1, c2, st, skip)));
+    }
+    HD_CHECK_LAUNCH(ctx);
+    return HD_OK;
 }
 
 int hd_spmm_apply(hd_ctx* ctx, const hd_graph* g, const float* P, float* Q, int32_t ld, int32_t B, float c1,
                   float c2) {
-    VecLaunch v = vec_launch(ctx, g->n, ld);
-    dim3 grid(v.nblk, v.slabs);
-    HD_DISPATCH_S(v.S, (k_spmm<SS><<<grid, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, P, Q, g->n, ld, c1, c2,
-                                                                   nullptr)));
-    HD_CHECK_LAUNCH(ctx);
-    return HD_OK;
+    return spmm_launch(ctx, g, P, Q, ld, 4 * spmm_lanes(ld, 4, spmm_exceeds_l2(g->n, ld, 4)), c1, c2, nullptr, nullptr);
 }
 
 // grid and block of the column reductions: one block row per chunk, up to 128 quads x 8 threads
@@ -1620,17 +1694,14 @@ static int launch_spmm(Engine& E, float c1, float c2, float2* part, const ColSta
     hd_ctx* ctx = E.ctx;
     const hd_graph* g = E.g;
     const float* Pin = V ? V : E.P;
-    dim3 grid(E.vl.nblk, E.vl.slabs);
+    int rc;
     if (!V && E.use_half) {
         // the iteration's SpMM: an fp16 copy of P is gathered when *use_half
-        // (columns 8 per lane; 64-column slabs make a row's slab 128 bytes)
-        const int S16 = E.Bp % 64 == 0 ? 64 : E.Bp % 32 == 0 ? 32 : E.Bp % 16 == 0 ? 16 : 8;
         const int nq = E.Bp / 4;
         const int rpb = 256 / nq;
         const dim3 gc((unsigned)std::min<int64_t>(ceil_div(E.n, rpb), (int64_t)ctx->num_sms * 8));
-        const int rpb16 = 256 / (S16 / 8);
-        const dim3 gh((unsigned)std::min<int64_t>(ceil_div(E.n, rpb16), (int64_t)ctx->num_sms * 4),
-                      (unsigned)(E.Bp / S16));
+        const int L16 = spmm_lanes(E.Bp, 8, spmm_exceeds_l2(E.n, E.Bp, 2));
+        const dim3 gh = spmm_grid(ctx, E.n, E.Bp, 8, L16, 7);
         {
             HD_PROF(ctx, "to_half");
             HD_CUDA(ctx, cudaMemsetAsync(E.p16_max, 0, (size_t)E.Bp * sizeof(unsigned), ctx->stream));
@@ -1641,22 +1712,13 @@ static int launch_spmm(Engine& E, float c1, float c2, float2* part, const ColSta
         }
         {
             HD_PROF(ctx, "spmm");
-            HD_DISPATCH_S(E.vl.S, (k_spmm<SS><<<grid, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.P, E.Q, E.n,
-                                                                              E.Bp, c1, c2, st, E.use_half)));
-            HD_CHECK_LAUNCH(ctx);
+            if ((rc = spmm_launch(ctx, g, E.P, E.Q, E.Bp, E.slab, c1, c2, st, E.use_half))) return rc;
         }
         {
             HD_PROF(ctx, "spmm_h");
-            switch (S16) {
-                case 64: k_spmm_h<64><<<gh, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.P16, E.p16_max, E.P,
-                                                                    E.Q, E.n, E.Bp, c1, c2, st, E.use_half); break;
-                case 32: k_spmm_h<32><<<gh, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.P16, E.p16_max, E.P,
-                                                                    E.Q, E.n, E.Bp, c1, c2, st, E.use_half); break;
-                case 16: k_spmm_h<16><<<gh, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.P16, E.p16_max, E.P,
-                                                                    E.Q, E.n, E.Bp, c1, c2, st, E.use_half); break;
-                default: k_spmm_h<8><<<gh, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.P16, E.p16_max, E.P,
-                                                                   E.Q, E.n, E.Bp, c1, c2, st, E.use_half); break;
-            }
+            HD_DISPATCH_L(L16, E.Bp / 8, (k_spmm_h<LC, G><<<gh, 128, 0, ctx->stream>>>(
+                                   g->row_ptr, g->col, g->val, E.P16, E.p16_max, E.P, E.Q, (unsigned)E.n, E.Bp, L16, c1,
+                                   c2, st, E.use_half)));
             HD_CHECK_LAUNCH(ctx);
         }
         if (part) return launch_dot(E, part, st);
@@ -1666,13 +1728,12 @@ static int launch_spmm(Engine& E, float c1, float c2, float2* part, const ColSta
         HD_PROF(ctx, "spmm");
         if (E.segK <= 1 && E.Bp == 4 && E.narrow4) {
             const dim3 g4((unsigned)std::max(1, ceil_div(E.n, N4_ROWS)));
-            k_spmm_n4<<<g4, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, Pin, E.Q, E.n, c1, c2, st);
+            k_spmm_n4<<<g4, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, Pin, E.Q, E.n, c1, c2, st, nullptr);
             HD_CHECK_LAUNCH(ctx);
         } else if (E.segK <= 1) {
-            HD_DISPATCH_S(E.vl.S, (k_spmm<SS><<<grid, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, Pin, E.Q,
-                                                                              E.n, E.Bp, c1, c2, st)));
-            HD_CHECK_LAUNCH(ctx);
+            if ((rc = spmm_launch(ctx, g, Pin, E.Q, E.Bp, E.slab, c1, c2, st, nullptr))) return rc;
         } else {
+            const dim3 grid(E.vl.nblk, E.vl.slabs);
             for (int s = 0; s < E.segK; ++s) {
                 const int32_t* lo = E.seg + (int64_t)s * E.n;
                 HD_DISPATCH_S(E.vl.S, (k_spmm_seg<SS><<<grid, 256, 0, ctx->stream>>>(
@@ -1704,7 +1765,7 @@ static const int32_t* seg_bounds_for(hd_ctx* ctx, const hd_graph* g, int K) {
     return b;
 }
 
-int tune_segments(hd_ctx* ctx, Engine& E) {
+int spmm_segments(hd_ctx* ctx, Engine& E) {
     const hd_graph* g = E.g;
     E.segK = 1;
     E.seg = nullptr;
@@ -1713,51 +1774,13 @@ int tune_segments(hd_ctx* ctx, Engine& E) {
         const char* s = getenv("HD_SEGMENTS");
         forced = s ? atoi(s) : -1;
     }
-    int K = 1;
-    auto it = g->seg_cache.find(E.Bp);
-    if (forced >= 1) {
-        K = forced;
-        g->seg_cache[E.Bp] = K;  // reported by hd_graph_tuning
-    } else if (it != g->seg_cache.end()) {
-        K = it->second;
-    } else if ((int64_t)g->n * E.Bp * 4 > (int64_t)64 << 20) {
-        // gathered block larger than about half of L2: time the candidates
-        float best_ms = 1e30f;
-        cudaEvent_t e0, e1;
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        for (int k : {1, 2, 4, 8}) {
-            if (k > 1 && !seg_bounds_for(ctx, g, k)) continue;
-            E.segK = k;
-            E.seg = k > 1 ? g->seg_bounds[k] : nullptr;
-            float tot = 0.f;
-            for (int rep = 0; rep < 3; ++rep) {
-                cudaEventRecord(e0, ctx->stream);
-                launch_spmm(E, 1.f, 1.f, nullptr, nullptr);
-                cudaEventRecord(e1, ctx->stream);
-                cudaEventSynchronize(e1);
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                if (rep) tot += ms;
-            }
-            if (tot < best_ms * 0.97f) {
-                best_ms = tot;
-                K = k;
-            }
-        }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        cudaGetLastError();
-        g->seg_cache[E.Bp] = K;
-    }
-    if (K > 1) {
-        const int32_t* b = seg_bounds_for(ctx, g, K);
+    if (forced < 1) return HD_OK;
+    g->seg_cache[E.Bp] = forced;  // reported by hd_graph_tuning
+    if (forced > 1) {
+        const int32_t* b = seg_bounds_for(ctx, g, forced);
         if (!b) return hd_fail(ctx, HD_ERR_OOM, "SpMM segment bounds");
-        E.segK = K;
+        E.segK = forced;
         E.seg = b;
-    } else {
-        E.segK = 1;
-        E.seg = nullptr;
     }
     return HD_OK;
 }
@@ -1884,7 +1907,7 @@ static std::vector<uint64_t> iteration_key(const Engine& E) {
             (uint64_t)E.R, (uint64_t)E.P, (uint64_t)E.Q, (uint64_t)E.X, (uint64_t)E.part, (uint64_t)E.st,
             (uint64_t)E.num_active, (uint64_t)E.lr.part, (uint64_t)E.lr.C, (uint64_t)E.lr.H, (uint64_t)E.lr.Hhi,
             (uint64_t)E.lr.Hlo, (uint64_t)E.dcoef, (uint64_t)E.opcoef, (uint64_t)E.segK, (uint64_t)E.seg,
-            (uint64_t)E.nch, (uint64_t)E.Bp, (uint64_t)E.vl.S, (uint64_t)E.vl.nblk, (uint64_t)E.vl.slabs,
+            (uint64_t)E.nch, (uint64_t)E.Bp, (uint64_t)E.slab, (uint64_t)E.vl.S, (uint64_t)E.vl.nblk, (uint64_t)E.vl.slabs,
             (uint64_t)E.lr.nchunk, (uint64_t)E.lr.rpad, (uint64_t)E.lr.Bp16, (uint64_t)E.has_lr,
             (uint64_t)E.eff_mode, (uint64_t)E.r, (uint64_t)E.max_iter, fbits(E.c1), fbits(E.c2), fbits(E.xs),
             (uint64_t)E.P16, (uint64_t)E.p16_max, (uint64_t)E.use_half, (uint64_t)E.ctx->stream};
@@ -2010,8 +2033,8 @@ static int true_residual(Engine& E, double alpha) {
     const double c1d = 1.0 / (1.0 - alpha), c2d = alpha / (1.0 - alpha);
     const float c1 = (float)c1d, c2 = (float)c2d;
     int rc;
-    dim3 grid(E.vl.nblk, E.vl.slabs);
     if (E.ts) {
+        const dim3 grid(E.vl.nblk, E.vl.slabs);
         // Q = -L_a(W_j) x column by column (truncated systems), in two words
         HD_PROF(ctx, "resid");
         HD_DISPATCH_S(E.vl.S, (k_resid_cols<SS><<<grid, 256, 0, ctx->stream>>>(E.ts->off, E.ts->ci, E.ts->wv, E.ts->B,
@@ -2033,11 +2056,17 @@ static int true_residual(Engine& E, double alpha) {
         }
         HD_CHECK_LAUNCH(ctx);
         HD_PROF(ctx, "resid");
-        HD_DISPATCH_S(E.vl.S, (k_spmm<SS><<<grid, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.X, E.Q, n, Bp,
-                                                                          -c1, -c2, nullptr, pick)));
-        HD_CHECK_LAUNCH(ctx);
-        HD_DISPATCH_S(E.vl.S, (k_resid<SS><<<grid, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.X, E.Q, n, Bp,
-                                                                           c1, c2, pick)));
+        if (Bp == 4 && E.narrow4) {
+            k_spmm_n4<<<std::max(1, ceil_div(n, N4_ROWS)), 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.X, E.Q,
+                                                                                  n, -c1, -c2, nullptr, pick);
+            HD_CHECK_LAUNCH(ctx);
+        } else if ((rc = spmm_launch(ctx, g, E.X, E.Q, Bp, E.slab, -c1, -c2, nullptr, pick))) {
+            return rc;
+        }
+        const int L = std::max(1, E.slab / 4);
+        const dim3 gr = spmm_grid(ctx, n, Bp, 4, L, 6);
+        HD_DISPATCH_L(L, Bp / 4, (k_resid<LC, G><<<gr, 128, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.X, E.Q, (unsigned)n,
+                                                                       Bp, L, c1, c2, pick)));
         HD_CHECK_LAUNCH(ctx);
     }
     if (E.has_lr && E.eff_mode != HD_MODE_PCG) {
@@ -2236,8 +2265,10 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         g->max_row = ctx->h_poll[0];
     }
-    S_.vl = vec_launch(ctx, n, Bp, ts ? pick_slab(Bp) : tune_slab(ctx, g, Bp, S_.P, S_.Q));
-    if (!ts && (rc = tune_segments(ctx, S_))) return rc;
+    if (!ts) {
+        S_.slab = spmm_slab(g, Bp);
+        if ((rc = spmm_segments(ctx, S_))) return rc;
+    }
     if (half_ok && S_.segK == 1 && !half_gathers_off()) {
         S_.P16 = p16;
         S_.p16_max = p16_max;

@@ -123,6 +123,7 @@ struct Engine {
     VecLaunch vl{};
     int rch = 64;                      // rows per reduction chunk (depends on n only)
     int64_t nch = 0;                   // reduction chunks: column partials are [nch][Bp]
+    int slab = 4;                      // SpMM column-slab width (any multiple of 4 up to 128)
     int segK = 1;                      // SpMM node-range segments (1: one pass)
     const int32_t* seg = nullptr;      // their row bounds [segK + 1][n]
     // a 4-column batch may use k_spmm_n4 (its sums run in another order than
@@ -157,13 +158,12 @@ struct Engine {
 };
 
 VecLaunch vec_launch(hd_ctx* ctx, int64_t n, int32_t Bp, int S = 0);
-// Column-slab width of the SpMM for this graph and batch width: measured once
-// per (graph, Bp) over the widths dividing Bp (HD_SLAB overrides).
-int tune_slab(hd_ctx* ctx, const hd_graph* g, int32_t Bp, const float* P, float* Q);
+// Column-slab width of the SpMM for this graph and batch width (HD_SLAB caps it).
+int spmm_slab(const hd_graph* g, int32_t Bp);
 int simt_nchunk(hd_ctx* ctx, int64_t n, int rpad, int Bp);
-// Node-range segments for the SpMM with slab width S: measured once per
-// (graph, Bp) over K in {1, 2, 4, 8} (HD_SEGMENTS overrides); sets E.segK / E.seg.
-int tune_segments(hd_ctx* ctx, Engine& E);
+// Node-range segments for the SpMM: one pass unless HD_SEGMENTS asks for more;
+// sets E.segK / E.seg.
+int spmm_segments(hd_ctx* ctx, Engine& E);
 int engine_iteration(Engine& E, int (*after_update)(void*), void* arg);
 // r += y for the columns of a server lane that took a request at the last
 // scalar step (after their first update), with the exact ||r||^2 correction
