@@ -181,6 +181,15 @@ __device__ __forceinline__ void ksum_add(KSum& a, float x) {
     a.s = t;
     a.c += e;
 }
+// a += x y with the product unrounded in both sums (the error term is then that
+// of the product too); intrinsics, so that every kernel forms the same bits
+__device__ __forceinline__ void ksum_add_product(KSum& a, float x, float y) {
+    const float t = __fmaf_rn(x, y, a.s);
+    const float bp = __fsub_rn(t, a.s);
+    const float e = __fadd_rn(__fsub_rn(a.s, __fsub_rn(t, bp)), __fmaf_rn(x, y, -bp));
+    a.s = t;
+    a.c = __fadd_rn(a.c, e);
+}
 __device__ __forceinline__ void ksum_merge(KSum& a, KSum b) {
     float t = a.s + b.s;
     float bp = t - a.s;

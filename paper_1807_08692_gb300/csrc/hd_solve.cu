@@ -35,24 +35,43 @@ __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<floa
 __device__ __forceinline__ void st4s(float* p, float4 v) { __stcs(reinterpret_cast<float4*>(p), v); }
 
 // ------------------------------------------------------------------ kernels
-// R[:, j] += y_j (one thread per column: duplicates summed in input order).
-__global__ void k_scatter_y(const int32_t* y_ptr, const int32_t* y_idx, const float* y_val, int32_t B, int64_t n,
-                            int32_t ld, float* R, int* err) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= B) return;
-    int32_t b = y_ptr[j], e = y_ptr[j + 1];
+// R[:, j] += y_j, one block per column.  Entries with one index are added in
+// input order by the thread of the first of them; ascending indices (as
+// hd_observe returns them) need no search for such entries, and a longer list
+// in another order is left to one thread.
+constexpr int SCATTER_SEARCH = 1024;
+__global__ void __launch_bounds__(128) k_scatter_y(const int32_t* y_ptr, const int32_t* y_idx, const float* y_val,
+                                                   int64_t n, int32_t ld, float* R, int* err) {
+    const int j = blockIdx.x;
+    const int32_t b = y_ptr[j], e = y_ptr[j + 1];
     if (b > e || b < 0) {
-        atomicExch(err, 1);
+        if (threadIdx.x == 0) atomicExch(err, 1);
         return;
     }
-    for (int32_t t = b; t < e; ++t) {
+    int unsorted = 0;
+    for (int32_t t = b + (int)threadIdx.x; t + 1 < e; t += blockDim.x) unsorted |= y_idx[t] >= y_idx[t + 1];
+    unsorted = __syncthreads_or(unsorted);
+    const bool serial = unsorted && e - b > SCATTER_SEARCH;
+    if (serial && threadIdx.x) return;
+    for (int32_t t = b + (int)threadIdx.x; t < e; t += serial ? 1 : (int)blockDim.x) {
         const int32_t i = y_idx[t];
         const float v = y_val[t];
         if (i < 0 || i >= n || !isfinite(v)) {
             atomicExch(err, 1);
             continue;
         }
-        R[(int64_t)i * ld + j] += v;
+        float* a = R + (int64_t)i * ld + j;
+        if (serial || !unsorted) {
+            *a += v;
+            continue;
+        }
+        bool first = true;
+        for (int32_t s = b; s < t; ++s) first &= y_idx[s] != i || !isfinite(y_val[s]);
+        if (!first) continue;
+        float sum = *a + v;
+        for (int32_t s = t + 1; s < e; ++s)
+            if (y_idx[s] == i && isfinite(y_val[s])) sum += y_val[s];
+        *a = sum;
     }
 }
 
@@ -759,139 +778,263 @@ __global__ void __launch_bounds__(256, 8) k_spmm_seg(const int32_t* __restrict__
 // [nch][ld] are added in chunk order by the fp64 column kernels.  A column's CG
 // scalars are therefore the same bit for bit whatever the slab width, the
 // batch width or the other columns of the batch.
+// A grid that fills the GPU runs these sums as they stand, one thread per (g,
+// quad), rows streamed from memory (1M x 64: 0.23 ms for k_update, the copy
+// bandwidth).  A small one would wait for memory 64 times in a row; there a
+// block of 256 threads loads (and updates) a whole chunk of 16 columns at once
+// into shared memory and one thread per (g, column) then sums its rows from
+// there, in the same order (k_red_staged: with cold caches 7 us against 42 for
+// the update of 2,000 x 16, 7 against 20 for the dot product).
 constexpr int RG = 8;      // threads per chunk and quad
-constexpr int RQ = 128;    // quads per block (at most)
+constexpr int RQ = 32;     // quads per block (at most)
 
 int reduction_chunk_rows(int64_t n) {
     const int64_t r = (n + 4095) / 4096;
     return (int)std::max<int64_t>(512, (r + RG - 1) / RG * RG);
 }
 
-// thread -> (chunk = blockIdx.x, quad, g); false when the quad has no column to work on
-__device__ __forceinline__ bool red_thread(int64_t n, int32_t ld, int rch, const ColState* st, int64_t& r0,
-                                           int64_t& r1, int& col, int& g) {
+// the rows and columns of a thread: `work` is false when it has none
+struct RedThread {
+    int64_t r0, r1, chunk;
+    int col, g, ql, qpb;
+    bool work;
+};
+__device__ __forceinline__ RedThread red_thread(int64_t n, int32_t ld, int rch, const ColState* st) {
+    RedThread t;
     const int nq = ld >> 2;
-    const int qpb = nq < RQ ? nq : RQ;
-    const int quad = blockIdx.y * RQ + (int)threadIdx.x % qpb;
-    g = (int)threadIdx.x / qpb;
-    col = 4 * quad;
-    r0 = (int64_t)blockIdx.x * rch + g;
-    r1 = min(n, (int64_t)(blockIdx.x + 1) * rch);
-    if (quad >= nq) return false;
-    if (!st) return true;
-    bool w = false;
+    t.qpb = nq < RQ ? nq : RQ;
+    t.ql = (int)threadIdx.x % t.qpb;
+    t.g = (int)threadIdx.x / t.qpb;
+    const int quad = blockIdx.y * RQ + t.ql;
+    t.col = 4 * quad;
+    t.chunk = blockIdx.x;
+    t.r0 = t.chunk * rch + t.g;
+    t.r1 = min(n, (t.chunk + 1) * rch);
+    t.work = quad < nq;
+    if (t.work && st) {
+        t.work = false;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) w |= st[col + c].active;
-    return w;
+        for (int c = 0; c < 4; ++c) t.work |= st[t.col + c].active != 0;
+    }
+    return t;
 }
 
 // combine the RG partial sums of each quad in g order and store the chunk partial
-__device__ __forceinline__ void red_finish(float2* part, int32_t ld, bool work, int col, int g, const KSum (&a)[4]) {
-    extern __shared__ float2 red_sm[];  // [RG][qpb * 4]
-    const int nq = ld >> 2;
-    const int qpb = nq < RQ ? nq : RQ;
-    const int ql = (int)threadIdx.x % qpb;
+__device__ __forceinline__ void red_finish(float2* part, int32_t ld, const RedThread& t, const KSum (&a)[4]) {
+    extern __shared__ float2 sm[];  // [RG][qpb * 4]
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-        red_sm[g * qpb * 4 + ql * 4 + c] = work ? make_float2(a[c].s, a[c].c) : make_float2(0.f, 0.f);
+        sm[(t.g * t.qpb + t.ql) * 4 + c] = t.work ? make_float2(a[c].s, a[c].c) : make_float2(0.f, 0.f);
     __syncthreads();
-    if (g != 0 || !work) return;
-    KSum t[4];
+    if (t.g != 0 || !t.work) return;
+    KSum s[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        t[c] = KSum{red_sm[ql * 4 + c].x, red_sm[ql * 4 + c].y};
-        for (int h = 1; h < RG; ++h)
-            ksum_merge(t[c], KSum{red_sm[h * qpb * 4 + ql * 4 + c].x, red_sm[h * qpb * 4 + ql * 4 + c].y});
+        s[c] = KSum{sm[t.ql * 4 + c].x, sm[t.ql * 4 + c].y};
+#pragma unroll
+        for (int h = 1; h < RG; ++h) {
+            const float2 v = sm[(h * t.qpb + t.ql) * 4 + c];
+            ksum_merge(s[c], KSum{v.x, v.y});
+        }
     }
-    float4* d = reinterpret_cast<float4*>(part + (int64_t)blockIdx.x * ld + col);
-    d[0] = make_float4(t[0].s, t[0].c, t[1].s, t[1].c);
-    d[1] = make_float4(t[2].s, t[2].c, t[3].s, t[3].c);
+    float4* d = reinterpret_cast<float4*>(part + t.chunk * ld + t.col);
+    d[0] = make_float4(s[0].s, s[0].c, s[1].s, s[1].c);
+    d[1] = make_float4(s[2].s, s[2].c, s[3].s, s[3].c);
 }
 
 // Partials of sum_i V_ij^2 (every column).
-__global__ void __launch_bounds__(1024) k_colsq(const float* __restrict__ V, int64_t n, int32_t ld, int rch,
-                                                float2* __restrict__ part) {
-    int64_t r0, r1;
-    int col, g;
-    const bool work = red_thread(n, ld, rch, nullptr, r0, r1, col, g);
+__global__ void __launch_bounds__(256) k_colsq(const float* __restrict__ V, int64_t n, int32_t ld, int rch,
+                                               float2* __restrict__ part) {
+    constexpr int U = 8;
+    const RedThread t = red_thread(n, ld, rch, nullptr);
     KSum acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-    // four rows' loads issued before their (row-ordered) compensated adds: one
-    // load in flight per thread left this single-array pass at half the HBM rate
-    if (work)
-        for (int64_t row = r0; row < r1; row += 4 * RG) {
-            float4 v[4];
+    if (t.work)
+        for (int64_t row = t.r0; row < t.r1; row += U * RG) {
+            float4 v[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                v[u] = row + u * RG < r1 ? ld4v(V + (row + u * RG) * ld + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int u = 0; u < U; ++u)
+                v[u] = row + u * RG < t.r1 ? ld4v(V + (row + u * RG) * ld + t.col) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (row + u * RG >= r1) break;
-                ksum_add(acc[0], v[u].x * v[u].x);
-                ksum_add(acc[1], v[u].y * v[u].y);
-                ksum_add(acc[2], v[u].z * v[u].z);
-                ksum_add(acc[3], v[u].w * v[u].w);
+            for (int u = 0; u < U; ++u) {
+                if (row + u * RG >= t.r1) break;
+                ksum_add_product(acc[0], v[u].x, v[u].x);
+                ksum_add_product(acc[1], v[u].y, v[u].y);
+                ksum_add_product(acc[2], v[u].z, v[u].z);
+                ksum_add_product(acc[3], v[u].w, v[u].w);
             }
         }
-    red_finish(part, ld, work, col, g, acc);
+    red_finish(part, ld, t, acc);
 }
 
 // Partials of P^T Q (columns being iterated).
-__global__ void __launch_bounds__(1024) k_dot(const float* __restrict__ P, const float* __restrict__ Q, int64_t n,
-                                              int32_t ld, int rch, float2* __restrict__ part,
-                                              const ColState* __restrict__ st) {
-    int64_t r0, r1;
-    int col, g;
-    const bool work = red_thread(n, ld, rch, st, r0, r1, col, g);
+__global__ void __launch_bounds__(256) k_dot(const float* __restrict__ P, const float* __restrict__ Q, int64_t n,
+                                             int32_t ld, int rch, float2* __restrict__ part,
+                                             const ColState* __restrict__ st) {
+    const RedThread t = red_thread(n, ld, rch, st);
     KSum acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-    if (work)
-        for (int64_t row = r0; row < r1; row += RG) {
-            const float4 a = ld4(P + row * ld + col), b = ld4(Q + row * ld + col);
-            ksum_add(acc[0], a.x * b.x);
-            ksum_add(acc[1], a.y * b.y);
-            ksum_add(acc[2], a.z * b.z);
-            ksum_add(acc[3], a.w * b.w);
+    if (t.work)
+        for (int64_t row = t.r0; row < t.r1; row += RG) {
+            const float4 a = ld4(P + row * ld + t.col), b = ld4(Q + row * ld + t.col);
+            ksum_add_product(acc[0], a.x, b.x);
+            ksum_add_product(acc[1], a.y, b.y);
+            ksum_add_product(acc[2], a.z, b.z);
+            ksum_add_product(acc[3], a.w, b.w);
         }
-    red_finish(part, ld, work, col, g, acc);
+    red_finish(part, ld, t, acc);
+}
+
+// The step lengths of a column quad and the columns that start afresh
+struct UpdateQuad {
+    float a[4], x[4];
+    bool f[4], any;
+};
+__device__ __forceinline__ UpdateQuad update_quad(const ColState* st, int col, float xs) {
+    UpdateQuad u;
+    u.any = false;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        u.a[c] = (float)st[col + c].a;
+        u.x[c] = xs * u.a[c];
+        // a served column that took a new request at the last scalar step starts
+        // from x0 = 0, r0 = y: x = a p, r = -a q here, y is added next
+        u.f[c] = st[col + c].refill;
+        u.any |= u.f[c];
+    }
+    return u;
+}
+__device__ __forceinline__ void update_row(const UpdateQuad& u, const float4& p, const float4& q, float4& x, float4& r) {
+    if (u.any) {
+        if (u.f[0]) x.x = r.x = 0.0f;
+        if (u.f[1]) x.y = r.y = 0.0f;
+        if (u.f[2]) x.z = r.z = 0.0f;
+        if (u.f[3]) x.w = r.w = 0.0f;
+    }
+    x.x = fmaf(u.x[0], p.x, x.x);
+    x.y = fmaf(u.x[1], p.y, x.y);
+    x.z = fmaf(u.x[2], p.z, x.z);
+    x.w = fmaf(u.x[3], p.w, x.w);
+    r.x = fmaf(-u.a[0], q.x, r.x);
+    r.y = fmaf(-u.a[1], q.y, r.y);
+    r.z = fmaf(-u.a[2], q.z, r.z);
+    r.w = fmaf(-u.a[3], q.w, r.w);
 }
 
 // X += xs a P; R -= a Q; partials of ||R||^2.
-__global__ void __launch_bounds__(1024) k_update(float* __restrict__ X, float* __restrict__ R,
-                                                 const float* __restrict__ P, const float* __restrict__ Q, int64_t n,
-                                                 int32_t ld, int rch, const ColState* __restrict__ st, float xs,
-                                                 float2* __restrict__ part) {
-    int64_t r0, r1;
-    int col, g;
-    const bool work = red_thread(n, ld, rch, st, r0, r1, col, g);
+__global__ void __launch_bounds__(256) k_update(float* __restrict__ X, float* __restrict__ R,
+                                                const float* __restrict__ P, const float* __restrict__ Q, int64_t n,
+                                                int32_t ld, int rch, const ColState* __restrict__ st,
+                                                float xs, float2* __restrict__ part) {
+    const RedThread t = red_thread(n, ld, rch, st);
     KSum acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-    if (work) {
-        const float a0 = (float)st[col].a, a1 = (float)st[col + 1].a, a2 = (float)st[col + 2].a,
-                    a3 = (float)st[col + 3].a;
-        const float x0 = xs * a0, x1 = xs * a1, x2 = xs * a2, x3 = xs * a3;
-        // a served column that took a new request at the last scalar step starts
-        // from x0 = 0, r0 = y: x = a p, r = -a q here, y is added next
-        const bool f0 = st[col].refill, f1 = st[col + 1].refill, f2 = st[col + 2].refill, f3 = st[col + 3].refill;
-        const bool any_refill = f0 | f1 | f2 | f3;
-        for (int64_t row = r0; row < r1; row += RG) {
-            const int64_t o = row * ld + col;
+    if (t.work) {
+        const UpdateQuad uq = update_quad(st, t.col, xs);
+        for (int64_t row = t.r0; row < t.r1; row += RG) {
+            const int64_t o = row * ld + t.col;
             const float4 p = ld4v(P + o), q = ld4v(Q + o);
             float4 x = ld4v(X + o), r = ld4v(R + o);
-            if (any_refill) {
-                if (f0) x.x = r.x = 0.0f;
-                if (f1) x.y = r.y = 0.0f;
-                if (f2) x.z = r.z = 0.0f;
-                if (f3) x.w = r.w = 0.0f;
-            }
-            x.x = fmaf(x0, p.x, x.x); x.y = fmaf(x1, p.y, x.y); x.z = fmaf(x2, p.z, x.z); x.w = fmaf(x3, p.w, x.w);
-            r.x = fmaf(-a0, q.x, r.x); r.y = fmaf(-a1, q.y, r.y); r.z = fmaf(-a2, q.z, r.z); r.w = fmaf(-a3, q.w, r.w);
+            update_row(uq, p, q, x, r);
             st4(X + o, x);
             st4(R + o, r);
-            ksum_add(acc[0], r.x * r.x);
-            ksum_add(acc[1], r.y * r.y);
-            ksum_add(acc[2], r.z * r.z);
-            ksum_add(acc[3], r.w * r.w);
+            ksum_add_product(acc[0], r.x, r.x);
+            ksum_add_product(acc[1], r.y, r.y);
+            ksum_add_product(acc[2], r.z, r.z);
+            ksum_add_product(acc[3], r.w, r.w);
         }
     }
-    red_finish(part, ld, work, col, g, acc);
+    red_finish(part, ld, t, acc);
+}
+
+// The three sums above for small grids: block (chunk, group of 4 quads).
+enum RedOp { RED_SQ, RED_DOT, RED_UPDATE };
+constexpr int RS_ROWS = 512;  // rows staged at a time (a whole chunk up to 2M rows)
+constexpr int RS_COLS = 16;   // columns of a block
+template <int OP>
+constexpr int rs_smem() {
+    return RS_ROWS * RS_COLS * 4 * (OP == RED_DOT ? 2 : 1);
+}
+template <int OP>
+__global__ void __launch_bounds__(256) k_red_staged(float* __restrict__ X, float* __restrict__ R,
+                                                    const float* __restrict__ P, const float* __restrict__ Q,
+                                                    int64_t n, int32_t ld, int rch, const ColState* __restrict__ st,
+                                                    float xs, float2* __restrict__ part) {
+    constexpr int UL = 4;  // rows in flight per thread
+    extern __shared__ float rs_sm[];
+    __shared__ float2 sums[RG * RS_COLS];
+    const int cq = min(RS_COLS / 4, (ld >> 2) - (int)blockIdx.y * (RS_COLS / 4)), nc = 4 * cq;
+    const int c0 = blockIdx.y * RS_COLS;
+    float4* A = reinterpret_cast<float4*>(rs_sm);  // [row][quad]
+    float4* B = A + RS_ROWS * cq;
+    const int64_t lo = (int64_t)blockIdx.x * rch, hi = min(n, lo + rch);
+    // loading threads: quad lq of the group, rows lr, lr + rows_per_pass, ...
+    const int lq = threadIdx.x % cq, lr = threadIdx.x / cq, pass = 256 / cq;
+    const int col = c0 + 4 * lq;
+    bool work = lr < pass;
+    UpdateQuad uq;
+    if (OP != RED_SQ) {
+        work = work && (st[col].active | st[col + 1].active | st[col + 2].active | st[col + 3].active);
+        if (OP == RED_UPDATE) uq = update_quad(st, col, xs);
+    }
+    // summing threads: column sc, partial sum sg
+    const int sc = threadIdx.x % nc, sg = threadIdx.x / nc;
+    bool sum = sg < RG;
+    if (OP != RED_SQ && sum) {
+        const ColState* q = st + c0 + (sc & ~3);
+        sum = q[0].active | q[1].active | q[2].active | q[3].active;
+    }
+    KSum acc{0.f, 0.f};
+    for (int64_t base = lo; base < hi; base += RS_ROWS) {
+        const int rows = (int)min((int64_t)RS_ROWS, hi - base);
+        if (work)
+            for (int r0 = lr; r0 < rows; r0 += UL * pass) {
+                float4 p[UL], q[UL], x[UL], r[UL];
+#pragma unroll
+                for (int u = 0; u < UL; ++u) {
+                    const int64_t o = (base + r0 + u * pass) * ld + col;
+                    if (r0 + u * pass < rows) {
+                        p[u] = ld4v(P + o);
+                        if (OP != RED_SQ) q[u] = ld4v(Q + o);
+                        if (OP == RED_UPDATE) {
+                            x[u] = ld4v(X + o);
+                            r[u] = ld4v(R + o);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < UL; ++u) {
+                    const int row = r0 + u * pass;
+                    if (row >= rows) break;
+                    if (OP == RED_UPDATE) {
+                        const int64_t o = (base + row) * ld + col;
+                        update_row(uq, p[u], q[u], x[u], r[u]);
+                        st4(X + o, x[u]);
+                        st4(R + o, r[u]);
+                        A[row * cq + lq] = r[u];
+                    } else {
+                        A[row * cq + lq] = p[u];
+                        if (OP == RED_DOT) B[row * cq + lq] = q[u];
+                    }
+                }
+            }
+        __syncthreads();
+        if (sum) {
+            const float* a = reinterpret_cast<const float*>(A);
+            const float* b = OP == RED_DOT ? reinterpret_cast<const float*>(B) : a;
+#pragma unroll 8
+            for (int row = sg; row < rows; row += RG) ksum_add_product(acc, a[row * nc + sc], b[row * nc + sc]);
+        }
+        __syncthreads();
+    }
+    if (sg < RG) sums[sg * RS_COLS + sc] = make_float2(acc.s, acc.c);
+    __syncthreads();
+    if (sum && sg == 0) {
+        KSum t = acc;
+#pragma unroll
+        for (int h = 1; h < RG; ++h) {
+            const float2 v = sums[h * RS_COLS + sc];
+            ksum_merge(t, KSum{v.x, v.y});
+        }
+        part[(int64_t)blockIdx.x * ld + c0 + sc] = make_float2(t.s, t.c);
+    }
 }
 
 // P = R + beta P.
@@ -933,12 +1076,18 @@ __device__ __forceinline__ double block_sum_f64(double v) {
     return t;
 }
 
-// sum over blocks of column j's compensated partials
+// sum over blocks of column j's compensated partials (eight loads ahead of their adds)
 __device__ __forceinline__ double col_sum(const float2* part, int nblk, int ld, int j) {
     double s = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
-        const float2 v = part[(int64_t)b * ld + j];
-        s += (double)v.x + (double)v.y;
+    const int step = blockDim.x;
+    for (int b = threadIdx.x; b < nblk; b += 8 * step) {
+        float2 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            v[u] = b + u * step < nblk ? part[(int64_t)(b + u * step) * ld + j] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (b + u * step < nblk) s += (double)v[u].x + (double)v[u].y;
     }
     return block_sum_f64(s);
 }
@@ -1388,7 +1537,14 @@ __global__ void __launch_bounds__(256) k_lr_finish(const float* __restrict__ par
     const int64_t tot = (int64_t)rpad * Bp;
     double s = 0.0;
     if (e < tot)
-        for (int c = w; c < nchunk; c += 8) s += (double)part[(int64_t)c * tot + e];
+        for (int c = w; c < nchunk; c += 64) {
+            float v[8];  // eight chunks' loads ahead of their adds
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = c + 8 * u < nchunk ? part[(int64_t)(c + 8 * u) * tot + e] : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (c + 8 * u < nchunk) s += (double)v[u];
+        }
     sm[w][lane] = s;
     __syncthreads();
     if (w != 0 || e >= tot) return;
@@ -1648,21 +1804,41 @@ int hd_spmm_apply(hd_ctx* ctx, const hd_graph* g, const float* P, float* Q, int3
     return spmm_launch(ctx, g, P, Q, ld, 4 * spmm_lanes(ld, 4, spmm_exceeds_l2(g->n, ld, 4)), c1, c2, nullptr, nullptr);
 }
 
-// grid and block of the column reductions: one block row per chunk, up to 128 quads x 8 threads
-static inline dim3 red_grid(const Engine& E) {
-    const int nq = E.Bp / 4;
-    return dim3((unsigned)E.nch, (unsigned)ceil_div(nq, RQ));
+// grid and block of the column reductions: one chunk per block row.  `staged`
+// (k_red_staged) when the thread-per-(g, quad) form would leave the GPU less
+// than half full: it lives off resident warps, about 1,024 threads per SM.
+struct RedLaunch {
+    dim3 grid;
+    unsigned block;
+    size_t smem;
+    bool staged;
+};
+static RedLaunch red_launch(const Engine& E) {
+    const int nq = E.Bp / 4, qpb = nq < RQ ? nq : RQ;
+    RedLaunch l;
+    l.staged = E.nch * nq * RG < (int64_t)E.ctx->num_sms * 1024;
+    l.grid = dim3((unsigned)E.nch, (unsigned)ceil_div(E.Bp, l.staged ? RS_COLS : 4 * RQ));
+    l.block = l.staged ? 256u : (unsigned)(RG * qpb);
+    l.smem = (size_t)l.block * 4 * sizeof(float2);
+    return l;
 }
-static inline unsigned red_block(const Engine& E) {
-    const int nq = E.Bp / 4;
-    return (unsigned)(RG * (nq < RQ ? nq : RQ));
+template <int OP>
+static int launch_staged(Engine& E, const RedLaunch& l, const float* P, float2* part, const ColState* st) {
+    hd_ctx* ctx = E.ctx;
+    static uint64_t attr = 0;
+    if (hd_first_on_device(attr, ctx->device))
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_red_staged<OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs_smem<OP>()));
+    k_red_staged<OP><<<l.grid, l.block, rs_smem<OP>(), ctx->stream>>>(E.X, E.R, P, E.Q, E.n, E.Bp, E.rch, st, E.xs, part);
+    HD_CHECK_LAUNCH(ctx);
+    return HD_OK;
 }
-static inline size_t red_smem(const Engine& E) { return (size_t)red_block(E) * 4 * sizeof(float2); }
 
 static int launch_dot(Engine& E, float2* part, const ColState* st) {
     hd_ctx* ctx = E.ctx;
     HD_PROF(ctx, "dot");
-    k_dot<<<red_grid(E), red_block(E), red_smem(E), ctx->stream>>>(E.P, E.Q, E.n, E.Bp, E.rch, part, st);
+    const RedLaunch l = red_launch(E);
+    if (l.staged) return launch_staged<RED_DOT>(E, l, E.P, part, st);
+    k_dot<<<l.grid, l.block, l.smem, ctx->stream>>>(E.P, E.Q, E.n, E.Bp, E.rch, part, st);
     HD_CHECK_LAUNCH(ctx);
     return HD_OK;
 }
@@ -1670,7 +1846,9 @@ static int launch_dot(Engine& E, float2* part, const ColState* st) {
 static int launch_update(Engine& E) {
     hd_ctx* ctx = E.ctx;
     HD_PROF(ctx, "update");
-    k_update<<<red_grid(E), red_block(E), red_smem(E), ctx->stream>>>(E.X, E.R, E.P, E.Q, E.n, E.Bp, E.rch, E.st, E.xs, E.part);
+    const RedLaunch l = red_launch(E);
+    if (l.staged) return launch_staged<RED_UPDATE>(E, l, E.P, E.part, E.st);
+    k_update<<<l.grid, l.block, l.smem, ctx->stream>>>(E.X, E.R, E.P, E.Q, E.n, E.Bp, E.rch, E.st, E.xs, E.part);
     HD_CHECK_LAUNCH(ctx);
     return HD_OK;
 }
@@ -1678,7 +1856,9 @@ static int launch_update(Engine& E) {
 static int launch_colsq(Engine& E, const float* V) {
     hd_ctx* ctx = E.ctx;
     HD_PROF(ctx, "colsq");
-    k_colsq<<<red_grid(E), red_block(E), red_smem(E), ctx->stream>>>(V, E.n, E.Bp, E.rch, E.part);
+    const RedLaunch l = red_launch(E);
+    if (l.staged) return launch_staged<RED_SQ>(E, l, V, E.part, nullptr);
+    k_colsq<<<l.grid, l.block, l.smem, ctx->stream>>>(V, E.n, E.Bp, E.rch, E.part);
     HD_CHECK_LAUNCH(ctx);
     return HD_OK;
 }
@@ -2080,7 +2260,7 @@ static int true_residual(Engine& E, double alpha) {
             if ((rc = lr_expand(ctx, E.lr, EXP_SUB_R, E.Q, nullptr, nullptr, n, Bp, nullptr))) return rc;
         }
     }
-    k_scatter_y<<<ceil_div(E.B, 128), 128, 0, ctx->stream>>>(E.yp, E.yi, E.yv, E.B, n, Bp, E.Q, E.err);
+    k_scatter_y<<<E.B, 128, 0, ctx->stream>>>(E.yp, E.yi, E.yv, n, Bp, E.Q, E.err);
     HD_CHECK_LAUNCH(ctx);
     return launch_colsq(E, E.Q);
 }
@@ -2291,8 +2471,8 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     HD_CUDA(ctx, cudaMemsetAsync(S_.R, 0, vec, ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(S_.X, 0, vec, ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(S_.err, 0, sizeof(int), ctx->stream));
-    k_scatter_y<<<ceil_div(B, 128), 128, 0, ctx->stream>>>((const int32_t*)yp, (const int32_t*)yi, (const float*)yv,
-                                                           B, n, Bp, S_.R, S_.err);
+    k_scatter_y<<<B, 128, 0, ctx->stream>>>((const int32_t*)yp, (const int32_t*)yi, (const float*)yv, n, Bp, S_.R,
+                                            S_.err);
     HD_CHECK_LAUNCH(ctx);
     const double* Cd = lr_on ? S_.lr.C : nullptr;
     const size_t cbytes = (size_t)rpad * Bp * sizeof(double);
@@ -2331,7 +2511,7 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         k_fin_setup<<<Bp, 128, 0, ctx->stream>>>(S_.part, (int)S_.nch, Bp, B, (const float*)tl, S_.st, Cd, S_.dcoef, r,
                                                 S_.num_active);
         HD_CHECK_LAUNCH(ctx);
-        HD_CUDA(ctx, cudaMemsetAsync(S_.P, 0, vec, ctx->stream));
+        // (beta is 0: whatever P holds is dropped)
         if ((rc = lr_expand(ctx, S_.lr, EXP_DIRECTION, S_.P, S_.R, S_.P, n, Bp, S_.st))) return rc;
     }
 
@@ -2561,8 +2741,7 @@ extern "C" int hd_filter_poly(hd_ctx* ctx, const hd_graph* g, const hd_eig* eig,
     }
     HD_CUDA(ctx, cudaMemsetAsync(Yd, 0, vec, ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
-    k_scatter_y<<<ceil_div(B, 128), 128, 0, ctx->stream>>>((const int32_t*)yp, (const int32_t*)yi, (const float*)yv, B,
-                                                           n, Bp, Yd, err);
+    k_scatter_y<<<B, 128, 0, ctx->stream>>>((const int32_t*)yp, (const int32_t*)yi, (const float*)yv, n, Bp, Yd, err);
     HD_CHECK_LAUNCH(ctx);
     const int64_t c4 = (int64_t)n * Bp / 4;
     // h(W_r) y by Horner's rule on the black box W_r z = W z - U (Lambda (U^T z)) (Eq. 32)
