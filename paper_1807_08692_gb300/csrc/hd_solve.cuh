@@ -75,10 +75,19 @@ struct LowRank {
     int32_t live = 0;   // > 0: only columns below this can be active (tensor-core paths skip the rest)
 };
 
+// What one iteration clears for its scalar step and for the next fp16 copy (see
+// iter_reset): max |P_j| of the Bp columns, the active count, the fp16 vote.
+struct IterReset {
+    unsigned* p16_max = nullptr;
+    int32_t Bp = 0;
+    int* num_active = nullptr;
+    int* use_half = nullptr;
+};
+
 // `gate` (device int, may be null): the kernels return at once when it is 0
 // (no column active), so iterations past convergence cost only their launch.
 int lr_reduce(hd_ctx* ctx, const LowRank& lr, const float* V, int64_t n, int32_t Bp, const int* gate = nullptr);
-int lr_finish(hd_ctx* ctx, const LowRank& lr, int32_t Bp, const double* coef);
+int lr_finish(hd_ctx* ctx, const LowRank& lr, int32_t Bp, const double* coef, const IterReset& z = {});
 int lr_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float* Rv, const float* Pv, int64_t n,
               int32_t Bp, const ColState* st, const int* gate = nullptr);
 bool lr_use_tensor_cores(const hd_eig* e);
