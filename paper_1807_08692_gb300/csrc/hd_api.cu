@@ -61,6 +61,23 @@ int hd_ws_reserve(hd_ctx* ctx, size_t bytes, void** out) {
     return HD_OK;
 }
 
+int hd_host_stage(hd_ctx* ctx, size_t bytes, void** out) {
+    if (bytes > ctx->h_stage_bytes) {
+        if (ctx->h_stage) HD_CUDA(ctx, cudaFreeHost(ctx->h_stage));
+        ctx->h_stage = nullptr;
+        ctx->h_stage_bytes = 0;
+        const size_t want = (bytes + bytes / 4 + 4095) & ~(size_t)4095;
+        if (cudaMallocHost(&ctx->h_stage, want) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->h_stage = nullptr;
+            return hd_fail(ctx, HD_ERR_OOM, "pinned staging of %zu bytes", want);
+        }
+        ctx->h_stage_bytes = want;
+    }
+    *out = ctx->h_stage;
+    return HD_OK;
+}
+
 int hd_stage_in(hd_ctx* ctx, const void* src, size_t bytes, void* dev_scratch, const void** dev_out) {
     if (bytes == 0 || hd_is_device_ptr(src)) {
         *dev_out = src;
@@ -119,6 +136,7 @@ int hd_destroy(hd_ctx* ctx) {
     hd_rank_static_forget(ctx->device);
     if (ctx->ws) cudaFree(ctx->ws);
     if (ctx->h_poll) cudaFreeHost(ctx->h_poll);
+    if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
     if (ctx->d_flags) cudaFree(ctx->d_flags);
     for (auto& kv : ctx->iter_graphs) cudaGraphExecDestroy(kv.second.exec);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);

@@ -23,6 +23,9 @@ struct hd_ctx {
     size_t ws_bytes = 0;
     // pinned host words for polling device counters
     int* h_poll = nullptr;
+    // grow-only pinned staging block (hd_host_stage)
+    void* h_stage = nullptr;
+    size_t h_stage_bytes = 0;
     int* d_flags = nullptr;   // [0]: device-side error flag, [1..]: misc counters
     // CUDA graphs of runs of CG iterations, keyed by everything the kernels
     // take as arguments plus the run length (a few kept; re-captured when the
@@ -148,6 +151,9 @@ bool hd_is_device_ptr(const void* p);
 // Workspace: returns a device pointer of at least `bytes`, 256-aligned,
 // valid until the next hd_ws_reserve on the same context.
 int hd_ws_reserve(hd_ctx* ctx, size_t bytes, void** out);
+// Pinned host block of at least `bytes`, valid until the next hd_host_stage on the
+// same context; the caller leaves no copy in flight from or to it.
+int hd_host_stage(hd_ctx* ctx, size_t bytes, void** out);
 // drop the cached device address of hd_rank_static's scratch on a device
 void hd_rank_static_forget(int device);
 struct WsCarver {

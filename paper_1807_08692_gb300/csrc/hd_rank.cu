@@ -13,6 +13,7 @@
 // with a bitonic sort on (key, ~id).
 #include <algorithm>
 #include <atomic>
+#include <cstring>
 #include <vector>
 
 #include "hd_internal.cuh"
@@ -183,8 +184,10 @@ __global__ void k_sort_out(const uint64_t* cand, const SelState* st, int32_t Kma
 constexpr int TK_SAMPLE = 4096;
 constexpr int TK_CAP = 16384;
 constexpr int TK_TOP = 2048;  // K <= Kmax <= 2048
+constexpr int TK_PAD = 32;    // ints between two columns' candidate counters: one 128-byte line each, so that
+                              // the columns' atomics do not queue in the one L2 slice holding them all
 // dynamic shared memory of k_topk_sort: candidates, the top K, histogram, scalars
-constexpr size_t TK_SORT_SMEM = (size_t)(TK_CAP + TK_TOP) * 8 + 256 * 4 + 2 * 8 + 16;
+constexpr size_t TK_SORT_SMEM = (size_t)(TK_CAP + TK_TOP) * 8 + 256 * 4 + 3 * 8 + 16;
 
 // Each thread takes compare-exchange pairs directly (pair q: t = the q-th index
 // with bit `stride` clear, u = t + stride), so no thread idles in a stage.
@@ -205,15 +208,29 @@ __device__ __forceinline__ void bitonic_desc_u64(uint64_t* a, int P) {
         }
 }
 
-// The k-th largest (1-based, counting repeats) of a[0 .. cnt) in shared
-// memory, by a most-significant-digit radix select over the low `nbits` bits
-// (8 per round): a 256-bin histogram of the elements that match the digits
-// chosen so far, then one warp finds the bin that holds the k-th (each lane sums
-// 8 bins, a shuffle scan over the lanes).  All threads of the block call it.
+// A threshold that exactly the k largest (1-based, counting repeats) of a[0 ..
+// cnt) in shared memory reach, or more of them when the k-th repeats: a
+// most-significant-digit radix select over the low `nbits` bits (8 per round).
+// Each round takes a 256-bin histogram of the elements that match the digits
+// chosen so far, then one warp finds the bin that holds the k-th (each lane
+// sums 8 bins, a shuffle scan over the lanes).  Rounds over digits that all
+// elements share are skipped (their one bin would take every atomic), and the
+// select ends when the whole bin is taken.  All threads of the block call it.
 __device__ uint64_t block_kth_desc(const uint64_t* a, int cnt, int k, int nbits, uint32_t* hist, uint64_t* sh) {
-    uint64_t prefix = 0;
+    // the bits in which the elements differ
+    uint64_t diff = 0;
+    for (int i = threadIdx.x; i < cnt; i += blockDim.x) diff |= a[i] ^ a[0];
+    uint32_t dl = __reduce_or_sync(0xffffffffu, (uint32_t)diff), dh = __reduce_or_sync(0xffffffffu, (uint32_t)(diff >> 32));
+    if (threadIdx.x == 0) sh[2] = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) atomicOr((unsigned long long*)&sh[2], (unsigned long long)dh << 32 | dl);
+    __syncthreads();
+    diff = sh[2];
+    int shift = nbits - 8;
+    while (shift >= 0 && !(diff >> shift)) shift -= 8;
+    uint64_t prefix = shift + 8 >= 64 ? 0ull : (a[0] >> (shift + 8)) << (shift + 8);
     int krem = k;
-    for (int shift = nbits - 8; shift >= 0; shift -= 8) {
+    for (; shift >= 0; shift -= 8) {
         for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
         __syncthreads();
         const uint64_t hi = shift + 8 >= 64 ? 0ull : (~0ull << (shift + 8));
@@ -239,23 +256,26 @@ __device__ uint64_t block_kth_desc(const uint64_t* a, int cnt, int k, int nbits,
             const int excl = incl - sum;
             const unsigned m = __ballot_sync(0xffffffffu, excl < krem && krem <= incl);
             if (m && lane == __ffs(m) - 1) {
-                int cum = excl, d = 255 - 8 * lane - 7;
+                int cum = excl, d = 255 - 8 * lane - 7, in_bin = h[7];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     if (cum + h[q] >= krem) {
                         d = 255 - 8 * lane - q;
+                        in_bin = h[q];
                         break;
                     }
                     cum += h[q];
                 }
                 sh[0] = prefix | ((uint64_t)d << shift);
-                sh[1] = (uint64_t)(krem - cum);
+                sh[1] = (uint64_t)(krem - cum) << 32 | (uint64_t)(in_bin == krem - cum);
             }
         }
         __syncthreads();
         prefix = sh[0];
-        krem = (int)sh[1];
+        krem = (int)(sh[1] >> 32);
+        const bool whole = sh[1] & 1;
         __syncthreads();
+        if (whole) break;
     }
     return prefix;
 }
@@ -268,7 +288,7 @@ __global__ void __launch_bounds__(1024) k_topk_sample(const float* X, int64_t n,
     if (K <= 0) {  // nothing to rank in this column (the filter and the sort skip it too)
         if (threadIdx.x == 0) {
             tau[j] = 0xFFFFFFFFu;
-            cnt[j] = 0;
+            cnt[j * TK_PAD] = 0;
         }
         return;
     }
@@ -284,21 +304,75 @@ __global__ void __launch_bounds__(1024) k_topk_sample(const float* X, int64_t n,
     __syncthreads();
     // the threshold is the (kp + 1)-th largest sample (a radix select, not a sort)
     __shared__ uint32_t hist[256];
-    __shared__ uint64_t sh[2];
+    __shared__ uint64_t sh[3];
     int64_t kp = (4 * K * s + n - 1) / n + 8;
     if (kp > s - 1) kp = s - 1;
     const uint64_t t = block_kth_desc(sk, TK_SAMPLE, (int)kp + 1, 32, hist, sh);
     if (threadIdx.x == 0) {
         tau[j] = (uint32_t)t;
-        cnt[j] = 0;
+        cnt[j * TK_PAD] = 0;
     }
 }
 
-// Each thread keeps one column (B <= 256: 256 / B rows per block step) so the
-// column's threshold and K stay in registers and no index is divided per element;
-// eight rows' loads are issued before their compares (0.136 ms against 0.159 ms
-// for a 1M x 64 block, cold L2).
+// The one pass over the scores.  Rows without gaps (ld = B, 16-byte aligned):
+// the block is read as one array of float4, the whole grid stepping by a
+// multiple of B, so that a thread's four columns and their thresholds stay the
+// same and only a candidate needs its row number.  Six blocks
+// per SM with two loads in flight per thread: a warp that claims a place for a
+// candidate waits for the answer, and more warps cover that better than more
+// loads per warp (1M x 64: 54 us; four blocks of four loads 58, two of eight 81;
+// candidates held back in shared memory 94; 131 us with 4-byte loads and
+// adjacent counters).  Other layouts:
+// each thread keeps one column (B <= 256: 256 / B rows per block step), eight
+// rows' 4-byte loads ahead of their compares.
 constexpr int TK_ROWS = 8;
+__device__ __forceinline__ void topk_push(int* cnt, uint64_t* cand, int j, uint32_t key, int64_t i) {
+    const int p = atomicAdd(&cnt[j * TK_PAD], 1);
+    if (p < TK_CAP) cand[(int64_t)j * TK_CAP + p] = ((uint64_t)key << 32) | (uint64_t)(~(uint32_t)i);
+}
+constexpr int TK_FLAT = 2;  // float4 loads in flight per thread of the flat pass
+__global__ void __launch_bounds__(256, 6) k_topk_filter_flat(const float* X, int64_t total, int32_t B, int64_t step4,
+                                                             const int32_t* Kd, const uint32_t* tau, int* cnt,
+                                                             uint64_t* cand) {
+    const int64_t t = blockIdx.x * 256ll + threadIdx.x;  // float4 of this thread's first load
+    if (t < (total & 3)) {  // the last elements of a block that is no multiple of four
+        const int64_t e = (total & ~3ll) + t;
+        const int jt = (int)(e % B);
+        const uint32_t key = float_key(X[e]);
+        if (__ldg(Kd + jt) > 0 && key >= __ldg(tau + jt)) topk_push(cnt, cand, jt, key, e / B);
+    }
+    if (t >= step4) return;
+    const int j0 = (int)(4 * t % B);
+    uint32_t tj[4];
+    unsigned take = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int j = (int)((4 * t + c) % B);
+        tj[c] = __ldg(tau + j);
+        take |= (__ldg(Kd + j) > 0) << c;
+    }
+    if (!take) return;
+    const int64_t n4 = total >> 2;
+    const float4* p = reinterpret_cast<const float4*>(X);
+    auto check = [&](const float4& v, int64_t e) {
+        const uint32_t k0 = float_key(v.x), k1 = float_key(v.y), k2 = float_key(v.z), k3 = float_key(v.w);
+        if (k0 >= tj[0] || k1 >= tj[1] || k2 >= tj[2] || k3 >= tj[3]) {
+            const uint32_t key[4] = {k0, k1, k2, k3};
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if ((take >> c & 1) && key[c] >= tj[c]) topk_push(cnt, cand, (j0 + c) % B, key[c], (4 * e + c) / B);
+        }
+    };
+    int64_t e = t;
+    for (; e + (TK_FLAT - 1) * step4 < n4; e += TK_FLAT * step4) {
+        float4 v[TK_FLAT];
+#pragma unroll
+        for (int u = 0; u < TK_FLAT; ++u) v[u] = __ldcs(p + e + u * step4);
+#pragma unroll
+        for (int u = 0; u < TK_FLAT; ++u) check(v[u], e + u * step4);
+    }
+    for (; e < n4; e += step4) check(__ldcs(p + e), e);
+}
 __global__ void __launch_bounds__(256) k_topk_filter(const float* X, int64_t n, int32_t B, int32_t ld,
                                                      const int32_t* Kd, const uint32_t* tau, int* cnt, uint64_t* cand) {
     const bool narrow = B <= 256;
@@ -320,10 +394,7 @@ __global__ void __launch_bounds__(256) k_topk_filter(const float* X, int64_t n, 
             for (int u = 0; u < TK_ROWS; ++u) {
                 const int64_t i = i0 + u * step;
                 const uint32_t key = float_key(v[u]);
-                if (i < n && key >= tj) {
-                    const int p = atomicAdd(&cnt[j], 1);
-                    if (p < TK_CAP) cand[(int64_t)j * TK_CAP + p] = ((uint64_t)key << 32) | (uint64_t)(~(uint32_t)i);
-                }
+                if (i < n && key >= tj) topk_push(cnt, cand, j, key, i);
             }
         }
     }
@@ -334,18 +405,18 @@ __global__ void __launch_bounds__(1024) k_topk_sort(const uint64_t* cand, const 
     extern __shared__ uint64_t sk[];
     const int j = blockIdx.x;
     const int K = (int)((int64_t)Kd[j] < n ? (int64_t)Kd[j] : n);
-    const int c = cnt[j];
+    const int c = cnt[j * TK_PAD];
     if (K > 0 && (c < K || c > TK_CAP)) {
         if (threadIdx.x == 0) fail[j] = 1;
         return;
     }
     if (threadIdx.x == 0) fail[j] = 0;
-    // candidates' keys (score key, ~id) are distinct: exactly K lie at or above
-    // the K-th largest, which a radix select finds; only those K are sorted
+    // candidates' keys (score key, ~id) are distinct: a radix select finds a
+    // threshold that exactly K reach; only those K are sorted
     uint64_t* top = sk + TK_CAP;  // [TK_TOP]
     uint32_t* hist = reinterpret_cast<uint32_t*>(top + TK_TOP);
     uint64_t* sh = reinterpret_cast<uint64_t*>(hist + 256);
-    int* fill = reinterpret_cast<int*>(sh + 2);
+    int* fill = reinterpret_cast<int*>(sh + 3);
     int P = 1;
     while (P < K) P <<= 1;
     if (K > 0) {
@@ -378,12 +449,16 @@ static int radix_rank(hd_ctx* ctx, const float* src, int64_t m, int32_t B, int32
                       int32_t Kmax, int32_t* idx_d, float* score_d, int skip_empty, WsCarver& cv);
 
 int hd_rank_impl(hd_ctx* ctx, const float* Xd, int64_t n, int32_t B, int32_t ldx, const int32_t* K_h, int32_t Kmax,
-                 int32_t pool, int32_t* idx_d, float* score_d) {
+                 int32_t pool, int32_t* idx_out, float* score_out) {
     const float* src = Xd;
     int64_t m = n;
     int32_t ld = ldx;
+    // results for the host go through the workspace in one block, ids then scores, behind the columns' status
+    const bool host = !(hd_is_device_ptr(idx_out) && hd_is_device_ptr(score_out));
+    const size_t res = (size_t)B * Kmax * 4, out_bytes = (size_t)B * 4 + (host ? 2 * res : 0);
     size_t bytes = ws_size(B * sizeof(SelState)) + ws_size((size_t)B * 256 * 4) + ws_size((size_t)B * Kmax * 8) +
-                   ws_size(B * 4) + ws_size((size_t)B * TK_CAP * 8) + 3 * ws_size(B * 4) + ws_size(B * 4);
+                   2 * ws_size(B * 4) + ws_size((size_t)B * TK_CAP * 8) + ws_size(B * 4) +
+                   ws_size((size_t)B * TK_PAD * 4) + ws_size(out_bytes);
     if (pool > 1) {
         m = n / pool;
         bytes += ws_size((size_t)m * B * 4);
@@ -391,12 +466,16 @@ int hd_rank_impl(hd_ctx* ctx, const float* Xd, int64_t n, int32_t B, int32_t ldx
     void* ws;
     int rc = hd_ws_reserve(ctx, bytes, &ws);
     if (rc) return rc;
+    char* hs;  // pinned: K on the way in, status and host results on the way out
+    if ((rc = hd_host_stage(ctx, (size_t)B * 4 + out_bytes, (void**)&hs))) return rc;
     WsCarver cv(ws);
     int32_t* Kd = cv.take<int32_t>(B);
     uint64_t* cand = cv.take<uint64_t>((size_t)B * TK_CAP);
     uint32_t* tau = cv.take<uint32_t>(B);
-    int* cnt = cv.take<int>(B);
-    int* fail = cv.take<int>(B);
+    int* cnt = cv.take<int>((size_t)B * TK_PAD);
+    int* fail = cv.take<int>(out_bytes / 4);
+    int32_t* idx_d = host ? fail + B : idx_out;
+    float* score_d = host ? (float*)(fail + B) + (size_t)B * Kmax : score_out;
     if (pool > 1) {
         float* Y = cv.take<float>((size_t)m * B);
         k_pool<<<ceil_div(m * B, 256), 256, 0, ctx->stream>>>(Xd, m, B, ldx, pool, Y);
@@ -404,30 +483,52 @@ int hd_rank_impl(hd_ctx* ctx, const float* Xd, int64_t n, int32_t B, int32_t ldx
         src = Y;
         ld = B;
     }
-    HD_CUDA(ctx, cudaMemcpyAsync(Kd, K_h, B * 4, cudaMemcpyHostToDevice, ctx->stream));
+    std::copy(K_h, K_h + B, (int32_t*)hs);
+    HD_CUDA(ctx, cudaMemcpyAsync(Kd, hs, B * 4, cudaMemcpyHostToDevice, ctx->stream));
     static uint64_t attr = 0;
     if (hd_first_on_device(attr, ctx->device)) {
         HD_CUDA(ctx, cudaFuncSetAttribute(k_topk_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, TK_SORT_SMEM));
     }
     k_topk_sample<<<B, 1024, 0, ctx->stream>>>(src, m, ld, Kd, tau, cnt);
     HD_CHECK_LAUNCH(ctx);
-    const int gc = std::max(1, std::min<int>(ceil_div(m * B, 256 * 8), ctx->num_sms * 8));
-    k_topk_filter<<<gc, 256, 0, ctx->stream>>>(src, m, B, ld, Kd, tau, cnt, cand);
+    if (ld == B && ((uintptr_t)src & 15) == 0) {
+        // threads: six blocks per SM or as many as there are loads, rounded up so that a step of the grid is a multiple of B
+        const int64_t per = B % 4 == 0 ? B / 4 : B % 2 == 0 ? B / 2 : B;  // float4 loads in lcm(4, B) elements
+        const int64_t want = std::max<int64_t>(1, std::min<int64_t>(m * B / 4 / TK_FLAT, ctx->num_sms * 1536ll));
+        const int64_t step4 = (want + per - 1) / per * per;
+        k_topk_filter_flat<<<ceil_div(step4, 256), 256, 0, ctx->stream>>>(src, m * B, B, step4, Kd, tau, cnt, cand);
+    } else {
+        const int gc = std::max(1, std::min<int>(ceil_div(m * B, 256 * 8), ctx->num_sms * 8));
+        k_topk_filter<<<gc, 256, 0, ctx->stream>>>(src, m, B, ld, Kd, tau, cnt, cand);
+    }
     HD_CHECK_LAUNCH(ctx);
     k_topk_sort<<<B, 1024, TK_SORT_SMEM, ctx->stream>>>(cand, cnt, Kd, m, Kmax, idx_d, score_d, fail);
     HD_CHECK_LAUNCH(ctx);
-    std::vector<int> hf(B);
-    HD_CUDA(ctx, cudaMemcpyAsync(hf.data(), fail, B * 4, cudaMemcpyDeviceToHost, ctx->stream));
+    int* hf = (int*)(hs + (size_t)B * 4);
+    HD_CUDA(ctx, cudaMemcpyAsync(hf, fail, out_bytes, cudaMemcpyDeviceToHost, ctx->stream));
     HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    std::vector<int32_t> Kf(B, 0);
-    bool any = false;
+    std::vector<int32_t> Kf;
     for (int j = 0; j < B; ++j)
         if (hf[j]) {
+            if (Kf.empty()) Kf.assign(B, 0);
             Kf[j] = K_h[j];
-            any = true;
         }
-    if (!any) return HD_OK;
-    return radix_rank(ctx, src, m, B, ld, Kf.data(), Kmax, idx_d, score_d, 1, cv);
+    if (!Kf.empty()) {
+        if ((rc = radix_rank(ctx, src, m, B, ld, Kf.data(), Kmax, idx_d, score_d, 1, cv))) return rc;
+        if (host) {
+            HD_CUDA(ctx, cudaMemcpyAsync(hf + B, idx_d, 2 * res, cudaMemcpyDeviceToHost, ctx->stream));
+            HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        }
+    }
+    if (host) {
+        const void* from[2] = {hf + B, hf + B + (size_t)B * Kmax};
+        void* to[2] = {idx_out, score_out};
+        for (int q = 0; q < 2; ++q) {
+            if (hd_is_device_ptr(to[q])) HD_CUDA(ctx, cudaMemcpy(to[q], from[q], res, cudaMemcpyHostToDevice));
+            else memcpy(to[q], from[q], res);
+        }
+    }
+    return HD_OK;
 }
 
 // Exact radix select for the columns with K > 0 (the others are left untouched
@@ -485,26 +586,8 @@ extern "C" int hd_rank(hd_ctx* ctx, const float* X, int64_t n, int32_t B, int32_
     for (int j = 0; j < B; ++j)
         if (K[j] < 0 || K[j] > Kmax) return hd_fail(ctx, HD_ERR_INVALID_ARG, "K[%d]=%d outside [0, Kmax]", j, K[j]);
     HD_CUDA(ctx, cudaSetDevice(ctx->device));
-    bool dev = hd_is_device_ptr(idx_out) && hd_is_device_ptr(score_out);
-    int32_t* id = idx_out;
-    float* sd = score_out;
-    if (!dev) {
-        HD_CUDA(ctx, cudaMallocAsync(&id, (size_t)B * Kmax * 4, ctx->stream));
-        HD_CUDA(ctx, cudaMallocAsync(&sd, (size_t)B * Kmax * 4, ctx->stream));
-    }
-    int rc;
-    {
-        HD_PROF(ctx, "rank");
-        rc = hd_rank_impl(ctx, X, n, B, ldx, K, Kmax, pool, id, sd);
-    }
-    if (!rc && !dev) {
-        HD_CUDA(ctx, cudaMemcpyAsync(idx_out, id, (size_t)B * Kmax * 4, cudaMemcpyDeviceToHost, ctx->stream));
-        HD_CUDA(ctx, cudaMemcpyAsync(score_out, sd, (size_t)B * Kmax * 4, cudaMemcpyDeviceToHost, ctx->stream));
-        HD_CUDA(ctx, cudaFreeAsync(id, ctx->stream));
-        HD_CUDA(ctx, cudaFreeAsync(sd, ctx->stream));
-        HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    }
-    return rc;
+    HD_PROF(ctx, "rank");
+    return hd_rank_impl(ctx, X, n, B, ldx, K, Kmax, pool, idx_out, score_out);
 }
 
 // ------------------------------------------------------------------ allocation-free ranking
