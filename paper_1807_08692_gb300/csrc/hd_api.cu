@@ -40,25 +40,41 @@ bool hd_is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-int hd_ws_reserve(hd_ctx* ctx, size_t bytes, void** out) {
+static int reserve_block(hd_ctx* ctx, void** block, size_t* have, size_t bytes, void** out) {
     if (bytes == 0) bytes = 256;
-    if (bytes > ctx->ws_bytes) {
-        if (ctx->ws) {
+    if (bytes > *have) {
+        if (*block) {
             HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-            HD_CUDA(ctx, cudaFree(ctx->ws));
-            ctx->ws = nullptr;
-            ctx->ws_bytes = 0;
+            HD_CUDA(ctx, cudaFree(*block));
+            *block = nullptr;
+            *have = 0;
         }
         size_t want = bytes + bytes / 8;
-        cudaError_t e = cudaMalloc(&ctx->ws, want);
+        cudaError_t e = cudaMalloc(block, want);
         if (e != cudaSuccess) {
             cudaGetLastError();
+            *block = nullptr;
             return hd_fail(ctx, HD_ERR_OOM, "workspace of %zu bytes: %s", want, cudaGetErrorString(e));
         }
-        ctx->ws_bytes = want;
+        *have = want;
     }
-    *out = ctx->ws;
+    *out = *block;
     return HD_OK;
+}
+
+int hd_ws_reserve(hd_ctx* ctx, size_t bytes, void** out) {
+    return reserve_block(ctx, &ctx->ws, &ctx->ws_bytes, bytes, out);
+}
+
+int hd_aux_reserve(hd_ctx* ctx, int which, size_t bytes, void** out) {
+    return reserve_block(ctx, &ctx->aux[which], &ctx->aux_bytes[which], bytes, out);
+}
+
+void hd_aux_trim(hd_ctx* ctx, int which, size_t most) {
+    if (ctx->aux_bytes[which] <= most) return;
+    cudaFree(ctx->aux[which]);
+    ctx->aux[which] = nullptr;
+    ctx->aux_bytes[which] = 0;
 }
 
 int hd_host_stage(hd_ctx* ctx, size_t bytes, void** out) {
@@ -135,6 +151,7 @@ int hd_destroy(hd_ctx* ctx) {
     cudaStreamSynchronize(ctx->stream);
     hd_rank_static_forget(ctx->device);
     if (ctx->ws) cudaFree(ctx->ws);
+    for (void* a : ctx->aux) cudaFree(a);
     if (ctx->h_poll) cudaFreeHost(ctx->h_poll);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
     if (ctx->d_flags) cudaFree(ctx->d_flags);
@@ -188,7 +205,7 @@ int hd_profile_read(hd_ctx* ctx, const char* name, int64_t* launches, double* to
 int64_t hd_launch_count(const hd_ctx* ctx) { return ctx ? ctx->launches : 0; }
 int hd_workspace_bytes(const hd_ctx* ctx, size_t* bytes) {
     if (!ctx || !bytes) return HD_ERR_INVALID_ARG;
-    *bytes = ctx->ws_bytes;
+    *bytes = ctx->ws_bytes + ctx->aux_bytes[0] + ctx->aux_bytes[1];
     return HD_OK;
 }
 int hd_num_sms(const hd_ctx* ctx) { return ctx ? ctx->num_sms : 0; }

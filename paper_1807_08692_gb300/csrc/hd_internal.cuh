@@ -21,6 +21,10 @@ struct hd_ctx {
     // grow-only device workspace, carved per call (stream ordered)
     void* ws = nullptr;
     size_t ws_bytes = 0;
+    // grow-only blocks for data that outlives a reservation of the workspace
+    // within one call (hd_aux_reserve)
+    void* aux[2] = {nullptr, nullptr};
+    size_t aux_bytes[2] = {0, 0};
     // pinned host words for polling device counters
     int* h_poll = nullptr;
     // grow-only pinned staging block (hd_host_stage)
@@ -151,6 +155,11 @@ bool hd_is_device_ptr(const void* p);
 // Workspace: returns a device pointer of at least `bytes`, 256-aligned,
 // valid until the next hd_ws_reserve on the same context.
 int hd_ws_reserve(hd_ctx* ctx, size_t bytes, void** out);
+// Auxiliary block `which` (0 or 1) of at least `bytes`, 256-aligned, valid until the
+// next hd_aux_reserve of the same block.
+int hd_aux_reserve(hd_ctx* ctx, int which, size_t bytes, void** out);
+// Gives an auxiliary block larger than `most` bytes back (nothing may be using it).
+void hd_aux_trim(hd_ctx* ctx, int which, size_t most);
 // Pinned host block of at least `bytes`, valid until the next hd_host_stage on the
 // same context; the caller leaves no copy in flight from or to it.
 int hd_host_stage(hd_ctx* ctx, size_t bytes, void** out);

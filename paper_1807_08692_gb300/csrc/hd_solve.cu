@@ -599,72 +599,210 @@ __global__ void __launch_bounds__(128, 6) k_resid(const int32_t* __restrict__ rp
     }
 }
 
-// Per-column operators (truncated systems): column j's row t holds the entries
-// off[j * n + t] .. off[j * n + t + 1] of (ci, wv); columns j >= B are empty.
-// Q = c1 P - c2 W_j P column by column.
-template <int S>
-__global__ void __launch_bounds__(256) k_spmm_cols(const int64_t* __restrict__ off, const int32_t* __restrict__ ci,
-                                                   const float* __restrict__ wv, int32_t B, const float* __restrict__ P,
-                                                   float* __restrict__ Q, int64_t n, int32_t ld, float c1, float c2,
-                                                   const ColState* __restrict__ st) {
-    constexpr int L = S / 4;
-    constexpr int RPB = 256 / L;
-    if (!slab_has_work<S>(st)) return;
-    const int g = (threadIdx.x & 31) % L;
-    const int col = blockIdx.y * S + 4 * g;
-    for (int64_t row = (int64_t)blockIdx.x * RPB + threadIdx.x / L; row < n; row += (int64_t)gridDim.x * RPB) {
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
+// ---- per-column operators (truncated systems)
+// Column j's row t holds the entries off[j * n + t] .. off[j * n + t + 1] of (ci,
+// wv); columns j >= B are empty.  The vectors are read column by column (VT, the
+// transposed block), so a column's gathers stay in its own n floats.
+//
+// Bound: one 4-byte gather per entry through L1 (110M entries: 0.38 ms at a line
+// per cycle).  One block per SM takes an equal share of the rows of all columns
+// in column order, so its L1 keeps to one or two columns' vectors.  It streams
+// the entries in order: coalesced (index, weight) loads two tiles ahead, the
+// gathers they name one tile ahead, (weight, value) pairs in shared memory; a
+// thread then sums its own rows from there, so the order of a row's sum does
+// not depend on the tiling.  64 systems of 75,000 rows, 110M entries: 0.55 ms;
+// with tiles of 2,048 entries, in which only three warps' rows are summed at a
+// time, 0.90 ms, of 8,192 (64 KB less L1) 0.64 ms; a thread per (row, 4 columns)
+// walking four rows in global memory and gathering 4 bytes of a 256-byte row
+// took 1.65 ms.
+constexpr int TC_T = 1024;           // threads
+constexpr int TC_E = 4;              // entries per thread and tile
+constexpr int TC_TILE = TC_T * TC_E;
+constexpr int TC_COLS = 4096;        // columns at most (hd_temporal_truncated)
+
+// VT[j][i] = V[i][j]; grid (rows / 32, columns / 32), 32 x 8 threads
+__global__ void __launch_bounds__(256) k_transpose(const float* __restrict__ V, int64_t n, int32_t ld,
+                                                   float* __restrict__ VT) {
+    __shared__ float t[32][33];
+    const int64_t r0 = blockIdx.x * 32ll;
+    const int c0 = blockIdx.y * 32;
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int j = col + c;
-            if (j >= B) continue;
-            const int64_t f = (int64_t)j * n + row;
-            const int64_t b = __ldg(off + f), e = __ldg(off + f + 1);
-            float s0 = 0.f, s1 = 0.f;
-            int64_t t = b;
-            for (; t + 2 <= e; t += 2) {
-                s0 = fmaf(__ldg(wv + t), __ldg(P + (int64_t)__ldg(ci + t) * ld + j), s0);
-                s1 = fmaf(__ldg(wv + t + 1), __ldg(P + (int64_t)__ldg(ci + t + 1) * ld + j), s1);
-            }
-            if (t < e) s0 = fmaf(__ldg(wv + t), __ldg(P + (int64_t)__ldg(ci + t) * ld + j), s0);
-            s[c] = s0 + s1;
+    for (int u = 0; u < 32; u += 8)
+        if (r0 + y + u < n && c0 + x < ld) t[y + u][x] = V[(r0 + y + u) * ld + c0 + x];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 32; u += 8)
+        if (c0 + y + u < ld && r0 + x < n) VT[(int64_t)(c0 + y + u) * n + r0 + x] = t[x][y + u];
+}
+
+// The columns to work on, in order (whole quads, as in the update that reads Q);
+// st == nullptr: all.  Block-wide; returns their number.
+__device__ __forceinline__ int trunc_columns(const ColState* st, int32_t ld, uint16_t* list) {
+    __shared__ int warp_count[TC_T / 32];
+    __shared__ int have;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) have = 0;
+    for (int c0 = 0; c0 < ld; c0 += TC_T) {
+        const int j = c0 + (int)threadIdx.x;
+        bool on = j < ld;
+        if (on && st) {
+            const ColState* q = st + (j & ~3);
+            on = q[0].active | q[1].active | q[2].active | q[3].active;
         }
-        const float4 own = ld4(P + row * ld + col);
-        float4 q;
-        q.x = c1 * own.x - c2 * s[0];
-        q.y = c1 * own.y - c2 * s[1];
-        q.z = c1 * own.z - c2 * s[2];
-        q.w = c1 * own.w - c2 * s[3];
-        st4(Q + row * ld + col, q);
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        if (lane == 0) warp_count[warp] = __popc(m);
+        __syncthreads();
+        int at = have;
+        for (int w = 0; w < warp; ++w) at += warp_count[w];
+        if (on) list[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
+        __syncthreads();
+        if (threadIdx.x == TC_T - 1) have = at + __popc(m);
+        __syncthreads();
+    }
+    return have;
+}
+
+// Streams the rows lo .. hi of one column (off, ci, wv: its CSR; v: its vector):
+// add(k, w, x) for a row's entries in order, k with the parity of the entry's
+// place, then done(row).
+template <class RS, class AD, class DN>
+__device__ __forceinline__ void trunc_rows(const int64_t* __restrict__ off, const int32_t* __restrict__ ci,
+                                           const float* __restrict__ wv, const float* __restrict__ v, int64_t lo,
+                                           int64_t hi, bool empty, float2 (*tile)[TC_TILE], RS reset, AD add, DN done) {
+    int64_t row = lo + threadIdx.x;
+    reset();
+    if (empty) {
+        for (; row < hi; row += TC_T) done(row);
+        return;
+    }
+    const int64_t first = __ldg(off + lo), last = __ldg(off + hi);
+    int64_t b = last, e = last, nb = last, ne = last;
+    auto bounds = [&](int64_t r, int64_t& x, int64_t& y) {
+        if (r < hi) {
+            x = __ldg(off + r);
+            y = __ldg(off + r + 1);
+        }
+    };
+    bounds(row, b, e);
+    bounds(row + TC_T, nb, ne);
+    int32_t c[TC_E];
+    float w[TC_E], x[TC_E], wn[TC_E];
+    auto indices = [&](int64_t t0) {
+#pragma unroll
+        for (int u = 0; u < TC_E; ++u) {
+            const int64_t q = t0 + u * TC_T + threadIdx.x;
+            c[u] = 0;
+            wn[u] = 0.f;
+            if (q < last) {
+                c[u] = __ldg(ci + q);
+                wn[u] = __ldg(wv + q);
+            }
+        }
+    };
+    auto gather = [&]() {
+#pragma unroll
+        for (int u = 0; u < TC_E; ++u) {
+            x[u] = __ldg(v + c[u]);
+            w[u] = wn[u];
+        }
+    };
+    indices(first);
+    gather();
+    indices(first + TC_TILE);
+    int buf = 0;
+    for (int64_t t0 = first; t0 < last; t0 += TC_TILE, buf ^= 1) {
+#pragma unroll
+        for (int u = 0; u < TC_E; ++u) tile[buf][u * TC_T + threadIdx.x] = make_float2(w[u], x[u]);
+        gather();                      // tile t0 + TC_TILE
+        indices(t0 + 2 * TC_TILE);
+        __syncthreads();  // this tile is complete, and every thread is done with the other buffer's last one
+        const int64_t t1 = min(last, t0 + TC_TILE);
+        while (row < hi && b < t1) {
+            // the row's part of this tile, four reads ahead of their sums
+            int q = (int)(max(b, t0) - t0);
+            const int g = (int)(min(e, t1) - t0);
+            if ((q + t0 - b) & 1) {
+                const float2 z = tile[buf][q++];
+                add(1, z.x, z.y);
+            }
+            for (; q + 4 <= g; q += 4) {
+                float2 z[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) z[u] = tile[buf][q + u];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) add(u, z[u].x, z[u].y);
+            }
+            for (int u = 0; q < g; ++q, ++u) {
+                const float2 z = tile[buf][q];
+                add(u, z.x, z.y);
+            }
+            if (e > t1) break;
+            done(row);
+            reset();
+            row += TC_T;
+            b = nb;
+            e = ne;
+            bounds(row + TC_T, nb, ne);
+        }
+    }
+    for (; row < hi; row += TC_T) {  // rows without entries after the last one
+        done(row);
+        reset();
+    }
+    __syncthreads();
+}
+
+// A block's share of the rows of `count` columns
+template <class F>
+__device__ __forceinline__ void trunc_share(int count, int64_t n, F each) {
+    const int64_t total = count * n, per = (total + gridDim.x - 1) / gridDim.x;
+    const int64_t g1 = min(total, (blockIdx.x + 1) * per);
+    for (int64_t g = blockIdx.x * per; g < g1;) {
+        const int k = (int)(g / n);
+        const int64_t lo = g - k * n, hi = min(n, lo + (g1 - g));
+        each(k, lo, hi);
+        g += hi - lo;
     }
 }
 
-// Q = -(c1 X - c2 W_j X) column by column (truncated systems), W_j X in two words.
-template <int S>
-__global__ void __launch_bounds__(256) k_resid_cols(const int64_t* __restrict__ off, const int32_t* __restrict__ ci,
-                                                    const float* __restrict__ wv, int32_t B, const float* __restrict__ X,
-                                                    float* __restrict__ Q, int64_t n, int32_t ld, float c1, float c2) {
-    constexpr int L = S / 4;
-    constexpr int RPB = 256 / L;
-    const int g = (threadIdx.x & 31) % L;
-    const int col = blockIdx.y * S + 4 * g;
-    for (int64_t row = (int64_t)blockIdx.x * RPB + threadIdx.x / L; row < n; row += (int64_t)gridDim.x * RPB) {
-        const float4 own = ld4(X + row * ld + col);
-        const float ox[4] = {own.x, own.y, own.z, own.w};
-        float q[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int j = col + c;
-            float hi = 0.f, lo = 0.f;
-            if (j < B) {
-                const int64_t f = (int64_t)j * n + row;
-                const int64_t b = __ldg(off + f), e = __ldg(off + f + 1);
-                for (int64_t t = b; t < e; ++t) df_fma(hi, lo, __ldg(wv + t), __ldg(X + (int64_t)__ldg(ci + t) * ld + j));
-            }
-            q[c] = neg_operator(c1, ox[c], c2, hi, lo);
-        }
-        st4(Q + row * ld + col, make_float4(q[0], q[1], q[2], q[3]));
-    }
+// Q = c1 P - c2 W_j P column by column (VT: the transposed P); even and odd
+// entries of a row sum separately.
+__global__ void __launch_bounds__(TC_T, 1)
+    k_spmm_cols(const int64_t* __restrict__ off, const int32_t* __restrict__ ci, const float* __restrict__ wv, int32_t B,
+                const float* __restrict__ VT, float* __restrict__ Q, int64_t n, int32_t ld, float c1, float c2,
+                const ColState* __restrict__ st) {
+    extern __shared__ float2 tc_sm[];
+    float2(*tile)[TC_TILE] = reinterpret_cast<float2(*)[TC_TILE]>(tc_sm);  // [2]
+    __shared__ uint16_t list[TC_COLS];
+    trunc_share(trunc_columns(st, ld, list), n, [&](int k, int64_t lo, int64_t hi) {
+        const int j = list[k];
+        const float* v = VT + (int64_t)j * n;
+        float s0, s1;
+        trunc_rows(
+            off + (int64_t)j * n, ci, wv, v, lo, hi, j >= B, tile, [&] { s0 = s1 = 0.f; },
+            [&](int i, float w, float p) {
+                if (i & 1) s1 = fmaf(w, p, s1);
+                else s0 = fmaf(w, p, s0);
+            },
+            [&](int64_t row) { Q[row * ld + j] = c1 * v[row] - c2 * (s0 + s1); });
+    });
+}
+
+// Q = -(c1 X - c2 W_j X) column by column, W_j X in two words (VT: the transposed X).
+__global__ void __launch_bounds__(TC_T, 1)
+    k_resid_cols(const int64_t* __restrict__ off, const int32_t* __restrict__ ci, const float* __restrict__ wv, int32_t B,
+                 const float* __restrict__ VT, float* __restrict__ Q, int64_t n, int32_t ld, float c1, float c2) {
+    extern __shared__ float2 tc_sm[];
+    float2(*tile)[TC_TILE] = reinterpret_cast<float2(*)[TC_TILE]>(tc_sm);  // [2]
+    trunc_share(ld, n, [&](int j, int64_t lo, int64_t hi) {
+        const float* v = VT + (int64_t)j * n;
+        float a, b;
+        trunc_rows(
+            off + (int64_t)j * n, ci, wv, v, lo, hi, j >= B, tile, [&] { a = b = 0.f; },
+            [&](int, float w, float p) { df_fma(a, b, w, p); },
+            [&](int64_t row) { Q[row * ld + j] = neg_operator(c1, v[row], c2, a, b); });
+    });
 }
 
 // *out = the largest row length (entries) of the CSR graph
@@ -2028,6 +2166,30 @@ static int launch_fin_rr(Engine& S_, const double* C, const double* coef, int r)
     return HD_OK;
 }
 
+// Truncated systems: Q = c1 V - c2 W_j V of the columns being iterated, or with
+// `resid` Q = -(c1 V - c2 W_j V) of every column in two words.
+static int launch_trunc(Engine& E, const float* V, float c1, float c2, bool resid) {
+    hd_ctx* ctx = E.ctx;
+    const TruncSys& ts = *E.ts;
+    HD_PROF(ctx, resid ? "resid" : "spmm");
+    k_transpose<<<dim3((unsigned)ceil_div(E.n, 32), (unsigned)ceil_div(E.Bp, 32)), 256, 0, ctx->stream>>>(V, E.n, E.Bp,
+                                                                                                        E.VT);
+    HD_CHECK_LAUNCH(ctx);
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms, E.n * E.Bp / TC_T));
+    constexpr int smem = 2 * TC_TILE * (int)sizeof(float2);
+    static uint64_t attr = 0;
+    if (hd_first_on_device(attr, ctx->device)) {
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_spmm_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_resid_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    }
+    if (resid)
+        k_resid_cols<<<grid, TC_T, smem, ctx->stream>>>(ts.off, ts.ci, ts.wv, ts.B, E.VT, E.Q, E.n, E.Bp, c1, c2);
+    else
+        k_spmm_cols<<<grid, TC_T, smem, ctx->stream>>>(ts.off, ts.ci, ts.wv, ts.B, E.VT, E.Q, E.n, E.Bp, c1, c2, E.st);
+    HD_CHECK_LAUNCH(ctx);
+    return HD_OK;
+}
+
 // One CG iteration of every column (Eq. 20 operator, CG update, direction).
 // `after_update`, if given, runs right after the X/R update (the serving loop
 // scatters newly admitted observations there).
@@ -2061,12 +2223,10 @@ int engine_iteration(Engine& S_, int (*after_update)(void*), void* arg) {
             HD_CHECK_LAUNCH(ctx);
         }
     } else {
-        if (S_.ts)
-        {
-            LAUNCH_VEC(k_spmm_cols, S_.ts->off, S_.ts->ci, S_.ts->wv, S_.ts->B, S_.P, S_.Q, n, Bp, c1, c2, S_.st);
+        if (S_.ts) {
+            if ((rc = launch_trunc(S_, S_.P, c1, c2, false))) return rc;
             if ((rc = launch_dot(S_, S_.part, S_.st))) return rc;
-        }
-        else if ((rc = launch_spmm(S_, c1, c2, S_.part, S_.st)))
+        } else if ((rc = launch_spmm(S_, c1, c2, S_.part, S_.st)))
             return rc;
         if (lr_on) {
             if ((rc = lr_expand(ctx, S_.lr, EXP_ADD_Q, S_.Q, nullptr, nullptr, n, Bp, S_.st, S_.num_active)))
@@ -2110,7 +2270,7 @@ static std::vector<uint64_t> iteration_key(const Engine& E) {
             (uint64_t)E.g->col, (uint64_t)E.g->val, (uint64_t)E.n, (uint64_t)E.lr.e,
             (uint64_t)(E.has_lr ? E.lr.e->U : nullptr), (uint64_t)(E.has_lr ? E.lr.e->storage : -1),
             (uint64_t)(E.has_lr ? E.lr.e->sp_rp : nullptr), (uint64_t)(E.has_lr ? E.lr.e->sp_cp : nullptr),
-            (uint64_t)E.R, (uint64_t)E.P, (uint64_t)E.Q, (uint64_t)E.X, (uint64_t)E.part, (uint64_t)E.st,
+            (uint64_t)E.R, (uint64_t)E.P, (uint64_t)E.Q, (uint64_t)E.X, (uint64_t)E.VT, (uint64_t)E.part, (uint64_t)E.st,
             (uint64_t)E.num_active, (uint64_t)E.lr.part, (uint64_t)E.lr.C, (uint64_t)E.lr.H, (uint64_t)E.lr.Hhi,
             (uint64_t)E.lr.Hlo, (uint64_t)E.dcoef, (uint64_t)E.opcoef, (uint64_t)E.segK, (uint64_t)E.seg,
             (uint64_t)E.nch, (uint64_t)E.Bp, (uint64_t)E.slab, (uint64_t)E.vl.S, (uint64_t)E.vl.nblk, (uint64_t)E.vl.slabs,
@@ -2240,12 +2400,8 @@ static int true_residual(Engine& E, double alpha) {
     const float c1 = (float)c1d, c2 = (float)c2d;
     int rc;
     if (E.ts) {
-        const dim3 grid(E.vl.nblk, E.vl.slabs);
         // Q = -L_a(W_j) x column by column (truncated systems), in two words
-        HD_PROF(ctx, "resid");
-        HD_DISPATCH_S(E.vl.S, (k_resid_cols<SS><<<grid, 256, 0, ctx->stream>>>(E.ts->off, E.ts->ci, E.ts->wv, E.ts->B,
-                                                                                E.X, E.Q, n, Bp, c1, c2)));
-        HD_CHECK_LAUNCH(ctx);
+        if ((rc = launch_trunc(E, E.X, c1, c2, true))) return rc;
     } else {
         // Q = -L_a(W) x: the fp32 SpMM when its rounding bound is small against
         // every column's tolerance, else the two-word kernel (k_resid_pick)
@@ -2393,6 +2549,7 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
                  ws_size((size_t)rpad * Bp * 4) + 2 * ws_size((size_t)Bp16 * rpad * 2) + 6 * ws_size(rpad * 8);
     // the fp16 gather copy of P: graph solves with 8 <= Bp <= 256 columns in multiples of 8
     const bool half_ok = !ts && Bp % 8 == 0 && Bp <= 256;
+    if (ts) bytes += ws_size(vec);  // the transposed block
     if (half_ok) bytes += ws_size((size_t)n * Bp * 2) + ws_size((size_t)Bp * 4);
     void* ws;
     int rc = hd_ws_reserve(ctx, bytes, &ws);
@@ -2402,6 +2559,7 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     S_.P = cv.take<float>((size_t)n * Bp);
     S_.Q = cv.take<float>((size_t)n * Bp);
     S_.X = x_direct ? X : cv.take<float>((size_t)n * Bp);
+    if (ts) S_.VT = cv.take<float>((size_t)n * Bp);
     S_.part = cv.take<float2>((size_t)S_.nch * Bp);
     S_.st = cv.take<ColState>(Bp);
     S_.num_active = cv.take<int>(16);

@@ -139,6 +139,7 @@ struct Engine {
     // k_spmm's; the server keeps one order at every lane width)
     bool narrow4 = true;
     float *R = nullptr, *P = nullptr, *Q = nullptr, *X = nullptr;
+    float* VT = nullptr;        // truncated systems: the transposed operand of their products [Bp][n]
     float2* part = nullptr;
     ColState* st = nullptr;
     int* num_active = nullptr;
