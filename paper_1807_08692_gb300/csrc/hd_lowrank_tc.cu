@@ -69,16 +69,6 @@ bool lr_use_tensor_cores(const hd_eig* e) {
            !off;
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t* r = reinterpret_cast<uint32_t*>(v);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
-
 template <uint32_t NC>
 __device__ __forceinline__ void tmem_alloc_dyn(uint32_t* slot, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(slot)),
@@ -336,7 +326,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                 for (int u = 0; u < 2; ++u) {
                     if (c0 + u >= ce) break;
                     float v[16];
-                    tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + ab * a.Nc + (c0 + u) * 16, v);
+                    tc::tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + ab * a.Nc + (c0 + u) * 16, v);
                     tc::tmem_ld_wait();
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
@@ -686,11 +676,11 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
             for (int c = cb; c < ce; ++c) {
                 float v[16];
                 if (have) {
-                    tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + m * a.Nc + c * 16, v);
+                    tc::tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + m * a.Nc + c * 16, v);
                     tc::tmem_ld_wait();
                     if (a.fold) {
                         float v2[16];
-                        tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (m + a.fold) * a.Nc + c * 16, v2);
+                        tc::tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (m + a.fold) * a.Nc + c * 16, v2);
                         tc::tmem_ld_wait();
 #pragma unroll
                         for (int q = 0; q < 16; ++q) v[q] += v2[q];
