@@ -117,6 +117,27 @@ __device__ __forceinline__ float knn_flush(uint64_t* list, const uint64_t* buf, 
     return key_sim(kth);
 }
 
+// The same for at most 32 candidates held as (similarity bits, id) pairs.
+__device__ __forceinline__ float knn_flush32(uint64_t* list, const uint64_t* buf, int cnt, int k, int lane) {
+    uint64_t a0 = list[lane], a1 = list[lane + 32];
+    uint64_t b = 0ull;
+    if (lane < cnt) {
+        const uint64_t raw = buf[lane];
+        b = knn_key(__uint_as_float((uint32_t)raw), (int64_t)(raw >> 32));
+    }
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+        for (int st = size >> 1; st > 0; st >>= 1) b = key_exchange(b, st, (size == 32 || !(lane & size)) == !(lane & st));
+    // the list's lower half against the candidates, smallest first: bitonic again
+    const uint64_t r = __shfl_xor_sync(0xffffffffu, b, 31);
+    a1 = a1 > r ? a1 : r;
+    merge64(a0, a1, lane);
+    list[lane] = a0;
+    list[lane + 32] = a1;
+    return key_sim(__shfl_sync(0xffffffffu, k > 32 ? a1 : a0, (k - 1) & 31));
+}
+
 // The k best of a query's per-segment lists: one block per query, each warp
 // merges every eighth segment, warp 0 the eight results.
 __global__ void __launch_bounds__(256) k_knn_merge(const uint64_t* __restrict__ part, int nseg, int64_t nq, int k,
@@ -155,16 +176,20 @@ struct KnnArgs {
     int d, k, excl;
     int nwork;         // query blocks
     int nseg, tps;     // database segments and tiles per segment
-    uint64_t* lists;   // [gridDim.x][rows of a query block][64] running lists
+    uint64_t* lists;   // running lists of 64: [gridDim.x][rows of a query block], twice for the bf16 kernel
     uint64_t* part;    // [nseg][nq][k] per-segment results (nseg > 1)
     int32_t* idx_out;  // [nq][k] (nseg == 1)
     float* sim_out;
 };
 
-// the final list of a row: the result itself, or the segment's part of it
-__device__ __forceinline__ void knn_store(const KnnArgs& a, int seg, int64_t row, const uint64_t* list, int lane) {
-    for (int c = lane; c < a.k; c += 32) {
-        const uint64_t key = list[c];
+// the final list of a row (entries lane and lane + 32 of each lane): the result
+// itself, or the segment's part of it
+__device__ __forceinline__ void knn_store(const KnnArgs& a, int seg, int64_t row, uint64_t x0, uint64_t x1, int lane) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c = lane + 32 * h;
+        const uint64_t key = h ? x1 : x0;
+        if (c >= a.k) continue;
         if (a.nseg > 1) {
             a.part[((int64_t)seg * a.nq + row) * a.k + c] = key;
         } else {
@@ -364,7 +389,7 @@ __global__ void __launch_bounds__(256, 2)
         for (int r = warp; r < BM; r += 8) {
             if (q0 + r >= a.nq) break;
             if (cnt[r] > 0) knn_flush(lists + r * 64, bufs + r * KBUF_LD, cnt[r], a.k, lane);
-            knn_store(a, seg, q0 + r, lists + r * 64, lane);
+            knn_store(a, seg, q0 + r, lists[r * 64 + lane], lists[r * 64 + lane + 32], lane);
         }
         __syncthreads();
     }
@@ -376,22 +401,30 @@ __global__ void __launch_bounds__(256, 2)
 // Bound: the tensor cores when there are many queries, the stream of the
 // database when there are few (64 queries against 1M x 2048: 0.80 ms for the
 // whole observation, 0.60 ms at the copy bandwidth; 43.4 ms with one block per
-// query block).  Selection: one query row per epilogue thread.  A row keeps a
-// threshold (its k-th best so far, from the last merge) and appends what beats
-// it to 64 slots of shared memory; when a row has more than 32, its warp sorts
-// them and merges them into the row's list by shuffles.  About k ln(n / k)
-// candidates per row pass the threshold, so the scan (one max over 32 columns
-// and one compare) is what runs in the steady state.  A thread inserting into
-// its row's list in global memory, as this kernel did before, took 409 ms for
-// the lists of 250,000 x 512 at k = 50.
+// query block).
+//
+// Selection: two epilogue threads per query row, each with half of a tile's
+// columns and a list of its own (merged at the end of the item).  A thread keeps
+// a threshold (its k-th best so far, from the last merge); what beats it is
+// appended to 32 slots of shared memory by predicated stores, 16 columns at a
+// time, and when a row holds more than 16 its warp sorts them and merges them
+// into the row's list by shuffles.  With one or two warps per scheduler the
+// epilogue lives off straight-line code: the lists of 250,000 x 512 at k = 50
+// take 47 ms, 34 at the tensor cores' rate; with one thread per row and a branch
+// per column it took 73 ms, bound by the epilogue at any depth, and with every
+// insertion a walk of the list in global memory 409 ms.  (Reading a chunk ahead
+// from TMEM gains nothing: 49 ms.)
 namespace knntc {
 constexpr int BM = 128, BN = 256, BK = 64, STAGES = 3;
 constexpr int A_BYTES = BM * BK * 2;   // 16 KB
 constexpr int B_BYTES = BN * BK * 2;   // 32 KB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr int BUF_BYTES = BM * KBUF_LD * 8;
+constexpr int CHUNK = 16;            // columns between two looks at the buffers
+constexpr int TBUF = 32, TBUF_LD = TBUF + 1;
+constexpr int BUF_BYTES = 2 * BM * TBUF_LD * 8;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + BUF_BYTES + 1024 + 256;
-constexpr int THREADS = 192;
+constexpr int EPI = 256;             // epilogue threads: two per query row
+constexpr int THREADS = 64 + EPI;
 }  // namespace knntc
 
 __global__ void __launch_bounds__(knntc::THREADS, 1)
@@ -400,8 +433,8 @@ __global__ void __launch_bounds__(knntc::THREADS, 1)
     using namespace knntc;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t* bufs = (uint64_t*)(smem + STAGES * STAGE_BYTES);  // [128][KBUF_LD]
-    uint64_t* full = bufs + BM * KBUF_LD;
+    uint64_t* bufs = (uint64_t*)(smem + STAGES * STAGE_BYTES);  // [2][128][TBUF_LD]
+    uint64_t* full = bufs + 2 * BM * TBUF_LD;
     uint64_t* empty = full + STAGES;
     uint64_t* acc_full = empty + STAGES;
     uint64_t* acc_empty = acc_full + 2;
@@ -421,7 +454,7 @@ __global__ void __launch_bounds__(knntc::THREADS, 1)
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&acc_full[b], 1);
-            tc::mbar_init(&acc_empty[b], 128);
+            tc::mbar_init(&acc_empty[b], EPI);
         }
         tc::mbar_init(drain, 1);
         *abort_flag = 0;
@@ -513,20 +546,20 @@ __global__ void __launch_bounds__(knntc::THREADS, 1)
             }
         }
     } else {
-        // ---------------- epilogue: warps 2..5, one query row per thread
-        const int quarter = warp & 3;
-        const int rloc = quarter * 32 + lane;
-        uint64_t* lists = a.lists + ((int64_t)blockIdx.x * BM + quarter * 32) * 64;  // this warp's 32 rows
-        uint64_t* wbuf = bufs + quarter * 32 * KBUF_LD;
-        uint64_t* buf = wbuf + lane * KBUF_LD;
+        // ---------------- epilogue: warps 2..9; the TMEM lanes (rows) of a warp are
+        // those of its quarter, its columns those of its half
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        uint64_t* lists = a.lists + (((int64_t)blockIdx.x * 2 + half) * BM + quarter * 32) * 64;  // this warp's 32 rows
+        uint64_t* wbuf = bufs + (half * BM + quarter * 32) * TBUF_LD;
+        const uint32_t slot0 = tc::smem_u32(wbuf + lane * TBUF_LD);
         uint32_t tcount = 0;
         bool ok = true;
         for (int item = blockIdx.x; item < nitem && ok; item += gridDim.x) {
             const int w = item % a.nwork, seg = item / a.nwork, t0 = seg * a.tps, t1 = min(ntile, t0 + a.tps);
-            const int64_t row = (int64_t)w * BM + rloc;
+            const int64_t row0 = (int64_t)w * BM + quarter * 32, row = row0 + lane;
             for (int c = lane; c < 32 * 64; c += 32) lists[c] = 0ull;
             float tau = row < a.nq ? -INFINITY : INFINITY;  // a row past the last query takes nothing
-            int cnt = 0;
+            uint32_t slot = slot0;
             for (int t = t0; t < t1; ++t, ++tcount) {
                 int ab = tcount & 1;
                 uint32_t aph = (tcount >> 1) & 1;
@@ -536,52 +569,78 @@ __global__ void __launch_bounds__(knntc::THREADS, 1)
                     break;
                 }
                 tc::fence_after_sync();
-                for (int c = 0; c < BN / 32; ++c) {
-                    float v[32];
-                    tc::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + ab * BN + c * 32, v);
-                    tc::tmem_ld_wait32(v);
-                    float m = v[0];
+                const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + ab * BN + half * (BN / 2);
+#pragma unroll 1
+                for (int c = 0; c < BN / 2; c += CHUNK) {
+                    float v[CHUNK];
+                    tc::tmem_ld16(acc + c, v);
+                    tc::tmem_ld_wait16(v);
+                    const int64_t base = (int64_t)t * BN + half * (BN / 2) + c;
+                    // columns past the database, and the row itself, take no part
+                    if (base + CHUNK > a.n) {
 #pragma unroll
-                    for (int i = 1; i < 32; ++i) m = fmaxf(m, v[i]);
-                    if (__any_sync(0xffffffffu, m > tau)) {
-                        const int64_t base = (int64_t)t * BN + c * 32;
+                        for (int i = 0; i < CHUNK; ++i)
+                            if (base + i >= a.n) v[i] = -INFINITY;
+                    }
+                    if (a.excl && base >> 5 == row0 >> 5) {
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            const int64_t id = base + i;
-                            if (v[i] > tau && id < a.n && !(a.excl && id == row)) buf[cnt++] = knn_key(v[i], id);
-                        }
-                        __syncwarp();
-                        unsigned need = __ballot_sync(0xffffffffu, cnt > KBUF - 32);
-                        while (need) {
-                            const int r = __ffs(need) - 1;
-                            need &= need - 1;
-                            const float th = knn_flush(lists + r * 64, wbuf + r * KBUF_LD,
-                                                       __shfl_sync(0xffffffffu, cnt, r), a.k, lane);
-                            if (lane == r) {
-                                tau = th;
-                                cnt = 0;
+                        for (int i = 0; i < CHUNK; ++i)
+                            if (base + i == row) v[i] = -INFINITY;
+                    }
+                    float m[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+                    for (int i = 4; i < CHUNK; ++i) m[i & 3] = fmaxf(m[i & 3], v[i]);
+                    if (__any_sync(0xffffffffu, fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])) > tau)) {
+#pragma unroll
+                        for (int i = 0; i < CHUNK; ++i)
+                            asm volatile(
+                                "{\n .reg .pred p;\n setp.gt.f32 p, %1, %2;\n"
+                                " @p st.shared.v2.b32 [%0], {%3, %4};\n @p add.u32 %0, %0, 8;\n}"
+                                : "+r"(slot)
+                                : "f"(v[i]), "f"(tau), "r"(__float_as_uint(v[i])), "r"((uint32_t)(base + i))
+                                : "memory");
+                        const int cnt = (int)(slot - slot0) >> 3;
+                        unsigned need = __ballot_sync(0xffffffffu, cnt > TBUF - CHUNK);
+                        if (need) {
+                            __syncwarp();
+                            while (need) {
+                                const int r = __ffs(need) - 1;
+                                need &= need - 1;
+                                const float th = knn_flush32(lists + r * 64, wbuf + r * TBUF_LD,
+                                                             __shfl_sync(0xffffffffu, cnt, r), a.k, lane);
+                                if (lane == r) {
+                                    tau = th;
+                                    slot = slot0;
+                                }
                             }
+                            __syncwarp();
                         }
-                        __syncwarp();
                     }
                 }
                 tc::fence_before_sync();
                 tc::mbar_arrive(&acc_empty[ab]);
             }
-            __syncwarp();
-            for (int r = 0; r < 32; ++r) {
-                const int64_t rrow = (int64_t)w * BM + quarter * 32 + r;
-                if (rrow >= a.nq) break;
-                const int rc = __shfl_sync(0xffffffffu, cnt, r);
-                if (rc > 0) knn_flush(lists + r * 64, wbuf + r * KBUF_LD, rc, a.k, lane);
-                __syncwarp();
-                knn_store(a, seg, rrow, lists + r * 64, lane);
+            if (!ok) {
+                *abort_flag = 1;
+                atomicExch(err, 3);
             }
             __syncwarp();
-        }
-        if (!ok) {
-            *abort_flag = 1;
-            atomicExch(err, 3);
+            const int left = (int)(slot - slot0) >> 3;
+            for (int r = 0; r < 32; ++r) {
+                const int rc = __shfl_sync(0xffffffffu, left, r);
+                if (rc > 0) knn_flush32(lists + r * 64, wbuf + r * TBUF_LD, rc, a.k, lane);
+            }
+            // the two halves of a row meet: each warp stores 16 rows of its quarter
+            asm volatile("bar.sync 1, %0;" ::"n"(EPI) : "memory");
+            const uint64_t* other = a.lists + (((int64_t)blockIdx.x * 2 + (half ^ 1)) * BM + quarter * 32) * 64;
+            for (int r = 16 * half; r < 16 * half + 16; ++r) {
+                if (row0 + r >= a.nq) break;
+                uint64_t x0 = lists[r * 64 + lane], x1 = lists[r * 64 + lane + 32];
+                take64(x0, x1, other[r * 64 + lane], other[r * 64 + lane + 32], lane);
+                knn_store(a, seg, row0 + r, x0, x1, lane);
+            }
+            asm volatile("bar.sync 1, %0;" ::"n"(EPI) : "memory");
+            ok = ok && !*abort_flag;  // an epilogue warp that gave up ends the others' loops with its own
         }
     }
     tc::fence_before_sync();
@@ -628,11 +687,15 @@ static KnnPlan knn_plan_for(const hd_ctx* ctx, int64_t n, int64_t nq, int k, int
     return knn_plan(nq, (n + knntc::BN - 1) / knntc::BN, knntc::BM, ctx->num_sms, k, 4);
 }
 
+static size_t knn_list_keys(const KnnPlan& p, int64_t nq, int dtype) {
+    return (size_t)p.grid * knn_bm(nq, dtype) * (dtype == HD_BF16 ? 2 : 1) * 64;
+}
+
 // Workspace bytes hd_knn_impl needs for a search (its `scratch`).
 static size_t knn_scratch_bytes(const hd_ctx* ctx, int64_t n, int64_t nq, int32_t k, int dtype) {
     if (k < 1 || k > KMAX || nq <= 0 || n <= 0) return 256;
     const KnnPlan p = knn_plan_for(ctx, n, nq, k, dtype);
-    return ws_size((size_t)p.grid * knn_bm(nq, dtype) * 64 * 8) + (p.nseg > 1 ? ws_size((size_t)p.nseg * nq * k * 8) : 0);
+    return ws_size(knn_list_keys(p, nq, dtype) * 8) + (p.nseg > 1 ? ws_size((size_t)p.nseg * nq * k * 8) : 0);
 }
 
 // Enqueue a search on the context's stream; `scratch` holds knn_scratch_bytes.
@@ -656,7 +719,7 @@ static int hd_knn_impl(hd_ctx* ctx, const void* Xd, int64_t n, int32_t d, int dt
     a.nseg = p.nseg;
     a.tps = p.tps;
     WsCarver cv(scratch);
-    a.lists = cv.take<uint64_t>((size_t)p.grid * knn_bm(nq, dtype) * 64);
+    a.lists = cv.take<uint64_t>(knn_list_keys(p, nq, dtype));
     a.part = p.nseg > 1 ? cv.take<uint64_t>((size_t)p.nseg * nq * k) : nullptr;
     a.idx_out = idx_d;
     a.sim_out = sim_d;
@@ -778,36 +841,17 @@ __global__ void k_fill(const int32_t* idx, const float* sim, const int8_t* recip
     }
 }
 
-__global__ void k_sort_rows2(const int32_t* rp, int32_t* col, float* val, int64_t n) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int32_t b = rp[i], e = rp[i + 1];
-    for (int32_t t = b + 1; t < e; ++t) {
-        int32_t c = col[t];
-        float v = val[t];
-        int32_t s = t - 1;
-        while (s >= b && col[s] > c) {
-            col[s + 1] = col[s];
-            val[s + 1] = val[s];
-            --s;
-        }
-        col[s + 1] = c;
-        val[s + 1] = v;
-    }
-}
-
 int hd_graph_from_lists(hd_ctx* ctx, int64_t n, int32_t k, const int32_t* idx_d, const float* sim_d, float gamma,
                         int sym, hd_graph** out) {
-    int8_t* recip;
-    float* wrev;
-    int32_t *extra, *len, *own, *cursor;
     size_t nk = (size_t)n * k;
-    HD_CUDA(ctx, cudaMalloc(&recip, nk));
-    HD_CUDA(ctx, cudaMalloc(&wrev, nk * 4));
-    HD_CUDA(ctx, cudaMalloc(&extra, n * 4));
-    HD_CUDA(ctx, cudaMalloc(&len, n * 4));
-    HD_CUDA(ctx, cudaMalloc(&own, n * 4));
-    HD_CUDA(ctx, cudaMalloc(&cursor, n * 4));
+    // temporaries: the context's second auxiliary block (the neighbour lists are in the first)
+    void* aux;
+    int rc = hd_aux_reserve(ctx, 1, ws_size(nk) + ws_size(nk * 4) + 4 * ws_size(n * 4), &aux);
+    if (rc) return rc;
+    WsCarver cv(aux);
+    int8_t* recip = cv.take<int8_t>(nk);
+    float* wrev = cv.take<float>(nk);
+    int32_t *extra = cv.take<int32_t>(n), *len = cv.take<int32_t>(n), *own = cv.take<int32_t>(n), *cursor = cv.take<int32_t>(n);
     HD_CUDA(ctx, cudaMemsetAsync(extra, 0, n * 4, ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(cursor, 0, n * 4, ctx->stream));
     k_recip<<<ceil_div(nk, 256), 256, 0, ctx->stream>>>(idx_d, sim_d, n, k, gamma, recip, wrev, extra);
@@ -825,22 +869,16 @@ int hd_graph_from_lists(hd_ctx* ctx, int64_t n, int32_t k, const int32_t* idx_d,
     h_ptr[n] = (int32_t)acc;
     if (acc >= (1ll << 31)) return hd_fail(ctx, HD_ERR_INVALID_ARG, "graph too large: nnz=%lld", (long long)acc);
     hd_graph* g;
-    int rc = hd_graph_alloc_internal(ctx, n, acc, &g);
+    rc = hd_graph_alloc_internal(ctx, n, acc, &g);
     if (rc) return rc;
     HD_CUDA(ctx, cudaMemcpyAsync(g->row_ptr, h_ptr.data(), (n + 1) * 4, cudaMemcpyHostToDevice, ctx->stream));
     k_fill<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(idx_d, sim_d, recip, wrev, g->row_ptr, own, cursor, n, k, gamma,
                                                       sym, g->col, g->val);
     HD_CHECK_LAUNCH(ctx);
-    k_sort_rows2<<<ceil_div(n, 128), 128, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, n);
-    HD_CHECK_LAUNCH(ctx);
-    rc = hd_normalize_graph(ctx, g);
-    HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    cudaFree(recip);
-    cudaFree(wrev);
-    cudaFree(extra);
-    cudaFree(len);
-    cudaFree(own);
-    cudaFree(cursor);
+    rc = hd_sort_rows(ctx, g->row_ptr, g->col, g->val, n);
+    if (!rc) rc = hd_normalize_graph(ctx, g);
+    const int rs = hd_check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "graph", __FILE__, __LINE__);
+    if (!rc) rc = rs;
     if (rc) {
         hd_graph_free_internal(g);
         return rc;
@@ -912,19 +950,22 @@ int hd_build_graph(hd_ctx* ctx, const void* X, int64_t n, int32_t d, int dtype, 
     const void* xd;
     int rc = stage_matrix(ctx, X, (size_t)n * d * es, &ox, &xd);
     if (rc) return rc;
-    int32_t* idx;
-    float* sim;
-    HD_CUDA(ctx, cudaMalloc(&idx, (size_t)n * k * 4));
-    HD_CUDA(ctx, cudaMalloc(&sim, (size_t)n * k * 4));
-    void* ws;
-    rc = hd_ws_reserve(ctx, knn_scratch_bytes(ctx, n, n, k, dtype), &ws);
+    int32_t* idx = nullptr;
+    float* sim = nullptr;
+    void *ws, *aux;
+    rc = k > KMAX ? hd_fail(ctx, HD_ERR_INVALID_ARG, "k=%d outside [1, %d]", k, KMAX)
+                  : hd_aux_reserve(ctx, 0, 2 * ws_size((size_t)n * k * 4), &aux);
+    if (!rc) {
+        idx = (int32_t*)aux;
+        sim = (float*)((char*)aux + ws_size((size_t)n * k * 4));
+        rc = hd_ws_reserve(ctx, knn_scratch_bytes(ctx, n, n, k, dtype), &ws);
+    }
     if (!rc) rc = hd_knn_impl(ctx, xd, n, d, dtype, xd, n, k, 1, idx, sim, ws);
     if (!rc) rc = hd_check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "k-NN search", __FILE__, __LINE__);
     if (!rc) rc = hd_knn_status(ctx);
     if (!rc) rc = hd_graph_from_lists(ctx, n, k, idx, sim, gamma, sym, out);
     cudaStreamSynchronize(ctx->stream);
-    cudaFree(idx);
-    cudaFree(sim);
+    for (int b = 0; b < 2; ++b) hd_aux_trim(ctx, b, (size_t)4 << 30);
     if (ox) cudaFree(ox);
     return rc;
 }

@@ -93,3 +93,28 @@ def test_observe_matches_oracle(gpu_ctx, cfg1_data):
     assert np.array_equal(yp, cfg1_data["yp"])
     assert np.array_equal(yi, cfg1_data["yi"])
     assert np.allclose(yv, cfg1_data["yv"], rtol=2e-5)
+
+
+@pytest.mark.parametrize("lengths", [[0, 1, 2, 31, 32, 33, 63, 64, 65, 96, 129], [511, 512, 513, 700], [0, 0, 1]])
+def test_rows_are_sorted_by_column(gpu_ctx, lengths):
+    # rows around the sort's lane and buffer sizes, in descending, random and
+    # ascending order, with repeated columns (which keep their given order)
+    import paper_1807_08692_gb300 as hd
+    rng = np.random.default_rng(len(lengths))
+    n = 1000
+    rows = []
+    for L in lengths:
+        c = np.sort(rng.choice(n, L, replace=L > 600)).astype(np.int32)
+        rows += [c[::-1].copy(), rng.permutation(c), c]
+        if L > 2:
+            rows.append(np.repeat(c[: L // 2 + 1], 2)[:L].astype(np.int32)[::-1].copy())
+    rows += [np.zeros(0, np.int32)] * (n - len(rows))
+    rp = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+    col = np.concatenate(rows).astype(np.int32)
+    val = np.arange(1, col.size + 1, dtype=np.float32)
+    grp, gcol, gval, _ = hd.graph_from_csr(gpu_ctx, rp, col, val, normalized=True).export()
+    assert np.array_equal(grp, rp)
+    for i in range(len(rows)):
+        order = np.argsort(col[rp[i]:rp[i + 1]], kind="stable")
+        assert np.array_equal(gcol[rp[i]:rp[i + 1]], col[rp[i]:rp[i + 1]][order]), i
+        assert np.array_equal(gval[rp[i]:rp[i + 1]], val[rp[i]:rp[i + 1]][order]), i
