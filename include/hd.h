@@ -264,8 +264,8 @@ int hd_eig_expand(hd_ctx* ctx, const hd_eig* e, const double* H, int32_t B, floa
  *             X[t][j] is the score of sl_idx[sl_ptr[j] + t]; rows t >= s_j
  *             are 0.
  *  tol, max_iter, iters, relres, status : as for hd_query_batch.
- * Temporary device memory of about B n 4 bytes (the position maps) plus the B
- * subsystems is allocated for the call.  Errors: HD_ERR_INVALID_ARG for a bad
+ * The position maps (about B n 8 bytes) and the B subsystems take two device
+ * blocks that the context keeps for the next call (up to 4 GiB each).  Errors: HD_ERR_INVALID_ARG for a bad
  * or duplicated shortlist id or observation index, HD_ERR_OOM. */
 int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, const int32_t* sl_ptr,
                           const int32_t* sl_idx, const int32_t* y_ptr, const int32_t* y_idx,

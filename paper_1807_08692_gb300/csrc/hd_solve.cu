@@ -20,6 +20,7 @@
 #include <climits>
 #include <cmath>
 #include <cstdio>
+#include <cstring>
 #include <vector>
 
 #include <cuda_fp16.h>
@@ -41,10 +42,10 @@ __device__ __forceinline__ void st4s(float* p, float4 v) { __stcs(reinterpret_ca
 // in another order is left to one thread.
 constexpr int SCATTER_SEARCH = 1024;
 __global__ void __launch_bounds__(128) k_scatter_y(const int32_t* y_ptr, const int32_t* y_idx, const float* y_val,
-                                                   int64_t n, int32_t ld, float* R, int* err) {
+                                                   int32_t nnz, int64_t n, int32_t ld, float* R, int* err) {
     const int j = blockIdx.x;
     const int32_t b = y_ptr[j], e = y_ptr[j + 1];
-    if (b > e || b < 0) {
+    if (b > e || b < 0 || e > nnz) {  // nnz = y_ptr[B], the entries there are
         if (threadIdx.x == 0) atomicExch(err, 1);
         return;
     }
@@ -2349,6 +2350,8 @@ extern "C" int hd_query_batch(hd_ctx* ctx, const hd_graph* g, const hd_eig* eig,
                          relres, status);
 }
 
+static const char* const BAD_OBSERVATION = "bad observation: index out of range, non-finite value or bad y_ptr";
+
 // Iterate until no column is active: runs of iterations (CUDA graphs when
 // enabled), each followed by a poll of the active count and of the
 // tensor-core kernels' wait flags.  The first run is as long as the previous
@@ -2379,11 +2382,12 @@ static int iterate_until_stopped(Engine& E, int& ran) {
         }
         ran += todo;
         ++run;
-        HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll, E.num_active, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+        HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll, E.num_active, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
         HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll + 8, ctx->d_flags + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost,
                                      ctx->stream));
         HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         active = ctx->h_poll[0];
+        if (ctx->h_poll[1]) return hd_fail(ctx, HD_ERR_INVALID_ARG, "%s", BAD_OBSERVATION);
         if (ctx->h_poll[8] || ctx->h_poll[9]) return lr_tc_check_flags(ctx);
     }
     return HD_OK;
@@ -2442,7 +2446,7 @@ static int true_residual(Engine& E, double alpha) {
             if ((rc = lr_expand(ctx, E.lr, EXP_SUB_R, E.Q, nullptr, nullptr, n, Bp, nullptr))) return rc;
         }
     }
-    k_scatter_y<<<E.B, 128, 0, ctx->stream>>>(E.yp, E.yi, E.yv, n, Bp, E.Q, E.err);
+    k_scatter_y<<<E.B, 128, 0, ctx->stream>>>(E.yp, E.yi, E.yv, E.nnz_y, n, Bp, E.Q, E.err);
     HD_CHECK_LAUNCH(ctx);
     return launch_colsq(E, E.Q);
 }
@@ -2542,15 +2546,27 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
 
     size_t vec = (size_t)n * Bp * sizeof(float);
     size_t bytes = 3 * ws_size(vec) + (x_direct ? 0 : ws_size(vec)) + ws_size((size_t)S_.nch * Bp * sizeof(float2)) +
-                   ws_size(Bp * sizeof(ColState)) + ws_size(64) + ws_size((B + 1) * 4) + 2 * ws_size(nnz_y * 4 + 4) +
-                   ws_size(B * 4);
+                   ws_size(Bp * sizeof(ColState));
+    // what the host sends in one copy: the observations and tolerances that are
+    // in host memory, then the six coefficient vectors
+    const void* host_in[4] = {y_ptr, y_idx, y_val, tol};
+    const size_t host_len[4] = {(size_t)(B + 1) * 4, (size_t)nnz_y * 4, (size_t)nnz_y * 4, (size_t)B * 4};
+    size_t host_at[5] = {0, 0, 0, 0, 0};
+    for (int k = 0; k < 4; ++k) {
+        if (host_len[k] && hd_is_device_ptr(host_in[k])) host_in[k] = nullptr;  // used where it is
+        host_at[k + 1] = host_at[k] + (host_in[k] ? ws_size(host_len[k]) : 0);
+    }
+    const size_t in_bytes = host_at[4] + 6 * (size_t)rpad * 8;
+    // what starts at zero: the counters, max |P_j|, the split H
+    const size_t zero_bytes = ws_size(64) + ws_size((size_t)Bp * 4) + (lr_on ? 2 * ws_size((size_t)Bp16 * rpad * 2) : 0);
+    bytes += ws_size(in_bytes) + zero_bytes;
     if (lr_on)
         bytes += ws_size((size_t)nchunk * rpad * Bp * 4) + 2 * ws_size((size_t)rpad * Bp * 8) +
-                 ws_size((size_t)rpad * Bp * 4) + 2 * ws_size((size_t)Bp16 * rpad * 2) + 6 * ws_size(rpad * 8);
+                 ws_size((size_t)rpad * Bp * 4);
     // the fp16 gather copy of P: graph solves with 8 <= Bp <= 256 columns in multiples of 8
     const bool half_ok = !ts && Bp % 8 == 0 && Bp <= 256;
     if (ts) bytes += ws_size(vec);  // the transposed block
-    if (half_ok) bytes += ws_size((size_t)n * Bp * 2) + ws_size((size_t)Bp * 4);
+    if (half_ok) bytes += ws_size((size_t)n * Bp * 2);
     void* ws;
     int rc = hd_ws_reserve(ctx, bytes, &ws);
     if (rc) return rc;
@@ -2562,22 +2578,27 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     if (ts) S_.VT = cv.take<float>((size_t)n * Bp);
     S_.part = cv.take<float2>((size_t)S_.nch * Bp);
     S_.st = cv.take<ColState>(Bp);
-    S_.num_active = cv.take<int>(16);
+    char* zero = cv.take<char>(zero_bytes);
+    WsCarver zv(zero);
+    S_.num_active = zv.take<int>(16);
     S_.err = S_.num_active + 1;
-    int32_t* d_yptr = cv.take<int32_t>(B + 1);
-    int32_t* d_yidx = cv.take<int32_t>(nnz_y + 1);
-    float* d_yval = cv.take<float>(nnz_y + 1);
-    float* d_tol = cv.take<float>(B);
-    const void *yp, *yi, *yv, *tl;
-    if ((rc = hd_stage_in(ctx, y_ptr, (B + 1) * 4, d_yptr, &yp))) return rc;
-    if ((rc = hd_stage_in(ctx, y_idx, (size_t)nnz_y * 4, d_yidx, &yi))) return rc;
-    if ((rc = hd_stage_in(ctx, y_val, (size_t)nnz_y * 4, d_yval, &yv))) return rc;
-    if ((rc = hd_stage_in(ctx, tol, (size_t)B * 4, d_tol, &tl))) return rc;
+    unsigned* p16_max = zv.take<unsigned>(Bp);
+    HD_CUDA(ctx, cudaMemsetAsync(zero, 0, zero_bytes, ctx->stream));
+    char* d_in = cv.take<char>(in_bytes);
+    char* hs;  // pinned: the inputs now, the columns' states after the confirmation
+    if ((rc = hd_host_stage(ctx, std::max(in_bytes, B * sizeof(ColState)), (void**)&hs))) return rc;
+    const void* dev_in[4] = {y_ptr, y_idx, y_val, tol};
+    for (int k = 0; k < 4; ++k)
+        if (host_in[k]) {
+            if (host_len[k]) memcpy(hs + host_at[k], host_in[k], host_len[k]);
+            dev_in[k] = d_in + host_at[k];
+        }
+    const void *yp = dev_in[0], *yi = dev_in[1], *yv = dev_in[2], *tl = dev_in[3];
+    S_.nnz_y = nnz_y;
     S_.yp = (const int32_t*)yp;
     S_.yi = (const int32_t*)yi;
     S_.yv = (const float*)yv;
     __half* p16 = half_ok ? cv.take<__half>((size_t)n * Bp) : nullptr;
-    unsigned* p16_max = half_ok ? cv.take<unsigned>(Bp) : nullptr;
     if (lr_on) {
         S_.lr.e = eig;
         S_.lr.rpad = rpad;
@@ -2587,15 +2608,13 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         S_.lr.C = cv.take<double>((size_t)rpad * Bp);
         S_.Cy = cv.take<double>((size_t)rpad * Bp);
         S_.lr.H = cv.take<float>((size_t)rpad * Bp);
-        S_.lr.Hhi = cv.take<__nv_bfloat16>((size_t)Bp16 * rpad);
-        S_.lr.Hlo = cv.take<__nv_bfloat16>((size_t)Bp16 * rpad);
-        S_.gcoef = cv.take<double>(rpad);
-        S_.hcoef = cv.take<double>(rpad);
-        S_.opcoef = cv.take<double>(rpad);
-        S_.dcoef = cv.take<double>(rpad);
-        S_.ones = cv.take<double>(rpad);
-        S_.negop = cv.take<double>(rpad);
-        std::vector<double> gc(rpad, 0.0), hc(rpad, 0.0), oc(rpad, 0.0), dc(rpad, 0.0), on(rpad, 0.0), ng(rpad, 0.0);
+        S_.lr.Hhi = zv.take<__nv_bfloat16>((size_t)Bp16 * rpad);
+        S_.lr.Hlo = zv.take<__nv_bfloat16>((size_t)Bp16 * rpad);
+        double** dst[6] = {&S_.gcoef, &S_.hcoef, &S_.opcoef, &S_.dcoef, &S_.ones, &S_.negop};
+        double* co = (double*)(hs + host_at[4]);
+        std::fill(co, co + 6 * (size_t)rpad, 0.0);
+        for (int k = 0; k < 6; ++k) *dst[k] = (double*)(d_in + host_at[4]) + (size_t)k * rpad;
+        double *gc = co, *hc = gc + rpad, *oc = hc + rpad, *dc = oc + rpad, *on = dc + rpad, *ng = on + rpad;
         const double a = alpha;
         const double c3 = mode == HD_MODE_PROJ ? a : a / (1.0 - a);
         for (int k = 0; k < r; ++k) {
@@ -2608,26 +2627,19 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
             on[k] = 1.0;
             ng[k] = -a / (1.0 - a) * l;
         }
-        HD_CUDA(ctx, cudaMemcpyAsync(S_.gcoef, gc.data(), rpad * 8, cudaMemcpyHostToDevice, ctx->stream));
-        HD_CUDA(ctx, cudaMemcpyAsync(S_.hcoef, hc.data(), rpad * 8, cudaMemcpyHostToDevice, ctx->stream));
-        HD_CUDA(ctx, cudaMemcpyAsync(S_.opcoef, oc.data(), rpad * 8, cudaMemcpyHostToDevice, ctx->stream));
-        HD_CUDA(ctx, cudaMemcpyAsync(S_.dcoef, dc.data(), rpad * 8, cudaMemcpyHostToDevice, ctx->stream));
-        HD_CUDA(ctx, cudaMemcpyAsync(S_.ones, on.data(), rpad * 8, cudaMemcpyHostToDevice, ctx->stream));
-        HD_CUDA(ctx, cudaMemcpyAsync(S_.negop, ng.data(), rpad * 8, cudaMemcpyHostToDevice, ctx->stream));
-        HD_CUDA(ctx, cudaMemsetAsync(S_.lr.Hhi, 0, (size_t)Bp16 * rpad * 2, ctx->stream));
-        HD_CUDA(ctx, cudaMemsetAsync(S_.lr.Hlo, 0, (size_t)Bp16 * rpad * 2, ctx->stream));
     }
+    if (in_bytes) HD_CUDA(ctx, cudaMemcpyAsync(d_in, hs, in_bytes, cudaMemcpyHostToDevice, ctx->stream));
 
     // ---------------- setup
     if (!ts && g->max_row < 0) {
         // the longest row bounds the rounding of the true residual (k_resid_pick)
-        HD_CUDA(ctx, cudaMemsetAsync(S_.num_active, 0, sizeof(int), ctx->stream));
         k_max_row<<<std::min<int64_t>(ceil_div(n, 256), (int64_t)ctx->num_sms * 8), 256, 0, ctx->stream>>>(
             g->row_ptr, n, S_.num_active);
         HD_CHECK_LAUNCH(ctx);
         HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll, S_.num_active, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
         HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         g->max_row = ctx->h_poll[0];
+        HD_CUDA(ctx, cudaMemsetAsync(S_.num_active, 0, sizeof(int), ctx->stream));
     }
     if (!ts) {
         S_.slab = spmm_slab(g, Bp);
@@ -2637,8 +2649,6 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         S_.P16 = p16;
         S_.p16_max = p16_max;
         S_.use_half = S_.num_active + 3;  // 0: the first iteration gathers fp32
-        HD_CUDA(ctx, cudaMemsetAsync(S_.use_half, 0, sizeof(int), ctx->stream));
-        HD_CUDA(ctx, cudaMemsetAsync(S_.p16_max, 0, (size_t)Bp * sizeof(unsigned), ctx->stream));
     }
     const int eff_mode = lr_on ? mode : HD_MODE_PAPER;
     const double a = alpha;
@@ -2655,15 +2665,13 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     // the true-residual confirmation
     HD_CUDA(ctx, cudaMemsetAsync(S_.R, 0, vec, ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(S_.X, 0, vec, ctx->stream));
-    HD_CUDA(ctx, cudaMemsetAsync(S_.err, 0, sizeof(int), ctx->stream));
-    k_scatter_y<<<B, 128, 0, ctx->stream>>>((const int32_t*)yp, (const int32_t*)yi, (const float*)yv, n, Bp, S_.R,
-                                            S_.err);
+    k_scatter_y<<<B, 128, 0, ctx->stream>>>((const int32_t*)yp, (const int32_t*)yi, (const float*)yv, nnz_y, n, Bp,
+                                            S_.R, S_.err);
     HD_CHECK_LAUNCH(ctx);
     const double* Cd = lr_on ? S_.lr.C : nullptr;
     const size_t cbytes = (size_t)rpad * Bp * sizeof(double);
     if (eff_mode == HD_MODE_PAPER) {
         if ((rc = launch_colsq(S_, S_.R))) return rc;
-        HD_CUDA(ctx, cudaMemsetAsync(S_.num_active, 0, sizeof(int), ctx->stream));
         k_fin_setup<<<Bp, 128, 0, ctx->stream>>>(S_.part, (int)S_.nch, Bp, B, (const float*)tl, S_.st, nullptr, nullptr,
                                                 0, S_.num_active);
         HD_CHECK_LAUNCH(ctx);
@@ -2681,7 +2689,6 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         HD_CUDA(ctx, cudaMemcpyAsync(S_.Cy, S_.lr.C, cbytes, cudaMemcpyDeviceToDevice, ctx->stream));
         if ((rc = lr_expand(ctx, S_.lr, EXP_SUB_R, S_.R, nullptr, nullptr, n, Bp, S_.st))) return rc;
         if ((rc = launch_colsq(S_, S_.R))) return rc;
-        HD_CUDA(ctx, cudaMemsetAsync(S_.num_active, 0, sizeof(int), ctx->stream));
         k_fin_setup<<<Bp, 128, 0, ctx->stream>>>(S_.part, (int)S_.nch, Bp, B, (const float*)tl, S_.st, nullptr, nullptr,
                                                 0, S_.num_active);
         HD_CHECK_LAUNCH(ctx);
@@ -2692,7 +2699,6 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         if ((rc = launch_colsq(S_, S_.R))) return rc;
         if ((rc = lr_reduce(ctx, S_.lr, S_.R, n, Bp))) return rc;
         if ((rc = lr_finish(ctx, S_.lr, Bp, S_.dcoef))) return rc;
-        HD_CUDA(ctx, cudaMemsetAsync(S_.num_active, 0, sizeof(int), ctx->stream));
         k_fin_setup<<<Bp, 128, 0, ctx->stream>>>(S_.part, (int)S_.nch, Bp, B, (const float*)tl, S_.st, Cd, S_.dcoef, r,
                                                 S_.num_active);
         HD_CHECK_LAUNCH(ctx);
@@ -2707,13 +2713,11 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     S_.xs = xs;
     S_.r = r;
     S_.max_iter = max_iter;
-    HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll, S_.num_active, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (ctx->h_poll[1])
-        return hd_fail(ctx, HD_ERR_INVALID_ARG, "bad observation: index out of range, non-finite value or bad y_ptr");
-    int active = ctx->h_poll[0];
-    int ran = 0, first_ran = -1;
-    std::vector<ColState> hs(B);
+    // (no poll here: the first run of iterations is queued behind the set-up; its
+    // kernels return at once if no column is active, and a bad observation, which
+    // the scatter left out, is reported by the poll after it)
+    int active = 1, ran = 0, first_ran = -1;
+    const ColState* hcol = (const ColState*)hs;
     for (int round = 0; round <= MAX_CONFIRM; ++round) {
         if (active > 0 && max_iter > 0 && (rc = iterate_until_stopped(S_, ran))) return rc;
         if (first_ran < 0) first_ran = ran;
@@ -2725,8 +2729,13 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         }
         HD_CHECK_LAUNCH(ctx);
         HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll, S_.num_active, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-        HD_CUDA(ctx, cudaMemcpyAsync(hs.data(), S_.st, B * sizeof(ColState), cudaMemcpyDeviceToHost, ctx->stream));
+        HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll + 1, S_.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+        HD_CUDA(ctx, cudaMemcpyAsync(hs, S_.st, B * sizeof(ColState), cudaMemcpyDeviceToHost, ctx->stream));
+        HD_CUDA(ctx, cudaMemcpyAsync(ctx->h_poll + 8, ctx->d_flags + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost,
+                                     ctx->stream));
         HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        if (ctx->h_poll[1]) return hd_fail(ctx, HD_ERR_INVALID_ARG, "%s", BAD_OBSERVATION);
+        if (ctx->h_poll[8] || ctx->h_poll[9]) return lr_tc_check_flags(ctx);
         active = ctx->h_poll[0];
         if (active == 0) break;
         if ((rc = restart_columns(S_))) return rc;
@@ -2735,13 +2744,13 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     // this one's columns took before any restart (without restarts the
     // columns' own count, else the iterations launched)
     int most = 0;
-    for (int j = 0; j < B; ++j) most = std::max(most, hs[j].iters);
+    for (int j = 0; j < B; ++j) most = std::max(most, hcol[j].iters);
     ctx->hint_key = iteration_key(S_);
     ctx->iter_hint = ran == first_ran ? most : first_ran;
     for (int j = 0; j < B; ++j) {
-        if (iters && !hd_is_device_ptr(iters)) iters[j] = hs[j].iters;
-        if (relres && !hd_is_device_ptr(relres)) relres[j] = hs[j].bb > 0 ? (float)std::sqrt(hs[j].rr / hs[j].bb) : 0.f;
-        if (status && !hd_is_device_ptr(status)) status[j] = hs[j].status;
+        if (iters && !hd_is_device_ptr(iters)) iters[j] = hcol[j].iters;
+        if (relres && !hd_is_device_ptr(relres)) relres[j] = hcol[j].bb > 0 ? (float)std::sqrt(hcol[j].rr / hcol[j].bb) : 0.f;
+        if (status && !hd_is_device_ptr(status)) status[j] = hcol[j].status;
     }
     // ---------------- spectral term (Eq. 17-18): X += U g(Lambda) U^T y, or U h(Lambda) U^T y (projected form)
     if (lr_on && eff_mode != HD_MODE_PCG && !temporal_only) {
@@ -2767,7 +2776,8 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
             HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         }
     }
-    if (lr_on && lr_use_tensor_cores(eig)) return lr_tc_check_flags(ctx);
+    // the tensor-core kernels' status was read with the confirmation unless more ran since
+    if (lr_on && lr_use_tensor_cores(eig) && (eff_mode != HD_MODE_PCG || !x_direct)) return lr_tc_check_flags(ctx);
     return HD_OK;
 }
 
@@ -2926,7 +2936,8 @@ extern "C" int hd_filter_poly(hd_ctx* ctx, const hd_graph* g, const hd_eig* eig,
     }
     HD_CUDA(ctx, cudaMemsetAsync(Yd, 0, vec, ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
-    k_scatter_y<<<B, 128, 0, ctx->stream>>>((const int32_t*)yp, (const int32_t*)yi, (const float*)yv, n, Bp, Yd, err);
+    k_scatter_y<<<B, 128, 0, ctx->stream>>>((const int32_t*)yp, (const int32_t*)yi, (const float*)yv, nnz_y, n, Bp,
+                                            Yd, err);
     HD_CHECK_LAUNCH(ctx);
     const int64_t c4 = (int64_t)n * Bp / 4;
     // h(W_r) y by Horner's rule on the black box W_r z = W z - U (Lambda (U^T z)) (Eq. 32)

@@ -148,6 +148,7 @@ struct Engine {
     const int32_t* yp = nullptr;
     const int32_t* yi = nullptr;
     const float* yv = nullptr;
+    int32_t nnz_y = 0;
     double* Cy = nullptr;       // U^T y [rpad][Bp] (paper and projected forms: x^s and b)
     // fp16 copy of P for the SpMM gathers of late iterations (hd_query_batch
     // only: the decision covers the whole batch, so a column's bits would
