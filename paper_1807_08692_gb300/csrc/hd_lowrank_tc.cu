@@ -103,6 +103,7 @@ struct ExpandArgs {
     float* out;
     const float* R;
     const float* P;
+    Panels pv;              // EXP_DIRECTION: layout of P and out
     const ColState* st;
     const int* gate;
     const float* scale;  // per-row scale of FP8 storage
@@ -295,6 +296,8 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
         auto load_ops = [&](int t_, int c0_) {
             const int j = a.c0 + c0_ * 16 + 4 * ch;
             const bool colok = c0_ + (ch >> 2) < ce && j < a.Bp && a.op != EXP_SET_X;
+            int pw;
+            const float* Pc = panel_column(a.pv, a.P, j, pw);
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 const int64_t row_ = (int64_t)t_ * BM + quarter * 32 + sr + 4 * k;
@@ -302,7 +305,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                 if (!colok || row_ >= a.n) continue;
                 if (a.op == EXP_DIRECTION) {
                     g1[k] = *reinterpret_cast<const float4*>(a.R + row_ * a.Bp + j);
-                    g2[k] = *reinterpret_cast<const float4*>(a.P + row_ * a.Bp + j);
+                    g2[k] = *reinterpret_cast<const float4*>(Pc + row_ * pw);
                 } else {
                     g1[k] = *reinterpret_cast<const float4*>(a.out + row_ * a.Bp + j);
                 }
@@ -343,6 +346,8 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                 __syncwarp();
                 const int j = a.c0 + c0 * 16 + 4 * ch;
                 const bool colok = c0 + (ch >> 2) < ce && j < a.Bp;
+                int ow;
+                float* oc = panel_column(a.pv, a.out, j, ow);
                 float b0 = 0.f, b1 = 0.f, b2 = 0.f, b3 = 0.f;
                 bool f0 = false, f1 = false, f2 = false, f3 = false;
                 if (colok && a.op == EXP_DIRECTION) {
@@ -378,7 +383,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                         w.z = (f2 ? 0.0f : r4.z) + acc.z + (b2 == 0.0f ? 0.0f : b2 * p4.z);
                         w.w = (f3 ? 0.0f : r4.w) + acc.w + (b3 == 0.0f ? 0.0f : b3 * p4.w);
                     }
-                    *reinterpret_cast<float4*>(a.out + row_g * a.Bp + j) = w;
+                    *reinterpret_cast<float4*>(oc + row_g * ow) = w;
                 }
                 __syncwarp();
             }
@@ -733,7 +738,7 @@ int lr_tc_check_flags(hd_ctx* ctx) {
 }
 
 int lr_tc_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float* Rv, const float* Pv, int64_t n,
-                 int32_t Bp, const ColState* st, const int* gate) {
+                 int32_t Bp, const ColState* st, const int* gate, const Panels* pv) {
     const hd_eig* e = lr.e;
     const int su = e->storage == HD_FP8 ? 1 : 0;
     const bool split = e->storage == HD_F32;  // [hi | lo] bf16 copy of the fp32 U
@@ -777,6 +782,7 @@ int lr_tc_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float
         a.out = out;
         a.R = Rv;
         a.P = Pv;
+        a.pv = pv && op == EXP_DIRECTION ? *pv : panel_rows(n, Bp);
         a.st = st;
         a.gate = gate;
         a.scale = e->scale;

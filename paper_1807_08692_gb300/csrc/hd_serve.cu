@@ -305,6 +305,7 @@ static int lane_open(hd_ctx* ctx, const hd_graph* g, const hd_eig* eig, double a
         HD_CUDA(ctx, cudaMemsetAsync(E.lr.Hhi, 0, (size_t)Bp16 * rpad * 2, ctx->stream));
         HD_CUDA(ctx, cudaMemsetAsync(E.lr.Hlo, 0, (size_t)Bp16 * rpad * 2, ctx->stream));
     }
+    engine_set_panels(E, E.eff_mode);
     HD_CUDA(ctx, cudaMemsetAsync(L.dev, 0, 4 * ws_size(vec), ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(E.num_active, 0, 16 * sizeof(int), ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(L.d_ctl, 0, 16 * sizeof(int), ctx->stream));

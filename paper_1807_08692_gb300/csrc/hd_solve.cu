@@ -102,9 +102,11 @@ __device__ __forceinline__ bool slab_has_work(const ColState* st) {
 // gathers and read the row's indices two at a time (0.28 ms against 0.38 ms
 // on the 1M-node graph, the same bits).  128 rows per block step.
 __device__ __forceinline__ void spmm_rows_pair4(const int32_t* rp, const int32_t* ci, const float* wv,
-                                                const float* P, float* Q, int64_t n, int32_t ld, float c1, float c2) {
+                                                const float* P, const Panels& pv, float* Q, int64_t n, int32_t ld,
+                                                int32_t col, float c1, float c2) {
     const int lane = threadIdx.x & 31, h = lane & 1;
-    const int col = blockIdx.y * 4;
+    int pw;
+    const float* Pc = panel_column(pv, P, col, pw);
     // rows advance warp-uniformly (the shuffle needs every lane); a lane past
     // the last row works on an empty row and writes nothing
     for (int64_t r0 = (int64_t)blockIdx.x * 128 + (threadIdx.x >> 5) * 16; r0 < n; r0 += (int64_t)gridDim.x * 128) {
@@ -121,7 +123,7 @@ __device__ __forceinline__ void spmm_rows_pair4(const int32_t* rp, const int32_t
             for (int u = 0; u < 8; ++u) {
                 const int32_t k = t + 2 * u + h;
                 w[u] = __ldg(wv + k);
-                v[u] = ld4(P + (int64_t)__ldg(ci + k) * ld + col);
+                v[u] = ld4(Pc + (int64_t)__ldg(ci + k) * pw);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -135,7 +137,7 @@ __device__ __forceinline__ void spmm_rows_pair4(const int32_t* rp, const int32_t
             for (int u = 0; u < 4; ++u) {
                 const int32_t k = t + 2 * u + h;
                 w[u] = __ldg(wv + k);
-                v[u] = ld4(P + (int64_t)__ldg(ci + k) * ld + col);
+                v[u] = ld4(Pc + (int64_t)__ldg(ci + k) * pw);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -151,7 +153,7 @@ __device__ __forceinline__ void spmm_rows_pair4(const int32_t* rp, const int32_t
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     w[u] = u < m ? __ldg(wv + t + u) : 0.f;
-                    v[u] = u < m ? ld4(P + (int64_t)__ldg(ci + t + u) * ld + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[u] = u < m ? ld4(Pc + (int64_t)__ldg(ci + t + u) * pw) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -168,7 +170,7 @@ __device__ __forceinline__ void spmm_rows_pair4(const int32_t* rp, const int32_t
             s.y += oy;
             s.z += oz;
             s.w += ow;
-            const float4 own = ld4(P + row * ld + col);
+            const float4 own = ld4(Pc + row * pw);
             float4 q;
             q.x = c1 * own.x - c2 * s.x;
             q.y = c1 * own.y - c2 * s.y;
@@ -182,11 +184,12 @@ __device__ __forceinline__ void spmm_rows_pair4(const int32_t* rp, const int32_t
 // 4-column slabs of Q = c1 P - c2 W P.  `skip` (may be null): the launch
 // returns at once when *skip is not 0.
 __global__ void __launch_bounds__(256, 8) k_spmm4(const int32_t* rp, const int32_t* ci, const float* wv, const float* P,
-                                                  float* Q, int64_t n, int32_t ld, float c1, float c2,
-                                                  const ColState* st, const int* skip) {
+                                                  const Panels pv, float* Q, int64_t n, int32_t ld, int32_t first,
+                                                  float c1, float c2, const ColState* st, const int* skip) {
     if (skip && *skip) return;
-    if (!slab_has_work<4>(st)) return;
-    spmm_rows_pair4(rp, ci, wv, P, Q, n, ld, c1, c2);
+    const int col = first + blockIdx.y * 4;
+    if (!columns_have_work(st, col, col + 4)) return;
+    spmm_rows_pair4(rp, ci, wv, P, pv, Q, n, ld, col, c1, c2);
 }
 
 // ---- the row gathers shared by the wider SpMM kernels
@@ -295,18 +298,20 @@ __device__ __forceinline__ void row_entries(const int32_t* __restrict__ ci, cons
 template <int LC, int G>
 __global__ void __launch_bounds__(128, spmm_blocks(LC)) k_spmm(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                  const float* __restrict__ wv, const float* __restrict__ P,
-                                                 float* __restrict__ Q, unsigned n, int32_t ld, int L_, float c1,
-                                                 float c2, const ColState* st, const int* skip) {
+                                                 const Panels pv, float* __restrict__ Q, unsigned n, int32_t ld,
+                                                 int32_t first, int32_t last, int L_, float c1, float c2,
+                                                 const ColState* st, const int* skip) {
     if (skip && *skip) return;
     const int Lq = LC ? LC : L_;
-    if (!columns_have_work(st, blockIdx.y * 4 * Lq, min(ld, (int)(blockIdx.y + 1) * 4 * Lq))) return;
+    const int c0 = first + blockIdx.y * 4 * Lq;
+    if (!columns_have_work(st, c0, min(last, c0 + 4 * Lq))) return;
     const RowLanes r = row_lanes<LC>(L_);
     if (r.idle) return;
-    const int quad = blockIdx.y * Lq + r.g, nq = ld >> 2;
-    const bool own_col = LC || quad < nq;
-    const int col = 4 * (own_col ? quad : nq - 1);
-    const float* Pc = P + col;
-    auto load = [&](int32_t j) { return ld4(Pc + (int64_t)j * ld); };
+    const bool own_col = LC || c0 + 4 * r.g < last;
+    const int col = own_col ? c0 + 4 * r.g : last - 4;
+    int pw;
+    const float* Pc = panel_column(pv, P, col, pw);
+    auto load = [&](int32_t j) { return ld4(Pc + (int64_t)j * pw); };
     for (unsigned row = r.row; row < n; row += r.step) {
         const unsigned b = __ldg(rp + row), e = __ldg(rp + row + 1);
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -325,7 +330,7 @@ __global__ void __launch_bounds__(128, spmm_blocks(LC)) k_spmm(const int32_t* __
         s.y += s2.y;
         s.z += s2.z;
         s.w += s2.w;
-        const float4 own = ld4(Pc + (int64_t)row * ld);
+        const float4 own = ld4(Pc + (int64_t)row * pw);
         float4 q;
         q.x = c1 * own.x - c2 * s.x;
         q.y = c1 * own.y - c2 * s.y;
@@ -411,7 +416,7 @@ constexpr double HALF_THETA = 25.0;
 
 // per-column max |P| (the bits of a non-negative float order like the value);
 // runs when the next SpMM gathers the fp16 copy and some column is active
-__global__ void __launch_bounds__(256) k_colmax(const float* __restrict__ P, int64_t n, int32_t ld,
+__global__ void __launch_bounds__(256) k_colmax(const float* __restrict__ P, const Panels pv, int64_t n, int32_t ld,
                                                 unsigned* __restrict__ mx, const int* __restrict__ use_half,
                                                 const int* __restrict__ num_active) {
     if (!*use_half || !*num_active) return;
@@ -422,9 +427,11 @@ __global__ void __launch_bounds__(256) k_colmax(const float* __restrict__ P, int
     __syncthreads();
     if ((int)threadIdx.x < rpb * nq) {
         const int q = threadIdx.x % nq;
+        int pw;
+        const float* Pc = panel_column(pv, P, 4 * q, pw);
         float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;
         for (int64_t row = (int64_t)blockIdx.x * rpb + threadIdx.x / nq; row < n; row += (int64_t)gridDim.x * rpb) {
-            const float4 v = ld4(P + row * ld + 4 * q);
+            const float4 v = ld4(Pc + row * pw);
             m0 = fmaxf(m0, fabsf(v.x));
             m1 = fmaxf(m1, fabsf(v.y));
             m2 = fmaxf(m2, fabsf(v.z));
@@ -451,8 +458,9 @@ __device__ __forceinline__ float half_scale(unsigned mbits, bool inverse) {
 }
 
 // P16 = fp16(P_j 2^k_j) column by column
-__global__ void __launch_bounds__(256) k_to_half(const float* __restrict__ P, int64_t n, int32_t ld,
+__global__ void __launch_bounds__(256) k_to_half(const float* __restrict__ P, const Panels pv, int64_t n, int32_t ld,
                                                  const unsigned* __restrict__ mx, __half* __restrict__ P16,
+                                                 const Panels hv,
                                                  const int* __restrict__ use_half,
                                                  const int* __restrict__ num_active) {
     if (!*use_half || !*num_active) return;
@@ -462,14 +470,17 @@ __global__ void __launch_bounds__(256) k_to_half(const float* __restrict__ P, in
     const int q = threadIdx.x % nq;
     const float s0 = half_scale(mx[4 * q], false), s1 = half_scale(mx[4 * q + 1], false);
     const float s2 = half_scale(mx[4 * q + 2], false), s3 = half_scale(mx[4 * q + 3], false);
+    int pw, hw;
+    const float* Pc = panel_column(pv, P, 4 * q, pw);
+    __half* Hc = panel_column(hv, P16, 4 * q, hw);
     for (int64_t row = (int64_t)blockIdx.x * rpb + threadIdx.x / nq; row < n; row += (int64_t)gridDim.x * rpb) {
-        const float4 v = ld4(P + row * ld + 4 * q);
+        const float4 v = ld4(Pc + row * pw);
         const __half2 a = __floats2half2_rn(v.x * s0, v.y * s1);
         const __half2 b = __floats2half2_rn(v.z * s2, v.w * s3);
         uint2 o;
         o.x = *reinterpret_cast<const unsigned*>(&a);
         o.y = *reinterpret_cast<const unsigned*>(&b);
-        *reinterpret_cast<uint2*>(P16 + row * ld + 4 * q) = o;
+        *reinterpret_cast<uint2*>(Hc + row * hw) = o;
     }
 }
 
@@ -491,31 +502,33 @@ __global__ void __launch_bounds__(256) k_to_half(const float* __restrict__ P, in
 template <int LC, int G>
 __global__ void __launch_bounds__(128, 7) k_spmm_h(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                    const float* __restrict__ wv, const __half* __restrict__ P16,
-                                                   const unsigned* __restrict__ mx, const float* __restrict__ P,
-                                                   float* __restrict__ Q, unsigned n, int32_t ld, int L_, float c1,
+                                                   const Panels hv, const unsigned* __restrict__ mx,
+                                                   const float* __restrict__ P, const Panels pv, float* __restrict__ Q,
+                                                   unsigned n, int32_t ld, int32_t first, int32_t last, int L_, float c1,
                                                    float c2, const ColState* st, const int* __restrict__ use_half) {
     if (!*use_half) return;
     const int Lq = LC ? LC : L_;
-    const int first = blockIdx.y * 8 * Lq, last = min(ld, first + 8 * Lq);
+    const int c0 = first + blockIdx.y * 8 * Lq, ce = min(last, c0 + 8 * Lq);
     // up to 256 columns of a slab against 128 threads
-    if (!columns_have_work(st, first, min(last, first + 128)) && !columns_have_work(st, first + 128, last)) return;
+    if (!columns_have_work(st, c0, min(ce, c0 + 128)) && !columns_have_work(st, c0 + 128, ce)) return;
     const RowLanes r = row_lanes<LC>(L_);
     if (r.idle) return;
-    const int oct = blockIdx.y * Lq + r.g, no = ld >> 3;
-    const bool own_col = LC || oct < no;
-    const int col = 8 * (own_col ? oct : no - 1);
+    const bool own_col = LC || c0 + 8 * r.g < last;
+    const int col = own_col ? c0 + 8 * r.g : last - 8;
+    int pw, hw;
+    const float* Po = panel_column(pv, P, col, pw);
+    const __half* Pc = panel_column(hv, P16, col, hw);
     float inv[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) inv[c] = half_scale(mx[col + c], true);
-    const __half* Pc = P16 + col;
-    auto load = [&](int32_t j) { return __ldg(reinterpret_cast<const uint4*>(Pc + (int64_t)j * ld)); };
+    auto load = [&](int32_t j) { return __ldg(reinterpret_cast<const uint4*>(Pc + (int64_t)j * hw)); };
     for (unsigned row = r.row; row < n; row += r.step) {
         const unsigned b = __ldg(rp + row), e = __ldg(rp + row + 1);
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         row_entries<LC, G, uint4>(
             ci, wv, b, e, r, load, [&](int, float w, const uint4& v) { FMA8H(acc, w, v); },
             [&](float w, const uint4& v) { FMA8H(acc, w, v); });
-        const float* po = P + (int64_t)row * ld + col;
+        const float* po = Po + (int64_t)row * pw;
         const float4 o0 = ld4(po), o1 = ld4(po + 4);
         const float own[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
         float q[8];
@@ -1006,14 +1019,16 @@ __global__ void __launch_bounds__(256) k_colsq(const float* __restrict__ V, int6
 }
 
 // Partials of P^T Q (columns being iterated).
-__global__ void __launch_bounds__(256) k_dot(const float* __restrict__ P, const float* __restrict__ Q, int64_t n,
-                                             int32_t ld, int rch, float2* __restrict__ part,
-                                             const ColState* __restrict__ st) {
+__global__ void __launch_bounds__(256) k_dot(const float* __restrict__ P, const Panels pv,
+                                             const float* __restrict__ Q, int64_t n, int32_t ld, int rch,
+                                             float2* __restrict__ part, const ColState* __restrict__ st) {
     const RedThread t = red_thread(n, ld, rch, st);
     KSum acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+    int pw;
+    const float* Pc = panel_column(pv, P, t.col, pw);
     if (t.work)
         for (int64_t row = t.r0; row < t.r1; row += RG) {
-            const float4 a = ld4(P + row * ld + t.col), b = ld4(Q + row * ld + t.col);
+            const float4 a = ld4(Pc + row * pw), b = ld4(Q + row * ld + t.col);
             ksum_add_product(acc[0], a.x, b.x);
             ksum_add_product(acc[1], a.y, b.y);
             ksum_add_product(acc[2], a.z, b.z);
@@ -1074,17 +1089,20 @@ __device__ __forceinline__ void update_row(const UpdateQuad& u, const float4& p,
 
 // X += xs a P; R -= a Q; partials of ||R||^2.
 __global__ void __launch_bounds__(256) k_update(float* __restrict__ X, float* __restrict__ R,
-                                                const float* __restrict__ P, const float* __restrict__ Q, int64_t n,
-                                                int32_t ld, int rch, const ColState* __restrict__ st,
-                                                float xs, float2* __restrict__ part, const IterReset z) {
+                                                const float* __restrict__ P, const Panels pv,
+                                                const float* __restrict__ Q, int64_t n, int32_t ld, int rch,
+                                                const ColState* __restrict__ st, float xs, float2* __restrict__ part,
+                                                const IterReset z) {
     iter_reset(z);
     const RedThread t = red_thread(n, ld, rch, st);
     KSum acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
     if (t.work) {
         const UpdateQuad uq = update_quad(st, t.col, xs);
+        int pw;
+        const float* Pc = panel_column(pv, P, t.col, pw);
         for (int64_t row = t.r0; row < t.r1; row += RG) {
             const int64_t o = row * ld + t.col;
-            const float4 p = ld4v(P + o), q = ld4v(Q + o);
+            const float4 p = ld4v(Pc + row * pw), q = ld4v(Q + o);
             float4 x = ld4v(X + o), r = ld4v(R + o);
             update_row(uq, p, q, x, r);
             st4(X + o, x);
@@ -1108,8 +1126,9 @@ constexpr int rs_smem() {
 }
 template <int OP>
 __global__ void __launch_bounds__(256) k_red_staged(float* __restrict__ X, float* __restrict__ R,
-                                                    const float* __restrict__ P, const float* __restrict__ Q,
-                                                    int64_t n, int32_t ld, int rch, const ColState* __restrict__ st,
+                                                    const float* __restrict__ P, const Panels pv,
+                                                    const float* __restrict__ Q, int64_t n, int32_t ld, int rch,
+                                                    const ColState* __restrict__ st,
                                                     float xs, float2* __restrict__ part, const IterReset z) {
     if (OP == RED_UPDATE) iter_reset(z);
     constexpr int UL = 4;  // rows in flight per thread
@@ -1129,6 +1148,8 @@ __global__ void __launch_bounds__(256) k_red_staged(float* __restrict__ X, float
         work = work && (st[col].active | st[col + 1].active | st[col + 2].active | st[col + 3].active);
         if (OP == RED_UPDATE) uq = update_quad(st, col, xs);
     }
+    int pw;
+    const float* Pc = panel_column(pv, P, col, pw);
     // summing threads: column sc, partial sum sg
     const int sc = threadIdx.x % nc, sg = threadIdx.x / nc;
     bool sum = sg < RG;
@@ -1146,7 +1167,7 @@ __global__ void __launch_bounds__(256) k_red_staged(float* __restrict__ X, float
                 for (int u = 0; u < UL; ++u) {
                     const int64_t o = (base + r0 + u * pass) * ld + col;
                     if (r0 + u * pass < rows) {
-                        p[u] = ld4v(P + o);
+                        p[u] = ld4v(Pc + (base + r0 + u * pass) * pw);
                         if (OP != RED_SQ) q[u] = ld4v(Q + o);
                         if (OP == RED_UPDATE) {
                             x[u] = ld4v(X + o);
@@ -1194,8 +1215,8 @@ __global__ void __launch_bounds__(256) k_red_staged(float* __restrict__ X, float
 
 // P = R + beta P.
 template <int S>
-__global__ void __launch_bounds__(256) k_direction(float* __restrict__ P, const float* __restrict__ R, int64_t n,
-                                                   int32_t ld, const ColState* __restrict__ st) {
+__global__ void __launch_bounds__(256) k_direction(float* __restrict__ P, const Panels pv, const float* __restrict__ R,
+                                                   int64_t n, int32_t ld, const ColState* __restrict__ st) {
     constexpr int L = S / 4;
     constexpr int RPB = 256 / L;
     if (!slab_has_work<S>(st)) return;
@@ -1205,15 +1226,17 @@ __global__ void __launch_bounds__(256) k_direction(float* __restrict__ P, const 
                 b3 = (float)st[col + 3].beta;
     // a served column that just took a new request: p0 = y, added after this
     const bool f0 = st[col].refill, f1 = st[col + 1].refill, f2 = st[col + 2].refill, f3 = st[col + 3].refill;
+    int pw;
+    float* Pc = panel_column(pv, P, col, pw);
     for (int64_t row = (int64_t)blockIdx.x * RPB + threadIdx.x / L; row < n; row += (int64_t)gridDim.x * RPB) {
-        const int64_t o = row * ld + col;
-        const float4 r = ld4v(R + o);
-        float4 p = ld4v(P + o);
+        float* o = Pc + row * pw;
+        const float4 r = ld4v(R + row * ld + col);
+        float4 p = ld4v(o);
         p.x = b0 == 0.0f ? (f0 ? 0.0f : r.x) : fmaf(b0, p.x, r.x);
         p.y = b1 == 0.0f ? (f1 ? 0.0f : r.y) : fmaf(b1, p.y, r.y);
         p.z = b2 == 0.0f ? (f2 ? 0.0f : r.z) : fmaf(b2, p.z, r.z);
         p.w = b3 == 0.0f ? (f3 ? 0.0f : r.w) : fmaf(b3, p.w, r.w);
-        st4(P + o, p);
+        st4(o, p);
     }
 }
 
@@ -1477,16 +1500,18 @@ __global__ void k_refill_h(Refill rf, const double* coef, int rpad, int32_t Bp, 
 // p0 += y for the columns that took a staged request (the direction left
 // U D U^T y there, or 0 without eigenpairs); y is kept with the column for its
 // first update
-__global__ void k_refill_p(Refill rf, float* P, int32_t Bp) {
+__global__ void k_refill_p(Refill rf, float* P, const Panels pv, int32_t Bp) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= Bp) return;
     const int c = rf.assign[j];
     if (c < 0) return;
     const int32_t b = rf.off[c], e = rf.off[c + 1];
+    int pw;
+    float* Pc = panel_column(pv, P, j, pw);
     for (int32_t t = b; t < e; ++t) {
         const int32_t i = rf.yidx[t];
         const float v = rf.yval[t];
-        P[(int64_t)i * Bp + j] += v;
+        Pc[(int64_t)i * pw] += v;
         rf.col_idx[(int64_t)j * REFILL_MAX_NNZ + (t - b)] = i;
         rf.col_val[(int64_t)j * REFILL_MAX_NNZ + (t - b)] = v;
     }
@@ -1831,10 +1856,10 @@ static int lr_coef(hd_ctx* ctx, const LowRank& lr, int32_t Bp, const double* coe
 }
 
 int lr_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float* Rv, const float* Pv, int64_t n,
-              int32_t Bp, const ColState* st, const int* gate) {
+              int32_t Bp, const ColState* st, const int* gate, const Panels* pv) {
     HD_PROF(ctx, "lr_expand");
     if (lr.e->sparse) return lr_sparse_expand(ctx, lr, op, out, Rv, Pv, n, Bp, st, gate);
-    if (lr_use_tensor_cores(lr.e)) return lr_tc_expand(ctx, lr, op, out, Rv, Pv, n, Bp, st, gate);
+    if (lr_use_tensor_cores(lr.e)) return lr_tc_expand(ctx, lr, op, out, Rv, Pv, n, Bp, st, gate, pv);
     const hd_eig* e = lr.e;
     size_t smem = (size_t)e->r * 16 * sizeof(float);
     int gx = (int)std::min<int64_t>(ceil_div(n, 64), (int64_t)ctx->num_sms * 8);
@@ -1899,7 +1924,8 @@ VecLaunch vec_launch(hd_ctx* ctx, int64_t n, int32_t Bp, int S) {
 // a 64-column pass over a block larger than L2 reads 1.3 times the DRAM bytes
 // (1M nodes, 64 columns: 1.18 ms against 1.50 ms).  16 lanes when the block fits
 // in L2 (100,000 x 64: 0.082 ms against 0.086 ms), and from 256 columns on, where
-// the 128-byte lines of one pass lie 1 KB apart (1M x 256: 6.1 ms against 6.7).
+// the 128-byte lines of one pass lie 1 KB apart (1M x 256: 6.1 ms against 6.7;
+// panels, see panels_for, take 5.2).
 // Other widths take the whole row at once up to 16 lanes, else the fewest even
 // parts of at most 16: 100,000 x 40 runs in 0.067 ms with 10 lanes, 0.12 ms in
 // two passes of 9 and 0.174 ms in five of 2.
@@ -1916,6 +1942,36 @@ int spmm_slab(const hd_graph* g, int32_t Bp) {
     const int S = getenv("HD_SLAB") ? pick_slab(Bp) : 4 * spmm_lanes(Bp, 4, spmm_exceeds_l2(g->n, Bp, 4));
     g->slab_cache[Bp] = S;
     return S;
+}
+
+// Layout of a gathered n x Bp block with `bytes` per entry: rows, or panels as wide
+// as a 128-byte line (32 fp32 or 64 fp16 columns).  A row of another width straddles
+// lines, and the passes of a wide one find their lines far apart; a panel row is one
+// line and neighbouring rows share DRAM pages.  Whole solves in rows / in panels, ms:
+//   ragged widths   1M x 40: 16.2 / 14.4   1M x 72: 38.0 / 26.2   1M x 100: 65.5 / 44.9
+//                   200,000 x 72: 3.70 / 3.44   30,000 x 148: 1.38 / 1.32   30,000 x 52: 0.67 / 0.69
+//   whole lines     1M x 64: 17.0 / 17.1   1M x 128: 37.9 / 34.3   1M x 256: 75.4 / 67.8
+//                   400,000 x 128: 11.6 / 11.7   250,000 x 256: 14.3 / 13.9
+// The columns past the last whole panel stand alone where the block exceeds L2 (1M x
+// 72: 26.2 against 29.1 when fewer than half a panel join the one before), and join
+// below that, where one launch less counts more (100,000 x 72: 1.84 against 1.90).
+static Panels panels_for(int64_t n, int32_t Bp, int bytes) {
+    const int32_t w = 128 / bytes;
+    const int64_t mb = n * Bp * bytes >> 20;
+    if (Bp % w ? Bp < w || mb < 16 : Bp <= 2 * w || mb < 256) return panel_rows(n, Bp);
+    const int32_t alone = spmm_exceeds_l2(n, Bp, bytes) ? 4 : w / 2;
+    const int32_t last = ((Bp + w - alone) / w - 1) * w;
+    return Panels{n, w, last, Bp - last};
+}
+
+void engine_set_panels(Engine& E, int eff_mode) {
+    E.pv = E.hv = panel_rows(E.n, E.Bp);
+    // (truncated systems and segments read rows, and so do the low-rank products of
+    // the deflated forms and those off the tensor cores; so does a forced slab width)
+    if (E.ts || E.segK > 1 || getenv("HD_SLAB")) return;
+    if (E.has_lr && (eff_mode != HD_MODE_PCG || !lr_use_tensor_cores(E.lr.e))) return;
+    E.pv = panels_for(E.n, E.Bp, 4);
+    E.hv = panels_for(E.n, E.Bp, 2);
 }
 
 // LC = L where L is a power of two that divides the width, else LC = 0
@@ -1938,26 +1994,34 @@ static dim3 spmm_grid(hd_ctx* ctx, int64_t n, int32_t cols, int per, int L, int 
     return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, rpb), (int64_t)ctx->num_sms * per_sm)),
                 (unsigned)ceil_div(cols / per, L));
 }
-// Q = c1 P - c2 W P in slabs of S columns
-static int spmm_launch(hd_ctx* ctx, const hd_graph* g, const float* P, float* Q, int32_t ld, int S, float c1, float c2,
-                       const ColState* st, const int* skip) {
-    if (S == 4) {
-        const VecLaunch v = vec_launch(ctx, g->n, ld, 4);
-        k_spmm4<<<dim3(v.nblk, v.slabs), 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, P, Q, g->n, ld, c1, c2, st,
-                                                                skip);
-    } else {
-        const int L = S / 4;
-        const dim3 grid = spmm_grid(ctx, g->n, ld, 4, L, spmm_blocks(L));
-        HD_DISPATCH_L(L, ld / 4, (k_spmm<LC, G><<<grid, 128, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, P, Q, (unsigned)g->n,
-                                                                        ld, L, c1, c2, st, skip)));
+// Q = c1 P - c2 W P in slabs of S columns, or panel by panel
+static int spmm_launch(hd_ctx* ctx, const hd_graph* g, const float* P, const Panels& pv, float* Q, int32_t ld, int S,
+                       float c1, float c2, const ColState* st, const int* skip) {
+    // panel by panel; apart, a last one of another width
+    if (pv.last) S = std::min(S, pv.w);
+    const int32_t cut = S == pv.w && pv.wlast != pv.w ? pv.last : 0;
+    for (int32_t first = 0; first < ld; first = first < cut ? cut : ld) {
+        const int32_t last = first < cut ? cut : ld;
+        const int L = cut && last == ld ? (ld - cut) / 4 : S / 4;
+        if (L == 1) {
+            const VecLaunch v = vec_launch(ctx, g->n, last - first, 4);
+            k_spmm4<<<dim3(v.nblk, v.slabs), 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, P, pv, Q, g->n, ld,
+                                                                    first, c1, c2, st, skip);
+        } else {
+            const dim3 grid = spmm_grid(ctx, g->n, last - first, 4, L, spmm_blocks(L));
+            HD_DISPATCH_L(L, (last - first) / 4,
+                          (k_spmm<LC, G><<<grid, 128, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, P, pv, Q,
+                                                                        (unsigned)g->n, ld, first, last, L, c1, c2, st,
+                                                                        skip)));
+        }
+        HD_CHECK_LAUNCH(ctx);
     }
-    HD_CHECK_LAUNCH(ctx);
     return HD_OK;
 }
 
 int hd_spmm_apply(hd_ctx* ctx, const hd_graph* g, const float* P, float* Q, int32_t ld, int32_t B, float c1,
                   float c2) {
-    return spmm_launch(ctx, g, P, Q, ld, 4 * spmm_lanes(ld, 4, spmm_exceeds_l2(g->n, ld, 4)), c1, c2, nullptr, nullptr);
+    return spmm_launch(ctx, g, P, panel_rows(g->n, ld), Q, ld, 4 * spmm_lanes(ld, 4, spmm_exceeds_l2(g->n, ld, 4)), c1, c2, nullptr, nullptr);
 }
 
 // grid and block of the column reductions: one chunk per block row.  `staged`
@@ -1979,14 +2043,14 @@ static RedLaunch red_launch(const Engine& E) {
     return l;
 }
 template <int OP>
-static int launch_staged(Engine& E, const RedLaunch& l, const float* P, float2* part, const ColState* st,
-                         const IterReset& z = {}) {
+static int launch_staged(Engine& E, const RedLaunch& l, const float* P, const Panels& pv, float2* part,
+                         const ColState* st, const IterReset& z = {}) {
     hd_ctx* ctx = E.ctx;
     static uint64_t attr = 0;
     if (hd_first_on_device(attr, ctx->device))
         HD_CUDA(ctx, cudaFuncSetAttribute(k_red_staged<OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs_smem<OP>()));
-    k_red_staged<OP><<<l.grid, l.block, rs_smem<OP>(), ctx->stream>>>(E.X, E.R, P, E.Q, E.n, E.Bp, E.rch, st, E.xs, part,
-                                                                        z);
+    k_red_staged<OP><<<l.grid, l.block, rs_smem<OP>(), ctx->stream>>>(E.X, E.R, P, pv, E.Q, E.n, E.Bp, E.rch, st, E.xs,
+                                                                        part, z);
     HD_CHECK_LAUNCH(ctx);
     return HD_OK;
 }
@@ -1995,8 +2059,8 @@ static int launch_dot(Engine& E, float2* part, const ColState* st) {
     hd_ctx* ctx = E.ctx;
     HD_PROF(ctx, "dot");
     const RedLaunch l = red_launch(E);
-    if (l.staged) return launch_staged<RED_DOT>(E, l, E.P, part, st);
-    k_dot<<<l.grid, l.block, l.smem, ctx->stream>>>(E.P, E.Q, E.n, E.Bp, E.rch, part, st);
+    if (l.staged) return launch_staged<RED_DOT>(E, l, E.P, E.pv, part, st);
+    k_dot<<<l.grid, l.block, l.smem, ctx->stream>>>(E.P, E.pv, E.Q, E.n, E.Bp, E.rch, part, st);
     HD_CHECK_LAUNCH(ctx);
     return HD_OK;
 }
@@ -2012,8 +2076,9 @@ static int launch_update(Engine& E) {
         z.num_active = E.num_active;
         z.use_half = E.use_half;
     }
-    if (l.staged) return launch_staged<RED_UPDATE>(E, l, E.P, E.part, E.st, z);
-    k_update<<<l.grid, l.block, l.smem, ctx->stream>>>(E.X, E.R, E.P, E.Q, E.n, E.Bp, E.rch, E.st, E.xs, E.part, z);
+    if (l.staged) return launch_staged<RED_UPDATE>(E, l, E.P, E.pv, E.part, E.st, z);
+    k_update<<<l.grid, l.block, l.smem, ctx->stream>>>(E.X, E.R, E.P, E.pv, E.Q, E.n, E.Bp, E.rch, E.st, E.xs, E.part,
+                                                      z);
     HD_CHECK_LAUNCH(ctx);
     return HD_OK;
 }
@@ -2022,7 +2087,7 @@ static int launch_colsq(Engine& E, const float* V) {
     hd_ctx* ctx = E.ctx;
     HD_PROF(ctx, "colsq");
     const RedLaunch l = red_launch(E);
-    if (l.staged) return launch_staged<RED_SQ>(E, l, V, E.part, nullptr);
+    if (l.staged) return launch_staged<RED_SQ>(E, l, V, panel_rows(E.n, E.Bp), E.part, nullptr);
     k_colsq<<<l.grid, l.block, l.smem, ctx->stream>>>(V, E.n, E.Bp, E.rch, E.part);
     HD_CHECK_LAUNCH(ctx);
     return HD_OK;
@@ -2045,25 +2110,32 @@ static int launch_spmm(Engine& E, float c1, float c2, float2* part, const ColSta
         const int nq = E.Bp / 4;
         const int rpb = 256 / nq;
         const dim3 gc((unsigned)std::min<int64_t>(ceil_div(E.n, rpb), (int64_t)ctx->num_sms * 8));
-        const int L16 = spmm_lanes(E.Bp, 8, spmm_exceeds_l2(E.n, E.Bp, 2));
-        const dim3 gh = spmm_grid(ctx, E.n, E.Bp, 8, L16, 7);
         {
             HD_PROF(ctx, "to_half");
-            k_colmax<<<gc, 256, 0, ctx->stream>>>(E.P, E.n, E.Bp, E.p16_max, E.use_half, E.num_active);
+            k_colmax<<<gc, 256, 0, ctx->stream>>>(E.P, E.pv, E.n, E.Bp, E.p16_max, E.use_half, E.num_active);
             HD_CHECK_LAUNCH(ctx);
-            k_to_half<<<gc, 256, 0, ctx->stream>>>(E.P, E.n, E.Bp, E.p16_max, E.P16, E.use_half, E.num_active);
+            k_to_half<<<gc, 256, 0, ctx->stream>>>(E.P, E.pv, E.n, E.Bp, E.p16_max, E.P16, E.hv, E.use_half,
+                                                 E.num_active);
             HD_CHECK_LAUNCH(ctx);
         }
         {
             HD_PROF(ctx, "spmm");
-            if ((rc = spmm_launch(ctx, g, E.P, E.Q, E.Bp, E.slab, c1, c2, st, E.use_half))) return rc;
+            if ((rc = spmm_launch(ctx, g, E.P, E.pv, E.Q, E.Bp, E.slab, c1, c2, st, E.use_half))) return rc;
         }
         {
             HD_PROF(ctx, "spmm_h");
-            HD_DISPATCH_L(L16, E.Bp / 8, (k_spmm_h<LC, G><<<gh, 128, 0, ctx->stream>>>(
-                                   g->row_ptr, g->col, g->val, E.P16, E.p16_max, E.P, E.Q, (unsigned)E.n, E.Bp, L16, c1,
-                                   c2, st, E.use_half)));
-            HD_CHECK_LAUNCH(ctx);
+            const int32_t cut = E.hv.wlast != E.hv.w ? E.hv.last : 0;
+            for (int32_t first = 0; first < E.Bp; first = first < cut ? cut : E.Bp) {
+                const int32_t last = first < cut ? cut : E.Bp;
+                const int L16 = cut && last == E.Bp ? (last - first) / 8
+                                : E.hv.last         ? E.hv.w / 8
+                                                    : spmm_lanes(E.Bp, 8, spmm_exceeds_l2(E.n, E.Bp, 2));
+                const dim3 gh = spmm_grid(ctx, E.n, last - first, 8, L16, 7);
+                HD_DISPATCH_L(L16, (last - first) / 8, (k_spmm_h<LC, G><<<gh, 128, 0, ctx->stream>>>(
+                                       g->row_ptr, g->col, g->val, E.P16, E.hv, E.p16_max, E.P, E.pv, E.Q,
+                                       (unsigned)E.n, E.Bp, first, last, L16, c1, c2, st, E.use_half)));
+                HD_CHECK_LAUNCH(ctx);
+            }
         }
         if (part) return launch_dot(E, part, st);
         return HD_OK;
@@ -2075,7 +2147,7 @@ static int launch_spmm(Engine& E, float c1, float c2, float2* part, const ColSta
             k_spmm_n4<<<g4, 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, Pin, E.Q, E.n, c1, c2, st, nullptr);
             HD_CHECK_LAUNCH(ctx);
         } else if (E.segK <= 1) {
-            if ((rc = spmm_launch(ctx, g, Pin, E.Q, E.Bp, E.slab, c1, c2, st, nullptr))) return rc;
+            if ((rc = spmm_launch(ctx, g, Pin, V ? panel_rows(E.n, E.Bp) : E.pv, E.Q, E.Bp, E.slab, c1, c2, st, nullptr))) return rc;
         } else {
             const dim3 grid(E.vl.nblk, E.vl.slabs);
             for (int s = 0; s < E.segK; ++s) {
@@ -2218,9 +2290,11 @@ int engine_iteration(Engine& S_, int (*after_update)(void*), void* arg) {
         z.use_half = S_.use_half;
         if ((rc = lr_finish(ctx, S_.lr, Bp, S_.dcoef, z))) return rc;
         if ((rc = launch_fin_rr(S_, Cd, S_.dcoef, r))) return rc;
-        if ((rc = lr_expand(ctx, S_.lr, EXP_DIRECTION, S_.P, S_.R, S_.P, n, Bp, S_.st, S_.num_active))) return rc;
+        if ((rc = lr_expand(ctx, S_.lr, EXP_DIRECTION, S_.P, S_.R, S_.P, n, Bp, S_.st, S_.num_active,
+                            &S_.pv)))
+            return rc;
         if (S_.refill) {
-            k_refill_p<<<ceil_div(Bp, 128), 128, 0, ctx->stream>>>(*S_.refill, S_.P, Bp);
+            k_refill_p<<<ceil_div(Bp, 128), 128, 0, ctx->stream>>>(*S_.refill, S_.P, S_.pv, Bp);
             HD_CHECK_LAUNCH(ctx);
         }
     } else {
@@ -2240,9 +2314,9 @@ int engine_iteration(Engine& S_, int (*after_update)(void*), void* arg) {
         if ((rc = launch_update(S_))) return rc;
     if (after_update && (rc = after_update(arg))) return rc;
         if ((rc = launch_fin_rr(S_, nullptr, nullptr, 0))) return rc;
-        LAUNCH_VEC(k_direction, S_.P, S_.R, n, Bp, S_.st);
+        LAUNCH_VEC(k_direction, S_.P, S_.pv, S_.R, n, Bp, S_.st);
         if (S_.refill) {
-            k_refill_p<<<ceil_div(Bp, 128), 128, 0, ctx->stream>>>(*S_.refill, S_.P, Bp);
+            k_refill_p<<<ceil_div(Bp, 128), 128, 0, ctx->stream>>>(*S_.refill, S_.P, S_.pv, Bp);
             HD_CHECK_LAUNCH(ctx);
         }
         if (lr_on) {
@@ -2276,7 +2350,7 @@ static std::vector<uint64_t> iteration_key(const Engine& E) {
             (uint64_t)E.lr.Hlo, (uint64_t)E.dcoef, (uint64_t)E.opcoef, (uint64_t)E.segK, (uint64_t)E.seg,
             (uint64_t)E.nch, (uint64_t)E.Bp, (uint64_t)E.slab, (uint64_t)E.vl.S, (uint64_t)E.vl.nblk, (uint64_t)E.vl.slabs,
             (uint64_t)E.lr.nchunk, (uint64_t)E.lr.rpad, (uint64_t)E.lr.Bp16, (uint64_t)E.has_lr,
-            (uint64_t)E.eff_mode, (uint64_t)E.r, (uint64_t)E.max_iter, fbits(E.c1), fbits(E.c2), fbits(E.xs),
+            (uint64_t)E.eff_mode, (uint64_t)E.r, (uint64_t)E.max_iter, fbits(E.c1), fbits(E.c2), fbits(E.xs), (uint64_t)E.pv.last, (uint64_t)E.hv.last,
             (uint64_t)E.P16, (uint64_t)E.p16_max, (uint64_t)E.use_half, (uint64_t)E.ctx->stream};
 }
 
@@ -2426,7 +2500,7 @@ static int true_residual(Engine& E, double alpha) {
             k_spmm_n4<<<std::max(1, ceil_div(n, N4_ROWS)), 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->val, E.X, E.Q,
                                                                                   n, -c1, -c2, nullptr, pick);
             HD_CHECK_LAUNCH(ctx);
-        } else if ((rc = spmm_launch(ctx, g, E.X, E.Q, Bp, E.slab, -c1, -c2, nullptr, pick))) {
+        } else if ((rc = spmm_launch(ctx, g, E.X, panel_rows(n, Bp), E.Q, Bp, E.slab, -c1, -c2, nullptr, pick))) {
             return rc;
         }
         const int L = std::max(1, E.slab / 4);
@@ -2470,7 +2544,7 @@ static int restart_columns(Engine& E) {
             k_fin_restart<<<Bp, 128, 0, ctx->stream>>>(E.st, E.lr.C, E.dcoef, E.r);
         }
         HD_CHECK_LAUNCH(ctx);
-        return lr_expand(ctx, E.lr, EXP_DIRECTION, E.P, E.R, E.P, n, Bp, E.st);
+        return lr_expand(ctx, E.lr, EXP_DIRECTION, E.P, E.R, E.P, n, Bp, E.st, nullptr, &E.pv);
     }
     {
         HD_PROF(ctx, "scalar");
@@ -2480,7 +2554,7 @@ static int restart_columns(Engine& E) {
     {
         HD_PROF(ctx, "direction");
         dim3 grid(E.vl.nblk, E.vl.slabs);
-        HD_DISPATCH_S(E.vl.S, (k_direction<SS><<<grid, 256, 0, ctx->stream>>>(E.P, E.R, n, Bp, E.st)));
+        HD_DISPATCH_S(E.vl.S, (k_direction<SS><<<grid, 256, 0, ctx->stream>>>(E.P, E.pv, E.R, n, Bp, E.st)));
         HD_CHECK_LAUNCH(ctx);
     }
     if (E.has_lr) {
@@ -2645,6 +2719,7 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         S_.slab = spmm_slab(g, Bp);
         if ((rc = spmm_segments(ctx, S_))) return rc;
     }
+    engine_set_panels(S_, lr_on ? mode : HD_MODE_PAPER);
     if (half_ok && S_.segK == 1 && !half_gathers_off()) {
         S_.P16 = p16;
         S_.p16_max = p16_max;
@@ -2675,7 +2750,10 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         k_fin_setup<<<Bp, 128, 0, ctx->stream>>>(S_.part, (int)S_.nch, Bp, B, (const float*)tl, S_.st, nullptr, nullptr,
                                                 0, S_.num_active);
         HD_CHECK_LAUNCH(ctx);
-        HD_CUDA(ctx, cudaMemcpyAsync(S_.P, S_.R, vec, cudaMemcpyDeviceToDevice, ctx->stream));
+        if (S_.pv.last)
+            LAUNCH_VEC(k_direction, S_.P, S_.pv, S_.R, n, Bp, S_.st);  // (beta is 0)
+        else
+            HD_CUDA(ctx, cudaMemcpyAsync(S_.P, S_.R, vec, cudaMemcpyDeviceToDevice, ctx->stream));
         if (lr_on) {
             // C = U^T y: kept for x^s = U g(Lambda) C (Eq. 18), and U^T P for the first operator
             if ((rc = lr_reduce(ctx, S_.lr, S_.R, n, Bp))) return rc;
@@ -2703,7 +2781,8 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
                                                 S_.num_active);
         HD_CHECK_LAUNCH(ctx);
         // (beta is 0: whatever P holds is dropped)
-        if ((rc = lr_expand(ctx, S_.lr, EXP_DIRECTION, S_.P, S_.R, S_.P, n, Bp, S_.st))) return rc;
+        if ((rc = lr_expand(ctx, S_.lr, EXP_DIRECTION, S_.P, S_.R, S_.P, n, Bp, S_.st, nullptr, &S_.pv)))
+            return rc;
     }
 
     // ---------------- iterations, then confirmation by the true residual

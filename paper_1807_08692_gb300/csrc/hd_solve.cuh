@@ -52,6 +52,22 @@ struct Refill {
 };
 constexpr int REFILL_MAX_NNZ = 512;
 
+// How P is laid out: columns p w .. p w + w - 1 of all n rows together (panel p, rows of
+// w columns), the last panel from column `last` on with rows of `wlast` columns.
+// last = 0: plain rows.
+struct Panels {
+    int64_t n = 0;
+    int32_t w = 32, last = 0, wlast = 0;   // w a power of two
+};
+inline Panels panel_rows(int64_t n, int32_t Bp) { return Panels{n, 32, 0, Bp}; }
+// column j of row 0, and the stride to its next row
+template <class T>
+__device__ __forceinline__ T* panel_column(const Panels& v, T* P, int j, int& stride) {
+    const int p0 = min(j & ~(v.w - 1), v.last);
+    stride = p0 == v.last ? v.wlast : v.w;
+    return P + (int64_t)p0 * v.n + (j - p0);
+}
+
 // Low-rank product helpers (storage-specific implementations).
 //  reduce: part[c][k][j] = sum over rows of chunk c of U[i][k] * V[i][j]
 //  expand: out = f(U H) for each row (see ExpandOp)
@@ -89,7 +105,7 @@ struct IterReset {
 int lr_reduce(hd_ctx* ctx, const LowRank& lr, const float* V, int64_t n, int32_t Bp, const int* gate = nullptr);
 int lr_finish(hd_ctx* ctx, const LowRank& lr, int32_t Bp, const double* coef, const IterReset& z = {});
 int lr_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float* Rv, const float* Pv, int64_t n,
-              int32_t Bp, const ColState* st, const int* gate = nullptr);
+              int32_t Bp, const ColState* st, const int* gate = nullptr, const Panels* pv = nullptr);
 bool lr_use_tensor_cores(const hd_eig* e);
 // HD_ERR_TIMEOUT (flags cleared) if a tensor-core kernel gave up a bounded wait
 // since the last check; synchronises the context's stream
@@ -102,7 +118,7 @@ int lr_sparse_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const f
                      int32_t Bp, const ColState* st, const int* gate);
 int lr_tc_reduce(hd_ctx* ctx, const LowRank& lr, const float* V, int64_t n, int32_t Bp, const int* gate);
 int lr_tc_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float* Rv, const float* Pv, int64_t n,
-                 int32_t Bp, const ColState* st, const int* gate);
+                 int32_t Bp, const ColState* st, const int* gate, const Panels* pv);
 int lr_tc_nchunk(hd_ctx* ctx, int64_t n);
 
 // ------------------------------------------------------------------ iteration engine
@@ -139,6 +155,7 @@ struct Engine {
     // k_spmm's; the server keeps one order at every lane width)
     bool narrow4 = true;
     float *R = nullptr, *P = nullptr, *Q = nullptr, *X = nullptr;
+    Panels pv, hv;              // layouts of P and P16 (engine_set_panels)
     float* VT = nullptr;        // truncated systems: the transposed operand of their products [Bp][n]
     float2* part = nullptr;
     ColState* st = nullptr;
@@ -171,6 +188,8 @@ struct Engine {
 VecLaunch vec_launch(hd_ctx* ctx, int64_t n, int32_t Bp, int S = 0);
 // Column-slab width of the SpMM for this graph and batch width (HD_SLAB caps it).
 int spmm_slab(const hd_graph* g, int32_t Bp);
+// Layouts of P and P16 for this solve (n, Bp, slab, ts, segK and the eigenpairs set).
+void engine_set_panels(Engine& E, int eff_mode);
 int simt_nchunk(hd_ctx* ctx, int64_t n, int rpad, int Bp);
 // Node-range segments for the SpMM: one pass unless HD_SEGMENTS asks for more;
 // sets E.segK / E.seg.
