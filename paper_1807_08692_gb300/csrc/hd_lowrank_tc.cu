@@ -99,6 +99,11 @@ struct ExpandArgs {
                     // reads U block kb (kb < nkb_b) or kb + a_off (the lo half) and H block kb mod nkb_b
     int32_t a_off;
     int32_t op;
+    int32_t alt;    // 1: the two warps of a TMEM lane quarter take alternate tiles, else halves of the columns.
+                    // For at most 32 columns: half of a 16-column tile is nobody's, and the epilogue's
+                    // chain of load, wait, store per tile is what a launch waits for.  Alternating, 1M rows x 1
+                    // column take 66 us against 101 with 128 eigenvectors and 83 against 104 with 192; with
+                    // 200 (a fourth, nearly empty block per row: bound by TMA's rows) 102 against 106.
     uint32_t tmem_cols;
     float* out;
     const float* R;
@@ -152,7 +157,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
         tc::mbar_init(bfull, 1);
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&acc_full[b], 1);
-            tc::mbar_init(&acc_empty[b], EPI);
+            tc::mbar_init(&acc_empty[b], a.alt ? EPI / 2 : EPI);
         }
         tc::mbar_init(drain, 1);
         *abort_flag = 0;
@@ -289,7 +294,8 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
         const int rloc = quarter * 32 + lane;
         const int nch = a.Nc / 16;
         const int nh = (nch + 1) / 2;
-        const int cb = half ? nh : 0, ce = half ? nch : nh;
+        const int cb = half && !a.alt ? nh : 0, ce = half || a.alt ? nch : nh;
+        const int tstep = a.alt ? 2 : 1;  // tiles from one of this warp's to the next
         const int sr = lane >> 3, ch = lane & 7;  // global-side mapping: row offset, 16-byte column chunk
         float4* stg = reinterpret_cast<float4*>(stage) + (warp - 2) * 256;  // 32 rows x 8 chunks
         float4 g1[8], g2[8];
@@ -311,10 +317,11 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                 }
             }
         };
-        if ((int)blockIdx.x < ntiles && cb < ce) load_ops(blockIdx.x, cb);
-        uint32_t tcount = 0;
+        uint32_t tcount = a.alt ? half : 0;
+        const int tfirst = blockIdx.x + tcount * gridDim.x;
+        if (tfirst < ntiles && cb < ce) load_ops(tfirst, cb);
         bool ok = true;
-        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
+        for (int t = tfirst; t < ntiles && ok; t += tstep * gridDim.x, tcount += tstep) {
             const int ab = tcount & 1;
             const int64_t row = (int64_t)t * BM + rloc;
             const float rsc = (SU && row < a.n) ? __ldg(a.scale + row) : 1.0f;
@@ -389,7 +396,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
             }
             tc::fence_before_sync();
             tc::mbar_arrive(&acc_empty[ab]);
-            const int tn = t + gridDim.x;
+            const int tn = t + tstep * gridDim.x;
             if (tn < ntiles && cb < ce) load_ops(tn, cb);
         }
         if (!ok) {
@@ -778,6 +785,7 @@ int lr_tc_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float
         a.nkb_b = nkb_b;
         a.a_off = a_off;
         a.op = op;
+        a.alt = nc <= 32;
         a.tmem_cols = tmem_cols_for(2 * nc);
         a.out = out;
         a.R = Rv;

@@ -64,3 +64,25 @@ def test_eig_roundtrip_storage(gpu_ctx):
     # e4m3 keeps 3 mantissa bits: relative error <= 2^-4 of the row scale
     scale = np.abs(U).max(axis=1, keepdims=True)
     assert np.all(np.abs(U8 - U) <= scale * 2.0 ** -4 + 1e-12)
+
+
+@pytest.mark.parametrize("storage", ["bf16", "f32", "fp8"])
+@pytest.mark.parametrize("r,B", [(24, 4), (130, 16), (70, 20), (200, 32), (70, 36), (200, 100), (200, 128)])
+def test_expand_over_many_tiles(gpu_ctx, storage, r, B):
+    # several 128-row tiles per block (the last one short) at every division of
+    # the columns among the epilogue's warps; the bound is that of the test above
+    import ctypes as C
+    import torch
+    import paper_1807_08692_gb300 as hd
+    from paper_1807_08692_gb300.hd import lib
+    n = 78001
+    gen = torch.Generator(device="cuda").manual_seed(r + B)
+    U = torch.randn((n, r), generator=gen, device="cuda") / n ** 0.5
+    eig = hd.eig_from_host(gpu_ctx, _graph(gpu_ctx, n), np.linspace(1.0, 0.1, r), U.cpu().numpy(), storage)
+    Uq = torch.from_numpy(np.asarray(eig.export()[1])).cuda().double()
+    H = np.random.default_rng(B).standard_normal((r, B))
+    Xd = torch.empty((n, B), dtype=torch.float32, device="cuda")
+    gpu_ctx.check(lib().hd_eig_expand(gpu_ctx.handle, eig.handle, H.ctypes.data_as(C.c_void_p), B,
+                                      C.c_void_p(Xd.data_ptr())), "expand")
+    ref = Uq @ torch.from_numpy(H).cuda()
+    assert float((Xd.double() - ref).norm() / ref.norm()) <= 2e-5
