@@ -309,9 +309,10 @@ __global__ void __launch_bounds__(128, spmm_blocks(LC)) k_spmm(const int32_t* __
     if (r.idle) return;
     const bool own_col = LC || c0 + 4 * r.g < last;
     const int col = own_col ? c0 + 4 * r.g : last - 4;
-    int pw;
-    const float* Pc = panel_column(pv, P, col, pw);
-    auto load = [&](int32_t j) { return ld4(Pc + (int64_t)j * pw); };
+    // (LC = 0: plain rows or the last panel, one stride for all, taken from the arguments)
+    int pw = pv.wlast;
+    const float* Pc = LC ? panel_column(pv, P, col, pw) : P + first * pv.n + (col - first);
+    auto load = [&](int32_t j) { return ld4(Pc + (int64_t)j * (LC ? pw : pv.wlast)); };
     for (unsigned row = r.row; row < n; row += r.step) {
         const unsigned b = __ldg(rp + row), e = __ldg(rp + row + 1);
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(128, spmm_blocks(LC)) k_spmm(const int32_t* __
         s.y += s2.y;
         s.z += s2.z;
         s.w += s2.w;
-        const float4 own = ld4(Pc + (int64_t)row * pw);
+        const float4 own = ld4(Pc + (int64_t)row * (LC ? pw : pv.wlast));
         float4 q;
         q.x = c1 * own.x - c2 * s.x;
         q.y = c1 * own.y - c2 * s.y;
@@ -511,17 +512,18 @@ __global__ void __launch_bounds__(128, 7) k_spmm_h(const int32_t* __restrict__ r
     const int c0 = first + blockIdx.y * 8 * Lq, ce = min(last, c0 + 8 * Lq);
     // up to 256 columns of a slab against 128 threads
     if (!columns_have_work(st, c0, min(ce, c0 + 128)) && !columns_have_work(st, c0 + 128, ce)) return;
+    // the scales wait in shared memory: in registers they cost gathers in flight
+    __shared__ __align__(16) float inv[256];
+    for (int c = c0 + threadIdx.x; c < ce; c += blockDim.x) inv[c - c0] = half_scale(mx[c], true);
+    __syncthreads();
     const RowLanes r = row_lanes<LC>(L_);
     if (r.idle) return;
     const bool own_col = LC || c0 + 8 * r.g < last;
     const int col = own_col ? c0 + 8 * r.g : last - 8;
-    int pw, hw;
+    int pw, hw = hv.wlast;
     const float* Po = panel_column(pv, P, col, pw);
-    const __half* Pc = panel_column(hv, P16, col, hw);
-    float inv[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) inv[c] = half_scale(mx[col + c], true);
-    auto load = [&](int32_t j) { return __ldg(reinterpret_cast<const uint4*>(Pc + (int64_t)j * hw)); };
+    const __half* Pc = LC ? panel_column(hv, P16, col, hw) : P16 + first * hv.n + (col - first);
+    auto load = [&](int32_t j) { return __ldg(reinterpret_cast<const uint4*>(Pc + (int64_t)j * (LC ? hw : hv.wlast))); };
     for (unsigned row = r.row; row < n; row += r.step) {
         const unsigned b = __ldg(rp + row), e = __ldg(rp + row + 1);
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -530,10 +532,13 @@ __global__ void __launch_bounds__(128, 7) k_spmm_h(const int32_t* __restrict__ r
             [&](float w, const uint4& v) { FMA8H(acc, w, v); });
         const float* po = Po + (int64_t)row * pw;
         const float4 o0 = ld4(po), o1 = ld4(po + 4);
+        const float4 i0 = *reinterpret_cast<const float4*>(inv + (col - c0));
+        const float4 i1 = *reinterpret_cast<const float4*>(inv + (col - c0) + 4);
+        const float iv[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
         const float own[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
         float q[8];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) q[c] = c1 * own[c] - c2 * (acc[c] * inv[c]);
+        for (int c = 0; c < 8; ++c) q[c] = c1 * own[c] - c2 * (acc[c] * iv[c]);
         if (own_col) {
             float* qo = Q + (int64_t)row * ld + col;
             st4s(qo, make_float4(q[0], q[1], q[2], q[3]));
