@@ -28,6 +28,7 @@ namespace {
 constexpr int BM = 128;           // rows of U per tile
 constexpr int BK = 64;            // bf16 elements per 128-byte swizzle row
 constexpr int XSTAGES = 6;
+constexpr int XMIN = 4;           // stages a wide expansion gets by with
 constexpr int RSTAGES = 3;
 constexpr int THREADS = 320;      // warp 0: TMA, warp 1: MMA, warps 2-9: epilogue / conversion
 constexpr int EPI = 256;          // epilogue threads: two warps per TMEM lane quarter, splitting the columns
@@ -104,6 +105,7 @@ struct ExpandArgs {
                     // chain of load, wait, store per tile is what a launch waits for.  Alternating, 1M rows x 1
                     // column take 66 us against 101 with 128 eigenvectors and 83 against 104 with 192; with
                     // 200 (a fourth, nearly empty block per row: bound by TMA's rows) 102 against 106.
+    uint32_t stages;  // stages of the U pipeline (XMIN .. XSTAGES)
     uint32_t tmem_cols;
     float* out;
     const float* R;
@@ -124,10 +126,11 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t btile = (uint32_t)a.Nc * 128;  // one k-block of H^T (Nc rows x 128 B)
-    constexpr int NA = SU ? CSTAGES : XSTAGES;    // bf16 A stages the MMA reads
+    const uint32_t xst = a.stages;
+    const uint32_t NA = SU ? CSTAGES : xst;       // bf16 A stages the MMA reads
     uint8_t* As = smem;
     uint8_t* Raw = As + NA * TILE_BYTES;          // raw fp8 stages (SU only)
-    uint8_t* Bhi = Raw + (SU ? XSTAGES * RAW_X : 0);
+    uint8_t* Bhi = Raw + (SU ? xst * RAW_X : 0);
     uint8_t* Blo = Bhi + a.nkb_b * btile;
     float* stage = reinterpret_cast<float*>(Blo + a.nkb_b * btile);  // epilogue transposition, 4 KB per warp
     uint64_t* bars = (uint64_t*)(reinterpret_cast<uint8_t*>(stage) + STAGE_BYTES);
@@ -180,8 +183,8 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
             }
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
                 for (int kb = 0; kb < a.nkb; ++kb, ++it) {
-                    const int s = it % XSTAGES;
-                    if (!tc::mbar_wait(&empty[s], ((it / XSTAGES) & 1) ^ 1, abort_flag)) {
+                    const int s = it % xst;
+                    if (!tc::mbar_wait(&empty[s], ((it / xst) & 1) ^ 1, abort_flag)) {
                         ok = false;
                         break;
                     }
@@ -199,9 +202,9 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                 atomicExch(err, 11);
             }
             tc::mbar_wait(bfull, 0, nullptr, 200000000ull);
-            for (uint32_t j = 0; j < (uint32_t)XSTAGES && j < it; ++j) {
+            for (uint32_t j = 0; j < xst && j < it; ++j) {
                 const uint32_t last = it - 1 - j;
-                tc::mbar_wait(&full[last % XSTAGES], (last / XSTAGES) & 1, nullptr, 200000000ull);
+                tc::mbar_wait(&full[last % xst], (last / xst) & 1, nullptr, 200000000ull);
             }
         }
     } else if (warp == 1) {
@@ -218,9 +221,9 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                 tc::fence_after_sync();
                 const uint32_t dt = tmem + ab * a.Nc;
                 for (int kb = 0; kb < a.nkb; ++kb, ++it) {
-                    const int s = SU ? it % CSTAGES : it % XSTAGES;
+                    const int s = SU ? it % CSTAGES : it % xst;
                     uint64_t* fb = SU ? &cfull[s] : &full[s];
-                    if (!tc::mbar_wait(fb, (SU ? it / CSTAGES : it / XSTAGES) & 1, abort_flag)) {
+                    if (!tc::mbar_wait(fb, (SU ? it / CSTAGES : it / xst) & 1, abort_flag)) {
                         ok = false;
                         break;
                     }
@@ -254,8 +257,8 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
         bool ok = true;
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
             for (int kb = 0; kb < a.nkb; ++kb, ++it) {
-                const int s = it % XSTAGES, s2 = it % CSTAGES;
-                if (!tc::mbar_wait(&full[s], (it / XSTAGES) & 1, abort_flag) ||
+                const int s = it % xst, s2 = it % CSTAGES;
+                if (!tc::mbar_wait(&full[s], (it / xst) & 1, abort_flag) ||
                     !tc::mbar_wait(&cempty[s2], ((it / CSTAGES) & 1) ^ 1, abort_flag)) {
                     ok = false;
                     break;
@@ -758,13 +761,25 @@ int lr_tc_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float
         return hd_fail(ctx, HD_ERR_CUDA, "tensor map for U failed");
     // column chunks so that H^T (hi + lo) fits next to the A pipeline
     const int max_smem = 227 * 1024 - 2048;
-    const int apipe = su ? CSTAGES * TILE_BYTES + XSTAGES * RAW_X : XSTAGES * TILE_BYTES;
+    const int stage = su ? RAW_X : TILE_BYTES, conv = su ? CSTAGES * TILE_BYTES : 0;
+    auto smem_of = [&](int nc, int ns) { return conv + ns * stage + STAGE_BYTES + 2 * nkb_b * nc * 128; };
     // columns that can be active (the server's occupied slots); the rest keep their values
     const int cols = lr.live > 0 ? std::min(lr.Bp16, (lr.live + 15) / 16 * 16) : lr.Bp16;
-    int Nc = cols;
-    while (Nc > 16 && (apipe + STAGE_BYTES + 2 * nkb_b * Nc * 128 > max_smem || Nc > 256)) Nc = (Nc / 2 + 15) / 16 * 16;
-    if (apipe + STAGE_BYTES + 2 * nkb_b * Nc * 128 > max_smem)
+    if (smem_of(16, XSTAGES) > max_smem)
         return hd_fail(ctx, HD_ERR_INVALID_ARG, "rank %d too large for the tensor-core expansion", e->r);
+    // the fewest launches (each reads all of U) that leave room for four stages; halves
+    // at six stages where four launches do not do
+    int ns = XSTAGES, Nc = 0;
+    for (int parts = 1; !Nc && parts <= 4; ++parts) {
+        const int c = (ceil_div(cols, parts) + 15) / 16 * 16;
+        if (c <= 256 && smem_of(c, XMIN) <= max_smem) Nc = c;
+    }
+    if (!Nc) {
+        Nc = cols;
+        while (Nc > 16 && (smem_of(Nc, XSTAGES) > max_smem || Nc > 256)) Nc = (Nc / 2 + 15) / 16 * 16;
+    }
+    while (ns > XMIN && smem_of(Nc, ns) > max_smem) --ns;
+    const int apipe = conv + ns * stage;
     static uint64_t attr[2] = {0, 0};
     if (hd_first_on_device(attr[su], ctx->device)) {
         HD_CUDA(ctx, cudaFuncSetAttribute(su ? k_lr_expand_tc<1> : k_lr_expand_tc<0>,
@@ -785,6 +800,7 @@ int lr_tc_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float
         a.nkb_b = nkb_b;
         a.a_off = a_off;
         a.op = op;
+        a.stages = ns;
         a.alt = nc <= 32;
         a.tmem_cols = tmem_cols_for(2 * nc);
         a.out = out;
