@@ -768,7 +768,9 @@ int lr_tc_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float
     if (smem_of(16, XSTAGES) > max_smem)
         return hd_fail(ctx, HD_ERR_INVALID_ARG, "rank %d too large for the tensor-core expansion", e->r);
     // the fewest launches (each reads all of U) that leave room for four stages; halves
-    // at six stages where four launches do not do
+    // at six stages where four launches do not do.  1M rows, 128 columns x 200 eigenvectors:
+    // 309 us in one launch of four stages, 331 in two of six; 64 x 400: 213 against 341
+    // in two of 32 columns
     int ns = XSTAGES, Nc = 0;
     for (int parts = 1; !Nc && parts <= 4; ++parts) {
         const int c = (ceil_div(cols, parts) + 15) / 16 * 16;

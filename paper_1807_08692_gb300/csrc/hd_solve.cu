@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(256) k_to_half(const float* __restrict__ P, co
 // Q = c1 P - c2 W P with the W P gathers from the fp16 copy (L lanes x 8
 // columns per slab: a row's slab of 64 columns is one 128-byte line); the sums
 // are fp32, unscaled by the column's power of two at the end.  Runs when
-// *use_half is set.  0.75 ms for a 1M x 64 product (0.82 ms with private index
+// *use_half is set.  0.74 ms for a 1M x 64 product (0.82 ms with private index
 // copies); 0.06 ms against 0.16 ms for 100,000 x 40, which took 8-column slabs.
 template <int LC, int G>
 __global__ void __launch_bounds__(128, 7) k_spmm_h(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
@@ -1930,7 +1930,7 @@ VecLaunch vec_launch(hd_ctx* ctx, int64_t n, int32_t Bp, int S) {
 // (1M nodes, 64 columns: 1.18 ms against 1.50 ms).  16 lanes when the block fits
 // in L2 (100,000 x 64: 0.082 ms against 0.086 ms), and from 256 columns on, where
 // the 128-byte lines of one pass lie 1 KB apart (1M x 256: 6.1 ms against 6.7;
-// panels, see panels_for, take 5.2).
+// panels, see panels_for, take 4.8).
 // Other widths take the whole row at once up to 16 lanes, else the fewest even
 // parts of at most 16: 100,000 x 40 runs in 0.067 ms with 10 lanes, 0.12 ms in
 // two passes of 9 and 0.174 ms in five of 2.
