@@ -3,6 +3,7 @@
 // Layout: every n x B block (R, P, Q, X) is row-major with a padded width Bp
 // (B rounded up to a multiple of 4) so that one gathered row of P is Bp
 // contiguous fp32 values: a group of Bp/4 lanes moves it with float4 loads.
+// P alone may be kept in panels of a 128-byte line instead (Panels, panels_for).
 //
 // One CG iteration for B columns at once (per-column scalars in fp64):
 //   Q = c1 P - c2 W P [+ U (c3 Lambda o (U^T P))]                 Eq. 20
