@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
 
     if (warp == 0) {
         if (lane == 0) {
-            uint32_t it = 0;
+            uint32_t it = 0, s = 0, ph = 0;  // k-blocks so far, their stage and the parity of its use
             bool ok = true;
             tc::mbar_arrive_expect_tx(bfull, 2u * a.nkb_b * btile);
             for (int kb = 0; kb < a.nkb_b; ++kb) {
@@ -183,8 +183,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
             }
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
                 for (int kb = 0; kb < a.nkb; ++kb, ++it) {
-                    const int s = it % xst;
-                    if (!tc::mbar_wait(&empty[s], ((it / xst) & 1) ^ 1, abort_flag)) {
+                    if (!tc::mbar_wait(&empty[s], ph ^ 1, abort_flag)) {
                         ok = false;
                         break;
                     }
@@ -196,6 +195,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                         tc::tma_load_2d(As + s * TILE_BYTES, &tmU, &full[s], (kb < a.nkb_b ? kb : kb + a.a_off) * BK,
                                         t * BM);
                     }
+                    if (++s == xst) s = 0, ph ^= 1;
                 }
             if (!ok) {
                 *abort_flag = 1;
@@ -211,7 +211,8 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
         if (lane == 0) {
             const uint32_t idesc = tc::idesc_bf16(BM, a.Nc, 0, 0);
             bool ok = tc::mbar_wait(bfull, 0, abort_flag);
-            uint32_t it = 0, tcount = 0;
+            const uint32_t nst = SU ? CSTAGES : xst;
+            uint32_t s = 0, ph = 0, tcount = 0;
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
                 const int ab = tcount & 1;
                 if (!tc::mbar_wait(&acc_empty[ab], ((tcount >> 1) & 1) ^ 1, abort_flag)) {
@@ -220,10 +221,9 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                 }
                 tc::fence_after_sync();
                 const uint32_t dt = tmem + ab * a.Nc;
-                for (int kb = 0; kb < a.nkb; ++kb, ++it) {
-                    const int s = SU ? it % CSTAGES : it % xst;
+                for (int kb = 0; kb < a.nkb; ++kb) {
                     uint64_t* fb = SU ? &cfull[s] : &full[s];
-                    if (!tc::mbar_wait(fb, (SU ? it / CSTAGES : it / xst) & 1, abort_flag)) {
+                    if (!tc::mbar_wait(fb, ph, abort_flag)) {
                         ok = false;
                         break;
                     }
@@ -240,6 +240,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                         tc::mma_bf16(dt, ad, tc::smem_desc(bl + kk * 32, 16, 1024, tc::SWIZZLE_128B), idesc, 1u);
                     }
                     tc::mma_commit(SU ? &cempty[s] : &empty[s]);
+                    if (++s == nst) s = 0, ph ^= 1;
                 }
                 if (ok) tc::mma_commit(&acc_full[ab]);
             }
@@ -253,12 +254,12 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
     } else if (SU && warp >= THREADS / 32) {
         // converters: raw 128 x 64 code tile -> bf16 128 x 128 B rows, 128-byte swizzle
         const int ct = threadIdx.x - THREADS;
-        uint32_t it = 0;
+        uint32_t it = 0, s = 0, ph = 0;
         bool ok = true;
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
             for (int kb = 0; kb < a.nkb; ++kb, ++it) {
-                const int s = it % xst, s2 = it % CSTAGES;
-                if (!tc::mbar_wait(&full[s], (it / xst) & 1, abort_flag) ||
+                const int s2 = it % CSTAGES;
+                if (!tc::mbar_wait(&full[s], ph, abort_flag) ||
                     !tc::mbar_wait(&cempty[s2], ((it / CSTAGES) & 1) ^ 1, abort_flag)) {
                     ok = false;
                     break;
@@ -277,6 +278,7 @@ __global__ void __launch_bounds__(THREADS + (SU ? CONV : 0), 1)
                 tc::fence_proxy_async_smem();
                 tc::mbar_arrive(&cfull[s2]);
                 tc::mbar_arrive(&empty[s]);
+                if (++s == xst) s = 0, ph ^= 1;
             }
         if (!ok) {
             *abort_flag = 1;
