@@ -324,18 +324,18 @@ def e2e_leg(ctx, wl, eig, mode, tol, alpha, K, B, topk):
 
 
 # DRAM bytes per launch of the SpMM measured by ncu (the SpMM summary under profiles/):
-# k_spmm<32> on a 1M-node k=50 graph (d=256 descriptors, nnz 62,097,728), B=64.
+# k_spmm<8, 8> (32-column slabs) on a 1M-node k=50 graph (d=256 descriptors, nnz 62,097,728), B=64.
 # Scaled to another graph by nnz (the gathered rows dominate); reported only
 # while the kernel source still hashes to the value the counters were taken on.
-SPMM_NCU = {"dram_bytes": 8468885888, "nnz": 62097728, "n": 1000000, "B": 64, "slab": 32,
-            "src_sha1": "b0a31b960a82f4637d356dc47bf415d4c28ca76d"}
+SPMM_NCU = {"dram_bytes": 8031695872, "nnz": 62097728, "n": 1000000, "B": 64, "slab": 32,
+            "src_sha1": "b1bcfcf584ac6e8129cdee20fa39cb6769a41a03"}
 
 
 def spmm_source_sha1():
     import hashlib
     src = open(os.path.join(ROOT, "paper_1807_08692_gb300", "csrc", "hd_solve.cu")).read()
-    a = src.index("k_spmm(const int32_t* rp,")
-    b = src.index("\n}\n", a)
+    a = src.index("void row_entries(")
+    b = src.index("\n}\n", src.index("k_spmm(const int32_t* __restrict__ rp,", a))
     return hashlib.sha1(src[a:b].encode()).hexdigest()
 
 
