@@ -642,8 +642,9 @@ __global__ void __launch_bounds__(knntc::THREADS, 1)
                 take64(x0, x1, other[r * 64 + lane], other[r * 64 + lane + 32], lane);
                 knn_store(a, seg, row0 + r, x0, x1, lane);
             }
-            asm volatile("bar.sync 1, %0;" ::"n"(EPI) : "memory");
-            ok = ok && !*abort_flag;  // an epilogue warp that gave up ends the others' loops with its own
+            // one answer for all eight warps: the flag may rise between two warps' reads of
+            // it, and a warp that went on alone would wait at the next barrier for ever
+            ok = !tc::bar_any<1, EPI>(!ok || *abort_flag);
         }
     }
     tc::fence_before_sync();

@@ -58,6 +58,22 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     }
 }
 
+// Named barrier ID of THREADS threads that also tells each of them whether any
+// came with `p` set.
+template <int ID, int THREADS>
+__device__ __forceinline__ bool bar_any(bool p) {
+    uint32_t any;
+    asm volatile(
+        "{\n .reg .pred p, q;\n"
+        " setp.ne.u32 p, %3, 0;\n"
+        " barrier.cta.red.or.pred q, %1, %2, p;\n"
+        " selp.u32 %0, 1, 0, q;\n}"
+        : "=r"(any)
+        : "n"(ID), "n"(THREADS), "r"((uint32_t)p)
+        : "memory");
+    return any != 0;
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int32_t c0,
                                             int32_t c1) {
