@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 #include <stdint.h>
+#include <atomic>
 #include <map>
 #include <string>
 #include <utility>
@@ -73,7 +74,16 @@ struct ProfScope {
 #define HD_CAT(a, b) HD_CAT2(a, b)
 #define HD_PROF(ctx, name) ProfScope HD_CAT(hd_prof_scope_, __LINE__)((ctx), (name))
 
+// A number that no other graph or set of eigenpairs of this process has, now or
+// later: their arrays never change or move after creation, so captured kernels
+// may be kept by it.  Addresses will not do, the next object may get them again.
+inline uint64_t hd_new_id() {
+    static std::atomic<uint64_t> last{0};
+    return ++last;
+}
+
 struct hd_graph {
+    const uint64_t id = hd_new_id();
     int64_t n = 0, nnz = 0;
     int device = 0;
     int32_t* row_ptr = nullptr;
@@ -93,6 +103,7 @@ struct hd_graph {
 };
 
 struct hd_eig {
+    const uint64_t id = hd_new_id();
     int64_t n = 0;
     int32_t r = 0;
     int32_t ldu = 0;          // leading dimension of U in elements (multiple of 16)

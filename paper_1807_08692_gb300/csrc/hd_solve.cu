@@ -2344,13 +2344,11 @@ static uint64_t fbits(float f) {
 }
 
 // Everything the iteration kernels take as arguments (the run length is added
-// by the caller).
+// by the caller); the graph's and the eigenpairs' ids stand for all their arrays.
 static std::vector<uint64_t> iteration_key(const Engine& E) {
-    return {(uint64_t)E.g, (uint64_t)E.ts, (uint64_t)(E.ts ? E.ts->off : nullptr), (uint64_t)(E.ts ? E.ts->ci : nullptr),
-            (uint64_t)(E.ts ? E.ts->wv : nullptr), (uint64_t)(E.ts ? E.ts->B : 0), (uint64_t)E.g->row_ptr,
-            (uint64_t)E.g->col, (uint64_t)E.g->val, (uint64_t)E.n, (uint64_t)E.lr.e,
-            (uint64_t)(E.has_lr ? E.lr.e->U : nullptr), (uint64_t)(E.has_lr ? E.lr.e->storage : -1),
-            (uint64_t)(E.has_lr ? E.lr.e->sp_rp : nullptr), (uint64_t)(E.has_lr ? E.lr.e->sp_cp : nullptr),
+    return {E.g->id, E.has_lr ? E.lr.e->id : 0, (uint64_t)E.ts, (uint64_t)(E.ts ? E.ts->off : nullptr),
+            (uint64_t)(E.ts ? E.ts->ci : nullptr), (uint64_t)(E.ts ? E.ts->wv : nullptr),
+            (uint64_t)(E.ts ? E.ts->B : 0), (uint64_t)E.n,
             (uint64_t)E.R, (uint64_t)E.P, (uint64_t)E.Q, (uint64_t)E.X, (uint64_t)E.VT, (uint64_t)E.part, (uint64_t)E.st,
             (uint64_t)E.num_active, (uint64_t)E.lr.part, (uint64_t)E.lr.C, (uint64_t)E.lr.H, (uint64_t)E.lr.Hhi,
             (uint64_t)E.lr.Hlo, (uint64_t)E.dcoef, (uint64_t)E.opcoef, (uint64_t)E.segK, (uint64_t)E.seg,
