@@ -89,8 +89,10 @@ int hd_destroy(hd_ctx* ctx);
 const char* hd_last_error(const hd_ctx* ctx);
 /* Number of library kernel launches issued on this context so far. */
 int64_t hd_launch_count(const hd_ctx* ctx);
-/* Bytes of device workspace the context currently holds (grown on demand by
- * the calls that need scratch, released by hd_destroy). */
+/* Bytes of device workspace the context currently holds: the block that the
+ * calls needing scratch grow on demand, and up to 1 GiB each of two blocks that
+ * hd_build_graph and hd_temporal_truncated keep for the next call (larger ones
+ * are given back when the call ends).  Released by hd_destroy. */
 int hd_workspace_bytes(const hd_ctx* ctx, size_t* bytes);
 /* Number of streaming multiprocessors of the context's device. */
 int hd_num_sms(const hd_ctx* ctx);
@@ -264,9 +266,10 @@ int hd_eig_expand(hd_ctx* ctx, const hd_eig* e, const double* H, int32_t B, floa
  *             X[t][j] is the score of sl_idx[sl_ptr[j] + t]; rows t >= s_j
  *             are 0.
  *  tol, max_iter, iters, relres, status : as for hd_query_batch.
- * The position maps (about B n 8 bytes) and the B subsystems take two device
- * blocks that the context keeps for the next call (up to 4 GiB each).  Errors: HD_ERR_INVALID_ARG for a bad
- * or duplicated shortlist id or observation index, HD_ERR_OOM. */
+ * Besides the B subsystems the call takes a bitmap of B n / 8 bytes and position
+ * maps of min(B n, max(64M, n)) 8 bytes (see hd_workspace_bytes).  Errors:
+ * HD_ERR_INVALID_ARG for a bad or duplicated shortlist id or observation index,
+ * HD_ERR_OOM. */
 int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, const int32_t* sl_ptr,
                           const int32_t* sl_idx, const int32_t* y_ptr, const int32_t* y_idx,
                           const float* y_val, double alpha, const float* tol, int32_t max_iter,

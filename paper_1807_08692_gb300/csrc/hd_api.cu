@@ -1,4 +1,5 @@
 // Context, memory staging, graph and eigenpair handles of the C ABI (include/hd.h).
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -40,7 +41,7 @@ bool hd_is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-static int reserve_block(hd_ctx* ctx, void** block, size_t* have, size_t bytes, void** out) {
+static int reserve_block(hd_ctx* ctx, void** block, size_t* have, size_t bytes, size_t slack, void** out) {
     if (bytes == 0) bytes = 256;
     if (bytes > *have) {
         if (*block) {
@@ -49,8 +50,13 @@ static int reserve_block(hd_ctx* ctx, void** block, size_t* have, size_t bytes, 
             *block = nullptr;
             *have = 0;
         }
-        size_t want = bytes + bytes / 8;
+        size_t want = bytes + slack;
         cudaError_t e = cudaMalloc(block, want);
+        if (e != cudaSuccess) {  // without room to grow, then
+            cudaGetLastError();
+            want = bytes;
+            e = cudaMalloc(block, want);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             *block = nullptr;
@@ -63,18 +69,21 @@ static int reserve_block(hd_ctx* ctx, void** block, size_t* have, size_t bytes, 
 }
 
 int hd_ws_reserve(hd_ctx* ctx, size_t bytes, void** out) {
-    return reserve_block(ctx, &ctx->ws, &ctx->ws_bytes, bytes, out);
+    return reserve_block(ctx, &ctx->ws, &ctx->ws_bytes, bytes, bytes / 8, out);
 }
 
 int hd_aux_reserve(hd_ctx* ctx, int which, size_t bytes, void** out) {
-    return reserve_block(ctx, &ctx->aux[which], &ctx->aux_bytes[which], bytes, out);
+    return reserve_block(ctx, &ctx->aux[which], &ctx->aux_bytes[which], bytes, std::min(bytes / 8, (size_t)64 << 20),
+                         out);
 }
 
-void hd_aux_trim(hd_ctx* ctx, int which, size_t most) {
-    if (ctx->aux_bytes[which] <= most) return;
-    cudaFree(ctx->aux[which]);
-    ctx->aux[which] = nullptr;
-    ctx->aux_bytes[which] = 0;
+void hd_aux_trim(hd_ctx* ctx) {
+    for (int k = 0; k < 2; ++k) {
+        if (ctx->aux_bytes[k] <= (size_t)1 << 30) continue;
+        cudaFree(ctx->aux[k]);
+        ctx->aux[k] = nullptr;
+        ctx->aux_bytes[k] = 0;
+    }
 }
 
 int hd_host_stage(hd_ctx* ctx, size_t bytes, void** out) {

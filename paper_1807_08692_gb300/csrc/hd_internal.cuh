@@ -169,8 +169,8 @@ int hd_ws_reserve(hd_ctx* ctx, size_t bytes, void** out);
 // Auxiliary block `which` (0 or 1) of at least `bytes`, 256-aligned, valid until the
 // next hd_aux_reserve of the same block.
 int hd_aux_reserve(hd_ctx* ctx, int which, size_t bytes, void** out);
-// Gives an auxiliary block larger than `most` bytes back (nothing may be using it).
-void hd_aux_trim(hd_ctx* ctx, int which, size_t most);
+// Gives the auxiliary blocks larger than 1 GiB back (nothing may be using them).
+void hd_aux_trim(hd_ctx* ctx);
 // Pinned host block of at least `bytes`, valid until the next hd_host_stage on the
 // same context; the caller leaves no copy in flight from or to it.
 int hd_host_stage(hd_ctx* ctx, size_t bytes, void** out);

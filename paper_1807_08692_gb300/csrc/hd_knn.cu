@@ -969,7 +969,7 @@ int hd_build_graph(hd_ctx* ctx, const void* X, int64_t n, int32_t d, int dtype, 
     if (!rc) rc = hd_knn_status(ctx);
     if (!rc) rc = hd_graph_from_lists(ctx, n, k, idx, sim, gamma, sym, out);
     cudaStreamSynchronize(ctx->stream);
-    for (int b = 0; b < 2; ++b) hd_aux_trim(ctx, b, (size_t)4 << 30);
+    hd_aux_trim(ctx);
     if (ox) cudaFree(ox);
     return rc;
 }

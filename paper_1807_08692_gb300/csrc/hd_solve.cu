@@ -2643,7 +2643,6 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
                  ws_size((size_t)rpad * Bp * 4);
     // the fp16 gather copy of P: graph solves with 8 <= Bp <= 256 columns in multiples of 8
     const bool half_ok = !ts && Bp % 8 == 0 && Bp <= 256;
-    if (ts) bytes += ws_size(vec);  // the transposed block
     if (half_ok) bytes += ws_size((size_t)n * Bp * 2);
     void* ws;
     int rc = hd_ws_reserve(ctx, bytes, &ws);
@@ -2653,7 +2652,7 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     S_.P = cv.take<float>((size_t)n * Bp);
     S_.Q = cv.take<float>((size_t)n * Bp);
     S_.X = x_direct ? X : cv.take<float>((size_t)n * Bp);
-    if (ts) S_.VT = cv.take<float>((size_t)n * Bp);
+    if (ts) S_.VT = ts->vt;
     S_.part = cv.take<float2>((size_t)S_.nch * Bp);
     S_.st = cv.take<ColState>(Bp);
     char* zero = cv.take<char>(zero_bytes);

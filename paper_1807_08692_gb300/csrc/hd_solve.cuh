@@ -137,6 +137,7 @@ struct TruncSys {
     const float* wv = nullptr;
     int32_t B = 0;
     int64_t smax = 0;
+    float* vt = nullptr;    // room for the transposed operand of the products [Bp][smax]
 };
 
 struct Engine {

@@ -10,7 +10,9 @@
 //                most entries of a row are outside S_j, and a test there costs
 //                no trip to L2
 //   pos[j][i]  = (position of id i in S_j, d_i^-1/2) for the ids of S_j: one
-//                gather per kept entry
+//                gather per kept entry.  Columns share up to 512 MB of it in
+//                turn (64 on 1M nodes at once), a bitmap of B n / 8 bytes is
+//                all that grows with B n
 //   row (j, t) = the entries of A's row S_j[t] whose column is in S_j, in the
 //                graph's column order, with their local positions
 //   counts (bitmap tests alone), offsets by an exclusive scan of them, entries
@@ -27,9 +29,10 @@
 
 namespace {
 
-// thread (t, j): pos[j][S_j[t]] = (t, D^-1/2); bad ids and duplicates raise the error flag
-__global__ void k_ts_mark(const int32_t* sl_ptr, const int32_t* sl_idx, const float* dinv, int32_t B, int64_t n, int2* pos,
-                          uint32_t* bits, int64_t words, int* err) {
+// thread (t, j): S_j's bitmap, and pos[j][S_j[t]] = (t, D^-1/2) of the first `placed`
+// columns; bad ids and duplicates raise the error flag
+__global__ void k_ts_mark(const int32_t* sl_ptr, const int32_t* sl_idx, const float* dinv, int64_t n, int2* pos,
+                          int32_t placed, uint32_t* bits, int64_t words, int* err) {
     const int j = blockIdx.y;
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int32_t b = sl_ptr[j], e = sl_ptr[j + 1];
@@ -41,6 +44,15 @@ __global__ void k_ts_mark(const int32_t* sl_ptr, const int32_t* sl_idx, const fl
     }
     const uint32_t bit = 1u << (i & 31);
     if (atomicOr(&bits[(int64_t)j * words + (i >> 5)], bit) & bit) atomicExch(err, 2);
+    if (j < placed) pos[(int64_t)j * n + i] = make_int2((int32_t)t, __float_as_int(dinv[i]));
+}
+// the same positions for a later group of columns (ids already checked)
+__global__ void k_ts_place(const int32_t* sl_ptr, const int32_t* sl_idx, const float* dinv, int64_t n, int2* pos) {
+    const int j = blockIdx.y;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int32_t b = sl_ptr[j], e = sl_ptr[j + 1];
+    if (t >= e - b) return;
+    const int32_t i = sl_idx[b + t];
     pos[(int64_t)j * n + i] = make_int2((int32_t)t, __float_as_int(dinv[i]));
 }
 
@@ -49,6 +61,7 @@ __global__ void k_ts_mark(const int32_t* sl_ptr, const int32_t* sl_idx, const fl
 // and then each row's columns, two per lane, one row ahead of the tests.
 constexpr int TS_T = 1024;
 constexpr int TS_SMEM_WORDS = 50 * 1024;  // bitmaps up to 200 KB (1.6M nodes) go to shared memory
+constexpr int64_t TS_POS_BYTES = (int64_t)512 << 20;  // position maps at a time (at least one column's)
 
 // For the rows lo .. hi of one column: row.rows32(t, valid, i) with each lane's own
 // row t (id i, -1 for an empty one) of the next 32, then for the r-th of them
@@ -357,10 +370,9 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
         bytes0 += ws_size(bytes ? bytes : 16);
         return at;
     };
-    // kept for the next call up to 4 GiB each
     auto release = [&]() {
         cudaStreamSynchronize(ctx->stream);
-        for (int k = 0; k < 2; ++k) hd_aux_trim(ctx, k, (size_t)4 << 30);
+        hd_aux_trim(ctx);
     };
     int rc = HD_OK;
 #define TS_TRY(x)         \
@@ -378,12 +390,16 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
     int* err;
     const size_t at_d_slp = part0((B + 1) * 4);
     const size_t at_d_sli = part0((size_t)nsl * 4);
-    const size_t at_pos = part0((size_t)B * n * 8);
-    const int64_t words = (n + 31) / 32;
-    const size_t at_bits = part0((size_t)B * words * 4);
+    // pos, cnt, deg and sdinv are done with when the solve starts, which keeps its
+    // transposed operand there (4 bytes a row and padded column)
+    const int32_t group = (int32_t)std::max<int64_t>(1, std::min<int64_t>(B, TS_POS_BYTES / (8 * n)));
+    const size_t at_pos = part0((size_t)group * n * 8);
     const size_t at_cnt = part0((size_t)rows * 4);
     const size_t at_deg = part0((size_t)rows * 4);
     const size_t at_sdinv = part0((size_t)rows * 4);
+    bytes0 = std::max(bytes0, at_pos + ws_size((size_t)smax * ((B + 3) / 4 * 4) * 4));
+    const int64_t words = (n + 31) / 32;
+    const size_t at_bits = part0((size_t)B * words * 4);
     const size_t at_bsum = part0((size_t)nblk * 8);
     const size_t at_off = part0((size_t)(rows + 1) * 8);
     const size_t at_d_yp = part0((B + 1) * 4);
@@ -430,8 +446,8 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
     }
     {
         HD_PROF(ctx, "trunc_build");
-        k_ts_mark<<<dim3((unsigned)((smax + 255) / 256), B), 256, 0, ctx->stream>>>(d_slp, d_sli, g->dinv, B, n,
-                                                                                    pos, bits, words, err);
+        k_ts_mark<<<dim3((unsigned)((smax + 255) / 256), B), 256, 0, ctx->stream>>>(d_slp, d_sli, g->dinv, n, pos,
+                                                                                    group, bits, words, err);
         TS_LAUNCH();
         k_ts_count<<<grid, TS_T, smem, ctx->stream>>>(g->row_ptr, g->col, d_slp, d_sli, B, n, smax, bits, words, cnt);
         TS_LAUNCH();
@@ -464,15 +480,24 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
         HD_PROF(ctx, "trunc_build");
         k_scan_apply<<<(unsigned)nblk, 1024, 0, ctx->stream>>>(cnt, rows, bsum, off);
         TS_LAUNCH();
-        k_ts_fill<<<grid, TS_T, smem, ctx->stream>>>(g->row_ptr, g->col, g->val, g->dinv, d_slp, d_sli, B, n, smax, pos,
-                                                     bits, words, off, ci, wv, deg);
-        TS_LAUNCH();
+        for (int32_t j0 = 0; j0 < B; j0 += group) {
+            const int32_t cols = std::min(group, B - j0);
+            if (j0) {
+                k_ts_place<<<dim3((unsigned)((smax + 255) / 256), cols), 256, 0, ctx->stream>>>(d_slp + j0, d_sli,
+                                                                                             g->dinv, n, pos);
+                TS_LAUNCH();
+            }
+            k_ts_fill<<<grid, TS_T, smem, ctx->stream>>>(g->row_ptr, g->col, g->val, g->dinv, d_slp + j0, d_sli, cols, n,
+                                                         smax, pos, bits + j0 * words, words, off + j0 * smax, ci, wv,
+                                                         deg + j0 * smax);
+            TS_LAUNCH();
+            k_ts_map_y<<<ceil_div(cols, 128), 128, 0, ctx->stream>>>(d_yp + j0, d_yi, d_yv, cols, n, pos,
+                                                                    bits + j0 * words, words, y_loc, y_lv, err);
+            TS_LAUNCH();
+        }
         k_ts_sdinv<<<ceil_div(rows, 256), 256, 0, ctx->stream>>>(deg, rows, sdinv);
         TS_LAUNCH();
         k_ts_scale<<<ceil_div(rows * 8, 256), 256, 0, ctx->stream>>>(off, ci, wv, sdinv, rows, smax);
-        TS_LAUNCH();
-        k_ts_map_y<<<ceil_div(B, 128), 128, 0, ctx->stream>>>(d_yp, d_yi, d_yv, B, n, pos, bits, words, y_loc,
-                                                                 y_lv, err);
         TS_LAUNCH();
     }
     TruncSys ts;
@@ -481,6 +506,7 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
     ts.wv = wv;
     ts.B = B;
     ts.smax = smax;
+    ts.vt = (float*)pos;
     rc = hd_query_impl(ctx, g, &ts, nullptr, HD_MODE_PAPER, B, d_yp, y_loc, y_lv, alpha, tol, max_iter, X, ldx, iters,
                        relres, status);
     if (!rc) {
