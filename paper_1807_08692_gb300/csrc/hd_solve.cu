@@ -625,12 +625,12 @@ __global__ void __launch_bounds__(128, 6) k_resid(const int32_t* __restrict__ rp
 // transposed block), so a column's gathers stay in its own n floats.
 //
 // Bound: one 4-byte gather per entry through L1 (110M entries: 0.38 ms at a line
-// per cycle).  One block per SM takes an equal share of the rows of all columns
-// in column order, so its L1 keeps to one or two columns' vectors.  It streams
+// per cycle).  One block per SM takes an equal share of the entries and rows of all
+// columns in column order, so its L1 keeps to one or two columns' vectors.  It streams
 // the entries in order: coalesced (index, weight) loads two tiles ahead, the
 // gathers they name one tile ahead, (weight, value) pairs in shared memory; a
 // thread then sums its own rows from there, so the order of a row's sum does
-// not depend on the tiling.  64 systems of 75,000 rows, 110M entries: 0.55 ms;
+// not depend on the tiling or on the shares.  64 systems of 75,000 rows, 110M entries: 0.55 ms;
 // with tiles of 2,048 entries, in which only three warps' rows are summed at a
 // time, 0.90 ms, of 8,192 (64 KB less L1) 0.64 ms; a thread per (row, 4 columns)
 // walking four rows in global memory and gathering 4 bytes of a 256-byte row
@@ -656,62 +656,123 @@ __global__ void __launch_bounds__(256) k_transpose(const float* __restrict__ V, 
         if (c0 + y + u < ld && r0 + x < n) VT[(int64_t)(c0 + y + u) * n + r0 + x] = t[x][y + u];
 }
 
-// The columns to work on, in order (whole quads, as in the update that reads Q);
-// st == nullptr: all.  Block-wide; returns their number.
-__device__ __forceinline__ int trunc_columns(const ColState* st, int32_t ld, uint16_t* list) {
+// Order of the columns that have rows, with the work before each: warp- and
+// block-wide scans over a chunk of TC_T columns.  `put(k, at)` is called for the
+// k-th of those with rows > 0 (w: the work of this thread's column); returns
+// through have / work the totals so far.
+template <class PUT>
+__device__ __forceinline__ void trunc_scan(bool on, int64_t w, int warps, int& have, int64_t& work, PUT put) {
     __shared__ int warp_count[TC_T / 32];
-    __shared__ int have;
+    __shared__ int64_t warp_work[TC_T / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) have = 0;
-    for (int c0 = 0; c0 < ld; c0 += TC_T) {
-        const int j = c0 + (int)threadIdx.x;
-        bool on = j < ld;
-        if (on && st) {
-            const ColState* q = st + (j & ~3);
-            on = q[0].active | q[1].active | q[2].active | q[3].active;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, on);
-        if (lane == 0) warp_count[warp] = __popc(m);
-        __syncthreads();
-        int at = have;
-        for (int w = 0; w < warp; ++w) at += warp_count[w];
-        if (on) list[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
-        __syncthreads();
-        if (threadIdx.x == TC_T - 1) have = at + __popc(m);
-        __syncthreads();
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    int64_t x = w;  // inclusive within the warp
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
     }
+    if (lane == 31) {
+        warp_count[warp] = __popc(m);
+        warp_work[warp] = x;
+    }
+    __syncthreads();
+    int k = have + __popc(m & ((1u << lane) - 1u));
+    int64_t at = work + x - w;
+    for (int v = 0; v < warps; ++v) {
+        k += v < warp ? warp_count[v] : 0;
+        at += v < warp ? warp_work[v] : 0;
+        have += warp_count[v];
+        work += warp_work[v];
+    }
+    if (on) put(k, at);
+    __syncthreads();
+}
+
+// The columns that have rows, in order, and their work; one block, once per call
+__global__ void __launch_bounds__(TC_T) k_trunc_work(const int32_t* __restrict__ sl_ptr, const int64_t* __restrict__ off,
+                                                     int32_t B, int64_t n, TruncWork* __restrict__ out) {
+    int have = 0;
+    int64_t work = 0;
+    for (int c0 = 0; c0 < B; c0 += TC_T) {
+        const int j = c0 + (int)threadIdx.x;
+        int rows = 0;
+        int64_t w = 0;
+        if (j < B) {
+            rows = sl_ptr[j + 1] - sl_ptr[j];
+            w = off[j * n + rows] - off[j * n] + rows;
+        }
+        trunc_scan(rows > 0, w, min(TC_T, B - c0 + 31) / 32, have, work,
+                   [&](int k, int64_t at) { out[k] = TruncWork{at, j, rows, (uint64_t)((double)rows / (double)w * 0x1p63)}; });
+    }
+    if (threadIdx.x == 0) out[have].at = work;
+}
+
+// The columns to work on, in order (whole quads, as in the update that reads Q;
+// st == nullptr: all), in shared memory.  Block-wide; returns their number,
+// list[number].at is the whole work.
+__device__ __forceinline__ int trunc_columns(const TruncSys& s, const ColState* st, TruncWork* list) {
+    int all = 1;
+    for (int i = threadIdx.x; i <= s.ncol; i += TC_T) {
+        const TruncWork w = s.work[i];
+        list[i] = w;
+        if (st && i < s.ncol) {
+            const ColState* q = st + (w.j & ~3);
+            all &= q[0].active | q[1].active | q[2].active | q[3].active;
+        }
+    }
+    if (__syncthreads_and(all)) return s.ncol;
+    int have = 0;
+    int64_t work = 0;
+    for (int c0 = 0; c0 < s.ncol; c0 += TC_T) {
+        const int i = c0 + (int)threadIdx.x;
+        TruncWork c{};
+        int64_t w = 0;
+        bool on = false;
+        if (i < s.ncol) {
+            c = s.work[i];
+            const ColState* q = st + (c.j & ~3);
+            on = q[0].active | q[1].active | q[2].active | q[3].active;
+            if (on) w = s.work[i + 1].at - c.at;
+        }
+        trunc_scan(on, w, min(TC_T, s.ncol - c0 + 31) / 32, have, work, [&](int k, int64_t at) {
+            c.at = at;
+            list[k] = c;
+        });
+    }
+    if (threadIdx.x == 0) list[have].at = work;
+    __syncthreads();
     return have;
 }
 
-// Streams the rows lo .. hi of one column (off, ci, wv: its CSR; v: its vector):
+// Streams the rows lo .. hi of one column (off, ci, wv: its CSR, fewer than 2^31
+// entries; v: its vector):
 // add(k, w, x) for a row's entries in order, k with the parity of the entry's
 // place, then done(row).
 template <class RS, class AD, class DN>
 __device__ __forceinline__ void trunc_rows(const int64_t* __restrict__ off, const int32_t* __restrict__ ci,
-                                           const float* __restrict__ wv, const float* __restrict__ v, int64_t lo,
-                                           int64_t hi, bool empty, float2 (*tile)[TC_TILE], RS reset, AD add, DN done) {
-    int64_t row = lo + threadIdx.x;
+                                           const float* __restrict__ wv, const float* __restrict__ v, unsigned lo,
+                                           unsigned hi, float2 (*tile)[TC_TILE], RS reset, AD add, DN done) {
+    unsigned row = lo + threadIdx.x;
     reset();
-    if (empty) {
-        for (; row < hi; row += TC_T) done(row);
-        return;
-    }
-    const int64_t first = __ldg(off + lo), last = __ldg(off + hi);
-    int64_t b = last, e = last, nb = last, ne = last;
-    auto bounds = [&](int64_t r, int64_t& x, int64_t& y) {
+    const int64_t first = __ldg(off + lo);
+    const unsigned last = (unsigned)(__ldg(off + hi) - first);
+    ci += first;
+    wv += first;
+    unsigned b = last, e = last, nb = last, ne = last;
+    auto bounds = [&](unsigned r, unsigned& x, unsigned& y) {
         if (r < hi) {
-            x = __ldg(off + r);
-            y = __ldg(off + r + 1);
+            x = (unsigned)(__ldg(off + r) - first);
+            y = (unsigned)(__ldg(off + r + 1) - first);
         }
     };
     bounds(row, b, e);
     bounds(row + TC_T, nb, ne);
     int32_t c[TC_E];
     float w[TC_E], x[TC_E], wn[TC_E];
-    auto indices = [&](int64_t t0) {
+    auto indices = [&](unsigned t0) {
 #pragma unroll
         for (int u = 0; u < TC_E; ++u) {
-            const int64_t q = t0 + u * TC_T + threadIdx.x;
+            const unsigned q = t0 + u * TC_T + threadIdx.x;
             c[u] = 0;
             wn[u] = 0.f;
             if (q < last) {
@@ -727,17 +788,17 @@ __device__ __forceinline__ void trunc_rows(const int64_t* __restrict__ off, cons
             w[u] = wn[u];
         }
     };
-    indices(first);
+    indices(0);
     gather();
-    indices(first + TC_TILE);
+    indices(TC_TILE);
     int buf = 0;
-    for (int64_t t0 = first; t0 < last; t0 += TC_TILE, buf ^= 1) {
+    for (unsigned t0 = 0; t0 < last; t0 += TC_TILE, buf ^= 1) {
 #pragma unroll
         for (int u = 0; u < TC_E; ++u) tile[buf][u * TC_T + threadIdx.x] = make_float2(w[u], x[u]);
         gather();                      // tile t0 + TC_TILE
         indices(t0 + 2 * TC_TILE);
         __syncthreads();  // this tile is complete, and every thread is done with the other buffer's last one
-        const int64_t t1 = min(last, t0 + TC_TILE);
+        const unsigned t1 = min(last, t0 + TC_TILE);
         while (row < hi && b < t1) {
             // the row's part of this tile, four reads ahead of their sums
             int q = (int)(max(b, t0) - t0);
@@ -773,55 +834,76 @@ __device__ __forceinline__ void trunc_rows(const int64_t* __restrict__ off, cons
     __syncthreads();
 }
 
-// A block's share of the rows of `count` columns
+// A block's share of the work; rows of a column count alike.  (Shares of equal
+// rows, those past a short list's end among them, left one shortlist of 500,000
+// among 15 of 1,000 to a tenth of the blocks: 14.7 ms for a call of 20 iterations
+// on 1M nodes with 54 entries a row against 4.7.)
 template <class F>
-__device__ __forceinline__ void trunc_share(int count, int64_t n, F each) {
-    const int64_t total = count * n, per = (total + gridDim.x - 1) / gridDim.x;
-    const int64_t g1 = min(total, (blockIdx.x + 1) * per);
-    for (int64_t g = blockIdx.x * per; g < g1;) {
-        const int k = (int)(g / n);
-        const int64_t lo = g - k * n, hi = min(n, lo + (g1 - g));
-        each(k, lo, hi);
-        g += hi - lo;
+__device__ __forceinline__ void trunc_share(int count, const TruncWork* list, F each) {
+    __shared__ volatile int64_t share[2];  // (in registers they would be spilled around the rows)
+    int k = 0;
+    {
+        const int64_t total = list[count].at, per = (total + gridDim.x - 1) / gridDim.x;
+        const int64_t x0 = blockIdx.x * per, x1 = min(total, x0 + per);
+        if (x0 >= x1) return;
+        for (int a = count; a - k > 1;) {  // the last column whose work starts at or before x0
+            const int m = (k + a) >> 1;
+            if (list[m].at <= x0) k = m;
+            else a = m;
+        }
+        if (threadIdx.x == 0) {
+            share[0] = x0;
+            share[1] = x1;
+        }
+        __syncthreads();
+    }
+    for (; list[k].at < share[1]; ++k) {  // (past the last column: the whole work)
+        const TruncWork c = list[k];
+        const int64_t y0 = share[0] - c.at, y1 = share[1] - c.at;
+        // neighbouring blocks round their common bound alike
+        auto row_at = [&](int64_t y) { return min((int64_t)__umul64hi((uint64_t)y << 1, c.rate), (int64_t)c.rows); };
+        const int64_t lo = y0 <= 0 ? 0 : row_at(y0);
+        const int64_t hi = y1 >= list[k + 1].at - c.at ? c.rows : row_at(y1);
+        if (lo < hi) each(c.j, lo, hi);
     }
 }
 
 // Q = c1 P - c2 W_j P column by column (VT: the transposed P); even and odd
-// entries of a row sum separately.
+// entries of a row sum separately.  Rows past a shortlist's end are left alone:
+// P is 0 there and Q was cleared at the start.
 __global__ void __launch_bounds__(TC_T, 1)
-    k_spmm_cols(const int64_t* __restrict__ off, const int32_t* __restrict__ ci, const float* __restrict__ wv, int32_t B,
-                const float* __restrict__ VT, float* __restrict__ Q, int64_t n, int32_t ld, float c1, float c2,
-                const ColState* __restrict__ st) {
+    k_spmm_cols(const TruncSys s, const float* __restrict__ VT, float* __restrict__ Q, int64_t n, int32_t ld, float c1,
+                float c2, const ColState* __restrict__ st) {
     extern __shared__ float2 tc_sm[];
     float2(*tile)[TC_TILE] = reinterpret_cast<float2(*)[TC_TILE]>(tc_sm);  // [2]
-    __shared__ uint16_t list[TC_COLS];
-    trunc_share(trunc_columns(st, ld, list), n, [&](int k, int64_t lo, int64_t hi) {
-        const int j = list[k];
+    TruncWork* list = reinterpret_cast<TruncWork*>(tc_sm + 2 * TC_TILE);
+    trunc_share(trunc_columns(s, st, list), list, [&](int j, int64_t lo, int64_t hi) {
         const float* v = VT + (int64_t)j * n;
         float s0, s1;
         trunc_rows(
-            off + (int64_t)j * n, ci, wv, v, lo, hi, j >= B, tile, [&] { s0 = s1 = 0.f; },
+            s.off + (int64_t)j * n, s.ci, s.wv, v, lo, hi, tile, [&] { s0 = s1 = 0.f; },
             [&](int i, float w, float p) {
                 if (i & 1) s1 = fmaf(w, p, s1);
                 else s0 = fmaf(w, p, s0);
             },
-            [&](int64_t row) { Q[row * ld + j] = c1 * v[row] - c2 * (s0 + s1); });
+            [&](unsigned row) { Q[(int64_t)row * ld + j] = c1 * v[row] - c2 * (s0 + s1); });
     });
 }
 
 // Q = -(c1 X - c2 W_j X) column by column, W_j X in two words (VT: the transposed X).
 __global__ void __launch_bounds__(TC_T, 1)
-    k_resid_cols(const int64_t* __restrict__ off, const int32_t* __restrict__ ci, const float* __restrict__ wv, int32_t B,
-                 const float* __restrict__ VT, float* __restrict__ Q, int64_t n, int32_t ld, float c1, float c2) {
+    k_resid_cols(const TruncSys s, const float* __restrict__ VT, float* __restrict__ Q, int64_t n, int32_t ld, float c1,
+                 float c2) {
     extern __shared__ float2 tc_sm[];
     float2(*tile)[TC_TILE] = reinterpret_cast<float2(*)[TC_TILE]>(tc_sm);  // [2]
-    trunc_share(ld, n, [&](int j, int64_t lo, int64_t hi) {
+    TruncWork* list = reinterpret_cast<TruncWork*>(tc_sm + 2 * TC_TILE);
+    trunc_share(trunc_columns(s, nullptr, list), list, [&](int j, int64_t lo, int64_t hi) {
         const float* v = VT + (int64_t)j * n;
         float a, b;
         trunc_rows(
-            off + (int64_t)j * n, ci, wv, v, lo, hi, j >= B, tile, [&] { a = b = 0.f; },
+            s.off + (int64_t)j * n, s.ci, s.wv, v, lo, hi, tile, [&] { a = b = 0.f; },
             [&](int, float w, float p) { df_fma(a, b, w, p); },
-            [&](int64_t row) { Q[row * ld + j] = neg_operator(c1, v[row], c2, a, b); });
+            [&](unsigned row) { Q[(int64_t)row * ld + j] = neg_operator(c1, v[row], c2, a, b); });
     });
 }
 
@@ -2255,16 +2337,18 @@ static int launch_trunc(Engine& E, const float* V, float c1, float c2, bool resi
                                                                                                         E.VT);
     HD_CHECK_LAUNCH(ctx);
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms, E.n * E.Bp / TC_T));
-    constexpr int smem = 2 * TC_TILE * (int)sizeof(float2);
+    constexpr int tiles = 2 * TC_TILE * (int)sizeof(float2);
+    const int smem = tiles + (ts.ncol + 1) * (int)sizeof(TruncWork);
     static uint64_t attr = 0;
     if (hd_first_on_device(attr, ctx->device)) {
-        HD_CUDA(ctx, cudaFuncSetAttribute(k_spmm_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        HD_CUDA(ctx, cudaFuncSetAttribute(k_resid_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        constexpr int most = tiles + (TC_COLS + 1) * (int)sizeof(TruncWork);
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_spmm_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_resid_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     }
     if (resid)
-        k_resid_cols<<<grid, TC_T, smem, ctx->stream>>>(ts.off, ts.ci, ts.wv, ts.B, E.VT, E.Q, E.n, E.Bp, c1, c2);
+        k_resid_cols<<<grid, TC_T, smem, ctx->stream>>>(ts, E.VT, E.Q, E.n, E.Bp, c1, c2);
     else
-        k_spmm_cols<<<grid, TC_T, smem, ctx->stream>>>(ts.off, ts.ci, ts.wv, ts.B, E.VT, E.Q, E.n, E.Bp, c1, c2, E.st);
+        k_spmm_cols<<<grid, TC_T, smem, ctx->stream>>>(ts, E.VT, E.Q, E.n, E.Bp, c1, c2, E.st);
     HD_CHECK_LAUNCH(ctx);
     return HD_OK;
 }
@@ -2348,7 +2432,7 @@ static uint64_t fbits(float f) {
 static std::vector<uint64_t> iteration_key(const Engine& E) {
     return {E.g->id, E.has_lr ? E.lr.e->id : 0, (uint64_t)E.ts, (uint64_t)(E.ts ? E.ts->off : nullptr),
             (uint64_t)(E.ts ? E.ts->ci : nullptr), (uint64_t)(E.ts ? E.ts->wv : nullptr),
-            (uint64_t)(E.ts ? E.ts->B : 0), (uint64_t)E.n,
+            (uint64_t)(E.ts ? E.ts->work : nullptr), (uint64_t)(E.ts ? E.ts->ncol : 0), (uint64_t)E.n,
             (uint64_t)E.R, (uint64_t)E.P, (uint64_t)E.Q, (uint64_t)E.X, (uint64_t)E.VT, (uint64_t)E.part, (uint64_t)E.st,
             (uint64_t)E.num_active, (uint64_t)E.lr.part, (uint64_t)E.lr.C, (uint64_t)E.lr.H, (uint64_t)E.lr.Hhi,
             (uint64_t)E.lr.Hlo, (uint64_t)E.dcoef, (uint64_t)E.opcoef, (uint64_t)E.segK, (uint64_t)E.seg,
@@ -2743,6 +2827,11 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     // the true-residual confirmation
     HD_CUDA(ctx, cudaMemsetAsync(S_.R, 0, vec, ctx->stream));
     HD_CUDA(ctx, cudaMemsetAsync(S_.X, 0, vec, ctx->stream));
+    if (ts) {
+        HD_CUDA(ctx, cudaMemsetAsync(S_.Q, 0, vec, ctx->stream));  // (rows past a shortlist's end stay 0)
+        k_trunc_work<<<1, TC_T, 0, ctx->stream>>>(ts->sl_ptr, ts->off, B, n, ts->work);
+        HD_CHECK_LAUNCH(ctx);
+    }
     k_scatter_y<<<B, 128, 0, ctx->stream>>>((const int32_t*)yp, (const int32_t*)yi, (const float*)yv, nnz_y, n, Bp,
                                             S_.R, S_.err);
     HD_CHECK_LAUNCH(ctx);

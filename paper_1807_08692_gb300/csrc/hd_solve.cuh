@@ -131,11 +131,21 @@ struct VecLaunch {
 // Truncated temporal systems (one per column): row t of column j has the
 // entries off[j * smax + t] .. off[j * smax + t + 1] of (ci, wv), ci a row
 // index of the same column's system; columns j >= B are empty.
+// One column's system in the list of work: `at` is where its share of the work
+// starts, counted in entries plus rows; rate: rows per unit of its work, times 2^63
+// (an integer: every thread of a block forms its bounds from it, and FP64 is slow)
+struct TruncWork {
+    int64_t at;
+    int32_t j, rows;
+    uint64_t rate;
+};
 struct TruncSys {
+    const int32_t* sl_ptr = nullptr;  // column j has sl_ptr[j + 1] - sl_ptr[j] rows, the others up to smax are empty
+    TruncWork* work = nullptr;        // room for the ncol columns that have rows, in order, and the whole work [ncol + 1]
+    int32_t ncol = 0;
     const int64_t* off = nullptr;
     const int32_t* ci = nullptr;
     const float* wv = nullptr;
-    int32_t B = 0;
     int64_t smax = 0;
     float* vt = nullptr;    // room for the transposed operand of the products [Bp][smax]
 };

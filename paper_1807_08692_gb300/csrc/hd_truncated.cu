@@ -56,9 +56,10 @@ __global__ void k_ts_place(const int32_t* sl_ptr, const int32_t* sl_idx, const f
     pos[(int64_t)j * n + i] = make_int2((int32_t)t, __float_as_int(dinv[i]));
 }
 
-// Both passes over the rows: a block takes an equal share of the B x smax rows in
-// column order; a warp takes 32 rows at a time, reads their bounds side by side
-// and then each row's columns, two per lane, one row ahead of the tests.
+// Both passes over the rows: a block takes an equal share of all shortlists' rows
+// in column order; a warp takes up to 32 rows at a time (fewer where a column's part
+// of the share is short, so that all warps have some), reads their bounds side by
+// side and then each row's columns, two per lane, one row ahead of the tests.
 constexpr int TS_T = 1024;
 constexpr int TS_SMEM_WORDS = 50 * 1024;  // bitmaps up to 200 KB (1.6M nodes) go to shared memory
 constexpr int64_t TS_POS_BYTES = (int64_t)512 << 20;  // position maps at a time (at least one column's)
@@ -69,12 +70,14 @@ constexpr int64_t TS_POS_BYTES = (int64_t)512 << 20;  // position maps at a time
 // and end(r), at last flush(t0, rows).
 template <class ROW>
 __device__ __forceinline__ void ts_rows(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
-                                        const int32_t* __restrict__ sl, int32_t len, int64_t n, int64_t lo, int64_t hi,
+                                        const int32_t* __restrict__ sl, int64_t n, int64_t lo, int64_t hi,
                                         const uint32_t* bits, ROW row) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t t0 = lo + 32 * warp; t0 < hi; t0 += TS_T) {
+    const int per = (int)min((int64_t)32, (hi - lo + TS_T / 32 - 1) / (TS_T / 32));
+    for (int64_t t0 = lo + per * warp; t0 < hi; t0 += per * (TS_T / 32)) {
+        const int rows = (int)min((int64_t)per, hi - t0);
         const int64_t mine = t0 + lane;
-        int32_t i = mine < hi && mine < len ? __ldg(sl + mine) : -1;
+        int32_t i = lane < rows ? __ldg(sl + mine) : -1;
         if (i >= n) i = -1;  // out of range (flagged by k_ts_mark): an empty row
         const int32_t b = i >= 0 ? __ldg(rp + i) : 0, e = i >= 0 ? __ldg(rp + i + 1) : 0;
         int32_t k[2], nk[2];
@@ -86,8 +89,7 @@ __device__ __forceinline__ void ts_rows(const int32_t* __restrict__ rp, const in
             }
         };
         columns(__shfl_sync(0xffffffffu, b, 0), __shfl_sync(0xffffffffu, e, 0), nk);
-        const int rows = (int)min((int64_t)32, hi - t0);
-        row.rows32(mine, mine < hi, i);
+        row.rows32(mine, lane < rows, i);
         for (int r = 0; r < rows; ++r) {
             const int32_t rb = __shfl_sync(0xffffffffu, b, r), re = __shfl_sync(0xffffffffu, e, r);
             const int r1 = min(r + 1, 31);
@@ -110,13 +112,22 @@ __device__ __forceinline__ void ts_rows(const int32_t* __restrict__ rp, const in
 }
 // A block's share of the rows, with the column's bitmap in shared memory if it fits
 template <class F>
-__device__ __forceinline__ void ts_share(int32_t B, int64_t smax, const uint32_t* bits, int64_t words, uint32_t* sm,
-                                         F each) {
-    const int64_t total = B * smax, per = (total + gridDim.x - 1) / gridDim.x;
-    const int64_t g1 = min(total, (blockIdx.x + 1) * per);
-    for (int64_t g = blockIdx.x * per; g < g1;) {
-        const int j = (int)(g / smax);
-        const int64_t lo = g - j * smax, hi = min(smax, lo + (g1 - g));
+__device__ __forceinline__ void ts_share(int32_t B, const int32_t* __restrict__ sl_ptr, const uint32_t* bits,
+                                         int64_t words, uint32_t* sm, F each) {
+    const int32_t first = __ldg(sl_ptr);
+    const int64_t total = (int64_t)__ldg(sl_ptr + B) - first, per = (total + gridDim.x - 1) / gridDim.x;
+    const int64_t g0 = blockIdx.x * per, g1 = min(total, g0 + per);
+    if (g0 >= g1) return;
+    int j = 0;  // the column of row g0: the last whose rows start at or before it
+    for (int a = B; a - j > 1;) {
+        const int m = (j + a) >> 1;
+        if (__ldg(sl_ptr + m) - first <= g0) j = m;
+        else a = m;
+    }
+    for (int64_t g = g0; g < g1; ++j) {
+        const int64_t at = (int64_t)__ldg(sl_ptr + j) - first, end = (int64_t)__ldg(sl_ptr + j + 1) - first;
+        const int64_t lo = g - at, hi = min(end, g1) - at;
+        if (lo >= hi) continue;  // an empty shortlist
         const uint32_t* bj = bits + j * words;
         if (words <= TS_SMEM_WORDS) {
             __syncthreads();
@@ -150,12 +161,11 @@ __global__ void __launch_bounds__(TS_T, 1) k_ts_count(const int32_t* rp, const i
                                                       const int32_t* sl_idx, int32_t B, int64_t n, int64_t smax,
                                                       const uint32_t* bits, int64_t words, int32_t* cnt) {
     extern __shared__ uint32_t ts_sm[];
-    ts_share(B, smax, bits, words, ts_sm, [&](int j, int64_t lo, int64_t hi, const uint32_t* bj) {
+    ts_share(B, sl_ptr, bits, words, ts_sm, [&](int j, int64_t lo, int64_t hi, const uint32_t* bj) {
         CountRow row;
         row.cnt = cnt + j * smax;
         row.mine = 0;
-        const int32_t b = sl_ptr[j];
-        ts_rows(rp, col, sl_idx + b, sl_ptr[j + 1] - b, n, lo, hi, bj, row);
+        ts_rows(rp, col, sl_idx + sl_ptr[j], n, lo, hi, bj, row);
     });
 }
 
@@ -218,7 +228,7 @@ __global__ void __launch_bounds__(TS_T, 1)
               const int32_t* sl_idx, int32_t B, int64_t n, int64_t smax, const int2* pos, const uint32_t* bits,
               int64_t words, const int64_t* off, int32_t* ci, float* wv, float* deg) {
     extern __shared__ uint32_t ts_sm[];
-    ts_share(B, smax, bits, words, ts_sm, [&](int j, int64_t lo, int64_t hi, const uint32_t* bj) {
+    ts_share(B, sl_ptr, bits, words, ts_sm, [&](int j, int64_t lo, int64_t hi, const uint32_t* bj) {
         FillRow row;
         row.val = val;
         row.dinv = dinv;
@@ -228,8 +238,7 @@ __global__ void __launch_bounds__(TS_T, 1)
         row.wv = wv;
         row.deg = deg + j * smax;
         row.mine = 0.f;
-        const int32_t b = sl_ptr[j];
-        ts_rows(rp, col, sl_idx + b, sl_ptr[j + 1] - b, n, lo, hi, bj, row);
+        ts_rows(rp, col, sl_idx + sl_ptr[j], n, lo, hi, bj, row);
     });
 }
 
@@ -400,6 +409,7 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
     bytes0 = std::max(bytes0, at_pos + ws_size((size_t)smax * ((B + 3) / 4 * 4) * 4));
     const int64_t words = (n + 31) / 32;
     const size_t at_bits = part0((size_t)B * words * 4);
+    const size_t at_work = part0((size_t)(B + 1) * sizeof(TruncWork));
     const size_t at_bsum = part0((size_t)nblk * 8);
     const size_t at_off = part0((size_t)(rows + 1) * 8);
     const size_t at_d_yp = part0((B + 1) * 4);
@@ -417,6 +427,7 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
     cnt = (int32_t*)((char*)aux + at_cnt);
     deg = (float*)((char*)aux + at_deg);
     sdinv = (float*)((char*)aux + at_sdinv);
+    TruncWork* work = (TruncWork*)((char*)aux + at_work);
     bsum = (int64_t*)((char*)aux + at_bsum);
     off = (int64_t*)((char*)aux + at_off);
     d_yp = (int32_t*)((char*)aux + at_d_yp);
@@ -437,6 +448,10 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
     TS_TRY(copy_in(d_yv, y_val, (size_t)nnz_y * 4));
     TS_CUDA(cudaMemsetAsync(err, 0, 16, ctx->stream));
     TS_CUDA(cudaMemsetAsync(bits, 0, (size_t)B * words * 4, ctx->stream));
+    if (nsl - hp[0] < rows) {  // rows past a shortlist's end: no entries, degree 0
+        TS_CUDA(cudaMemsetAsync(cnt, 0, (size_t)rows * 4, ctx->stream));
+        TS_CUDA(cudaMemsetAsync(deg, 0, (size_t)rows * 4, ctx->stream));
+    }
     const size_t smem = words <= TS_SMEM_WORDS ? (size_t)words * 4 : 0;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms, rows / 256));
     static uint64_t attr = 0;
@@ -501,10 +516,12 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
         TS_LAUNCH();
     }
     TruncSys ts;
+    ts.sl_ptr = d_slp;
+    ts.work = work;
+    for (int j = 0; j < B; ++j) ts.ncol += hp[j + 1] > hp[j];
     ts.off = off;
     ts.ci = ci;
     ts.wv = wv;
-    ts.B = B;
     ts.smax = smax;
     ts.vt = (float*)pos;
     rc = hd_query_impl(ctx, g, &ts, nullptr, HD_MODE_PAPER, B, d_yp, y_loc, y_lv, alpha, tol, max_iter, X, ldx, iters,
