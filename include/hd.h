@@ -153,9 +153,11 @@ int hd_observe(hd_ctx* ctx, const void* X, int64_t n, int32_t d, int dtype, cons
 
 int hd_graph_info(const hd_graph* g, int64_t* n, int64_t* nnz);
 /* The SpMM launch shape the library chose for this graph at padded batch
- * width Bp (B rounded up to 4) during an earlier solve: *slab = columns per
- * row group (4..128), *segments = node-range passes.  HD_ERR_INVALID_ARG if no
- * solve with that width has run on the graph yet. */
+ * width Bp (B rounded up to 4) during the latest solve: *slab = columns per
+ * row group (a multiple of 4 up to 128; 32 where a wide or ragged block is kept
+ * in panels of 32 columns, whose last one may have another width), *segments =
+ * node-range passes.  HD_ERR_INVALID_ARG if no solve with that width has run on
+ * the graph yet. */
 int hd_graph_tuning(const hd_graph* g, int32_t Bp, int32_t* slab, int32_t* segments);
 /* Copy the normalised graph out (any pointer may be NULL; host or device):
  * row_ptr[n+1], col[nnz], val[nnz] = W, dinv[n] = D^-1/2. Rows sorted by column. */

@@ -90,7 +90,7 @@ struct hd_graph {
     int32_t* col = nullptr;
     float* val = nullptr;     // normalised W
     float* dinv = nullptr;    // D^-1/2
-    // SpMM column-slab width taken per padded batch width (Bp -> S), for hd_graph_tuning
+    // SpMM column-slab width of the latest solve per padded batch width (Bp -> S), for hd_graph_tuning
     mutable std::map<int, int> slab_cache;
     // node-range segments of the SpMM: per segment count K, the entry bounds
     // [K + 1][n] of every row's part in each range of ceil(n / K) columns

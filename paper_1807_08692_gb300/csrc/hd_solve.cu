@@ -2024,12 +2024,9 @@ static int spmm_lanes(int32_t cols, int per, bool big) {
 }
 static bool spmm_exceeds_l2(int64_t n, int32_t Bp, int bytes) { return n * Bp * bytes > (int64_t)64 << 20; }
 
-// Column-slab width of the SpMM (4 x lanes per row); recorded per graph and
-// batch width for hd_graph_tuning.  HD_SLAB caps it.
+// Column-slab width of the SpMM over plain rows (4 x lanes per row).  HD_SLAB caps it.
 int spmm_slab(const hd_graph* g, int32_t Bp) {
-    const int S = getenv("HD_SLAB") ? pick_slab(Bp) : 4 * spmm_lanes(Bp, 4, spmm_exceeds_l2(g->n, Bp, 4));
-    g->slab_cache[Bp] = S;
-    return S;
+    return getenv("HD_SLAB") ? pick_slab(Bp) : 4 * spmm_lanes(Bp, 4, spmm_exceeds_l2(g->n, Bp, 4));
 }
 
 // Layout of a gathered n x Bp block with `bytes` per entry: rows, or panels as wide
@@ -2056,10 +2053,13 @@ void engine_set_panels(Engine& E, int eff_mode) {
     E.pv = E.hv = panel_rows(E.n, E.Bp);
     // (truncated systems and segments read rows, and so do the low-rank products of
     // the deflated forms and those off the tensor cores; so does a forced slab width)
-    if (E.ts || E.segK > 1 || getenv("HD_SLAB")) return;
-    if (E.has_lr && (eff_mode != HD_MODE_PCG || !lr_use_tensor_cores(E.lr.e))) return;
-    E.pv = panels_for(E.n, E.Bp, 4);
-    E.hv = panels_for(E.n, E.Bp, 2);
+    if (E.ts) return;
+    if (E.segK == 1 && !getenv("HD_SLAB") && (!E.has_lr || (eff_mode == HD_MODE_PCG && lr_use_tensor_cores(E.lr.e)))) {
+        E.pv = panels_for(E.n, E.Bp, 4);
+        E.hv = panels_for(E.n, E.Bp, 2);
+    }
+    // what the products of this solve run with, for hd_graph_tuning
+    E.g->slab_cache[E.Bp] = E.segK > 1 ? E.vl.S : E.pv.last ? std::min(E.slab, E.pv.w) : E.slab;
 }
 
 // LC = L where L is a power of two that divides the width, else LC = 0

@@ -225,7 +225,7 @@ class Graph:
         self.ctx.check(lib().hd_graph_save(self.ctx.handle, self._h, str(path).encode()), "hd_graph_save")
 
     def tuning(self, B: int):
-        """(slab, segments) the SpMM measured for batch width B, or None before any solve at that width."""
+        """(slab, segments) of the SpMM in the latest solve at batch width B, or None before any (hd_graph_tuning)."""
         sl, sg = i32(), i32()
         if lib().hd_graph_tuning(self._h, (B + 3) // 4 * 4, C.byref(sl), C.byref(sg)) != OK:
             return None
