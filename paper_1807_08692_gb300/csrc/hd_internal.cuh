@@ -172,7 +172,10 @@ int hd_aux_reserve(hd_ctx* ctx, int which, size_t bytes, void** out);
 // Gives the auxiliary blocks larger than 1 GiB back (nothing may be using them).
 void hd_aux_trim(hd_ctx* ctx);
 // Pinned host block of at least `bytes`, valid until the next hd_host_stage on the
-// same context; the caller leaves no copy in flight from or to it.
+// same context; the caller leaves no copy in flight from or to it.  For what is
+// small: an array above HD_STAGE_MOST is copied from or to the caller's own memory,
+// so that the block, which the context keeps, stays small too.
+constexpr size_t HD_STAGE_MOST = (size_t)8 << 20;
 int hd_host_stage(hd_ctx* ctx, size_t bytes, void** out);
 // drop the cached device address of hd_rank_static's scratch on a device
 void hd_rank_static_forget(int device);

@@ -466,8 +466,11 @@ int hd_rank_impl(hd_ctx* ctx, const float* Xd, int64_t n, int32_t B, int32_t ldx
     void* ws;
     int rc = hd_ws_reserve(ctx, bytes, &ws);
     if (rc) return rc;
-    char* hs;  // pinned: K on the way in, status and host results on the way out
-    if ((rc = hd_host_stage(ctx, (size_t)B * 4 + out_bytes, (void**)&hs))) return rc;
+    // pinned: K on the way in, status and host results (unless they are long) on the way out
+    const bool staged = host && 2 * res <= HD_STAGE_MOST;
+    const size_t back = (size_t)B * 4 + (staged ? 2 * res : 0);
+    char* hs;
+    if ((rc = hd_host_stage(ctx, (size_t)B * 4 + back, (void**)&hs))) return rc;
     WsCarver cv(ws);
     int32_t* Kd = cv.take<int32_t>(B);
     uint64_t* cand = cv.take<uint64_t>((size_t)B * TK_CAP);
@@ -505,7 +508,7 @@ int hd_rank_impl(hd_ctx* ctx, const float* Xd, int64_t n, int32_t B, int32_t ldx
     k_topk_sort<<<B, 1024, TK_SORT_SMEM, ctx->stream>>>(cand, cnt, Kd, m, Kmax, idx_d, score_d, fail);
     HD_CHECK_LAUNCH(ctx);
     int* hf = (int*)(hs + (size_t)B * 4);
-    HD_CUDA(ctx, cudaMemcpyAsync(hf, fail, out_bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    HD_CUDA(ctx, cudaMemcpyAsync(hf, fail, back, cudaMemcpyDeviceToHost, ctx->stream));
     HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     std::vector<int32_t> Kf;
     for (int j = 0; j < B; ++j)
@@ -515,12 +518,16 @@ int hd_rank_impl(hd_ctx* ctx, const float* Xd, int64_t n, int32_t B, int32_t ldx
         }
     if (!Kf.empty()) {
         if ((rc = radix_rank(ctx, src, m, B, ld, Kf.data(), Kmax, idx_d, score_d, 1, cv))) return rc;
-        if (host) {
+        if (staged) {
             HD_CUDA(ctx, cudaMemcpyAsync(hf + B, idx_d, 2 * res, cudaMemcpyDeviceToHost, ctx->stream));
             HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         }
     }
-    if (host) {
+    if (host && !staged) {
+        HD_CUDA(ctx, cudaMemcpyAsync(idx_out, idx_d, res, cudaMemcpyDefault, ctx->stream));
+        HD_CUDA(ctx, cudaMemcpyAsync(score_out, score_d, res, cudaMemcpyDefault, ctx->stream));
+        HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    } else if (host) {
         const void* from[2] = {hf + B, hf + B + (size_t)B * Kmax};
         void* to[2] = {idx_out, score_out};
         for (int q = 0; q < 2; ++q) {

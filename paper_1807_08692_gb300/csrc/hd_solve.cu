@@ -2710,15 +2710,24 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     size_t bytes = 3 * ws_size(vec) + (x_direct ? 0 : ws_size(vec)) + ws_size((size_t)S_.nch * Bp * sizeof(float2)) +
                    ws_size(Bp * sizeof(ColState));
     // what the host sends in one copy: the observations and tolerances that are
-    // in host memory, then the six coefficient vectors
+    // in host memory, then the six coefficient vectors; long observations follow
+    // in copies of their own
     const void* host_in[4] = {y_ptr, y_idx, y_val, tol};
     const size_t host_len[4] = {(size_t)(B + 1) * 4, (size_t)nnz_y * 4, (size_t)nnz_y * 4, (size_t)B * 4};
-    size_t host_at[5] = {0, 0, 0, 0, 0};
+    size_t host_at[4] = {0, 0, 0, 0}, in_bytes = 0;
     for (int k = 0; k < 4; ++k) {
         if (host_len[k] && hd_is_device_ptr(host_in[k])) host_in[k] = nullptr;  // used where it is
-        host_at[k + 1] = host_at[k] + (host_in[k] ? ws_size(host_len[k]) : 0);
+        if (!host_in[k] || host_len[k] > HD_STAGE_MOST) continue;
+        host_at[k] = in_bytes;
+        in_bytes += ws_size(host_len[k]);
     }
-    const size_t in_bytes = host_at[4] + 6 * (size_t)rpad * 8;
+    const size_t coef_at = in_bytes, staged = coef_at + 6 * (size_t)rpad * 8;
+    in_bytes = ws_size(staged);
+    for (int k = 0; k < 4; ++k)
+        if (host_in[k] && host_len[k] > HD_STAGE_MOST) {
+            host_at[k] = in_bytes;
+            in_bytes += ws_size(host_len[k]);
+        }
     // what starts at zero: the counters, max |P_j|, the split H
     const size_t zero_bytes = ws_size(64) + ws_size((size_t)Bp * 4) + (lr_on ? 2 * ws_size((size_t)Bp16 * rpad * 2) : 0);
     bytes += ws_size(in_bytes) + zero_bytes;
@@ -2747,12 +2756,15 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
     HD_CUDA(ctx, cudaMemsetAsync(zero, 0, zero_bytes, ctx->stream));
     char* d_in = cv.take<char>(in_bytes);
     char* hs;  // pinned: the inputs now, the columns' states after the confirmation
-    if ((rc = hd_host_stage(ctx, std::max(in_bytes, B * sizeof(ColState)), (void**)&hs))) return rc;
+    if ((rc = hd_host_stage(ctx, std::max(staged, B * sizeof(ColState)), (void**)&hs))) return rc;
     const void* dev_in[4] = {y_ptr, y_idx, y_val, tol};
     for (int k = 0; k < 4; ++k)
         if (host_in[k]) {
-            if (host_len[k]) memcpy(hs + host_at[k], host_in[k], host_len[k]);
             dev_in[k] = d_in + host_at[k];
+            if (host_len[k] > HD_STAGE_MOST)
+                HD_CUDA(ctx, cudaMemcpyAsync(d_in + host_at[k], host_in[k], host_len[k], cudaMemcpyHostToDevice, ctx->stream));
+            else if (host_len[k])
+                memcpy(hs + host_at[k], host_in[k], host_len[k]);
         }
     const void *yp = dev_in[0], *yi = dev_in[1], *yv = dev_in[2], *tl = dev_in[3];
     S_.nnz_y = nnz_y;
@@ -2772,9 +2784,9 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
         S_.lr.Hhi = zv.take<__nv_bfloat16>((size_t)Bp16 * rpad);
         S_.lr.Hlo = zv.take<__nv_bfloat16>((size_t)Bp16 * rpad);
         double** dst[6] = {&S_.gcoef, &S_.hcoef, &S_.opcoef, &S_.dcoef, &S_.ones, &S_.negop};
-        double* co = (double*)(hs + host_at[4]);
+        double* co = (double*)(hs + coef_at);
         std::fill(co, co + 6 * (size_t)rpad, 0.0);
-        for (int k = 0; k < 6; ++k) *dst[k] = (double*)(d_in + host_at[4]) + (size_t)k * rpad;
+        for (int k = 0; k < 6; ++k) *dst[k] = (double*)(d_in + coef_at) + (size_t)k * rpad;
         double *gc = co, *hc = gc + rpad, *oc = hc + rpad, *dc = oc + rpad, *on = dc + rpad, *ng = on + rpad;
         const double a = alpha;
         const double c3 = mode == HD_MODE_PROJ ? a : a / (1.0 - a);
@@ -2789,7 +2801,7 @@ int hd_query_impl(hd_ctx* ctx, const hd_graph* g, const TruncSys* ts, const hd_e
             ng[k] = -a / (1.0 - a) * l;
         }
     }
-    if (in_bytes) HD_CUDA(ctx, cudaMemcpyAsync(d_in, hs, in_bytes, cudaMemcpyHostToDevice, ctx->stream));
+    if (staged) HD_CUDA(ctx, cudaMemcpyAsync(d_in, hs, staged, cudaMemcpyHostToDevice, ctx->stream));
 
     // ---------------- setup
     if (!ts && g->max_row < 0) {
