@@ -731,13 +731,14 @@ static int hd_knn_impl(hd_ctx* ctx, const void* Xd, int64_t n, int32_t d, int dt
     if (dtype == HD_F32) {
         // float4 loads need 16-byte rows
         const int vec = d % 4 == 0 && ((uintptr_t)Xd & 15) == 0 && ((uintptr_t)Qd & 15) == 0;
-        static uint64_t attr_f = 0;
-        if (hd_first_on_device(attr_f, ctx->device)) {
+        static HdDeviceOnce attr_f;
+        if (const int ra = attr_f.run(ctx->device, [&]() -> int {
             HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knnf::Cfg<1>::SMEM));
             HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knnf::Cfg<2>::SMEM));
             HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_f32<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knnf::Cfg<4>::SMEM));
             HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)knnf::Cfg<8>::SMEM));
-        }
+            return HD_OK;
+        })) return ra;
         const float *X = (const float*)Xd, *Q = (const float*)Qd;
         switch (knn_f32_tm(nq)) {
             case 1: k_knn_f32<1><<<p.grid, 256, knnf::Cfg<1>::SMEM, ctx->stream>>>(X, Q, a, vec); break;
@@ -751,10 +752,11 @@ static int hd_knn_impl(hd_ctx* ctx, const void* Xd, int64_t n, int32_t d, int dt
         CUtensorMap tq, tx;
         if (hd_make_tmap_2d(&tq, Qd, 2, nq, d, d, BM, BK, 1) || hd_make_tmap_2d(&tx, Xd, 2, n, d, d, BN, BK, 1))
             return hd_fail(ctx, HD_ERR_CUDA, "cuTensorMapEncodeTiled failed");
-        static uint64_t attr = 0;
-        if (hd_first_on_device(attr, ctx->device)) {
+        static HdDeviceOnce attr;
+        if (const int ra = attr.run(ctx->device, [&]() -> int {
             HD_CUDA(ctx, cudaFuncSetAttribute(k_knn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-        }
+            return HD_OK;
+        })) return ra;
         HD_CUDA(ctx, cudaMemsetAsync(ctx->d_flags + 1, 0, sizeof(int), ctx->stream));
         k_knn_tc<<<p.grid, THREADS, SMEM_BYTES, ctx->stream>>>(tq, tx, a, ctx->d_flags + 1);
         HD_CHECK_LAUNCH(ctx);

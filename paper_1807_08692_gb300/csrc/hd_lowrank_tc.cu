@@ -784,11 +784,12 @@ int lr_tc_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float
     }
     while (ns > XMIN && smem_of(Nc, ns) > max_smem) --ns;
     const int apipe = conv + ns * stage;
-    static uint64_t attr[2] = {0, 0};
-    if (hd_first_on_device(attr[su], ctx->device)) {
+    static HdDeviceOnce attr[2];
+    if (const int ra = attr[su].run(ctx->device, [&]() -> int {
         HD_CUDA(ctx, cudaFuncSetAttribute(su ? k_lr_expand_tc<1> : k_lr_expand_tc<0>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    }
+        return HD_OK;
+    })) return ra;
     for (int c0 = 0; c0 < cols; c0 += Nc) {
         const int nc = std::min(Nc, cols - c0);
         CUtensorMap th, tl;
@@ -847,11 +848,12 @@ int lr_tc_reduce(hd_ctx* ctx, const LowRank& lr, const float* V, int64_t n, int3
     while (Nc > 64 && (smem_of(Nc) > (size_t)max_smem || mt * Nc > 512 || Nc > 256)) Nc -= 64;
     if (mt * Nc > 512 || smem_of(Nc) > (size_t)max_smem)
         return hd_fail(ctx, HD_ERR_INVALID_ARG, "rank %d too large for the tensor-core reduction", e->r);
-    static uint64_t attr[2] = {0, 0};
-    if (hd_first_on_device(attr[su], ctx->device)) {
+    static HdDeviceOnce attr[2];
+    if (const int ra = attr[su].run(ctx->device, [&]() -> int {
         HD_CUDA(ctx, cudaFuncSetAttribute(su ? k_lr_reduce_tc<1> : k_lr_reduce_tc<0>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    }
+        return HD_OK;
+    })) return ra;
     const int64_t tiles = (n + BM - 1) / BM;
     const int grid = lr.nchunk;
     for (int c0 = 0; c0 < Bp64; c0 += Nc) {

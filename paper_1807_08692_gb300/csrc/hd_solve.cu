@@ -1952,12 +1952,13 @@ int lr_expand(hd_ctx* ctx, const LowRank& lr, int op, float* out, const float* R
     size_t smem = (size_t)e->r * 16 * sizeof(float);
     int gx = (int)std::min<int64_t>(ceil_div(n, 64), (int64_t)ctx->num_sms * 8);
     dim3 grid(gx, ceil_div(Bp, 16));
-    static uint64_t attr = 0;
-    if (hd_first_on_device(attr, ctx->device)) {
-        cudaFuncSetAttribute(k_lr_expand_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024 + 1024);
-        cudaFuncSetAttribute(k_lr_expand_simt<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024 + 1024);
-        cudaFuncSetAttribute(k_lr_expand_simt<__nv_fp8_e4m3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024 + 1024);
-    }
+    static HdDeviceOnce attr;
+    if (const int ra = attr.run(ctx->device, [&]() -> int {
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_lr_expand_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024 + 1024));
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_lr_expand_simt<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024 + 1024));
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_lr_expand_simt<__nv_fp8_e4m3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024 + 1024));
+        return HD_OK;
+    })) return ra;
     if (e->storage == HD_F32)
         k_lr_expand_simt<float><<<grid, 256, smem, ctx->stream>>>((const float*)e->U, e->scale, e->ldu, e->r, lr.H, op,
                                                                   out, Rv, Pv, n, Bp, st, gate);
@@ -2134,9 +2135,11 @@ template <int OP>
 static int launch_staged(Engine& E, const RedLaunch& l, const float* P, const Panels& pv, float2* part,
                          const ColState* st, const IterReset& z = {}) {
     hd_ctx* ctx = E.ctx;
-    static uint64_t attr = 0;
-    if (hd_first_on_device(attr, ctx->device))
+    static HdDeviceOnce attr;
+    if (const int ra = attr.run(ctx->device, [&]() -> int {
         HD_CUDA(ctx, cudaFuncSetAttribute(k_red_staged<OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs_smem<OP>()));
+        return HD_OK;
+    })) return ra;
     k_red_staged<OP><<<l.grid, l.block, rs_smem<OP>(), ctx->stream>>>(E.X, E.R, P, pv, E.Q, E.n, E.Bp, E.rch, st, E.xs,
                                                                         part, z);
     HD_CHECK_LAUNCH(ctx);
@@ -2339,12 +2342,13 @@ static int launch_trunc(Engine& E, const float* V, float c1, float c2, bool resi
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms, E.n * E.Bp / TC_T));
     constexpr int tiles = 2 * TC_TILE * (int)sizeof(float2);
     const int smem = tiles + (ts.ncol + 1) * (int)sizeof(TruncWork);
-    static uint64_t attr = 0;
-    if (hd_first_on_device(attr, ctx->device)) {
+    static HdDeviceOnce attr;
+    if (const int ra = attr.run(ctx->device, [&]() -> int {
         constexpr int most = tiles + (TC_COLS + 1) * (int)sizeof(TruncWork);
         HD_CUDA(ctx, cudaFuncSetAttribute(k_spmm_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
         HD_CUDA(ctx, cudaFuncSetAttribute(k_resid_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    }
+        return HD_OK;
+    })) return ra;
     if (resid)
         k_resid_cols<<<grid, TC_T, smem, ctx->stream>>>(ts, E.VT, E.Q, E.n, E.Bp, c1, c2);
     else

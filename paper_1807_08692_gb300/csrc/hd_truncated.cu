@@ -454,11 +454,12 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
     }
     const size_t smem = words <= TS_SMEM_WORDS ? (size_t)words * 4 : 0;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms, rows / 256));
-    static uint64_t attr = 0;
-    if (hd_first_on_device(attr, ctx->device)) {
-        TS_CUDA(cudaFuncSetAttribute(k_ts_count, cudaFuncAttributeMaxDynamicSharedMemorySize, TS_SMEM_WORDS * 4));
-        TS_CUDA(cudaFuncSetAttribute(k_ts_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, TS_SMEM_WORDS * 4));
-    }
+    static HdDeviceOnce attr;
+    TS_TRY(attr.run(ctx->device, [&]() -> int {
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_ts_count, cudaFuncAttributeMaxDynamicSharedMemorySize, TS_SMEM_WORDS * 4));
+        HD_CUDA(ctx, cudaFuncSetAttribute(k_ts_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, TS_SMEM_WORDS * 4));
+        return HD_OK;
+    }));
     {
         HD_PROF(ctx, "trunc_build");
         k_ts_mark<<<dim3((unsigned)((smax + 255) / 256), B), 256, 0, ctx->stream>>>(d_slp, d_sli, g->dinv, n, pos,
