@@ -532,6 +532,7 @@ int hd_graph_from_csr(hd_ctx* ctx, int64_t n, int64_t nnz, const int32_t* row_pt
 
 int hd_graph_tuning(const hd_graph* g, int32_t Bp, int32_t* slab, int32_t* segments) {
     if (!g) return HD_ERR_INVALID_ARG;
+    std::lock_guard<std::mutex> hold(g->found);
     auto it = g->slab_cache.find(Bp);
     if (it == g->slab_cache.end()) return HD_ERR_INVALID_ARG;
     if (slab) *slab = it->second;

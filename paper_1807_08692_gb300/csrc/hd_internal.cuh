@@ -7,6 +7,7 @@
 #include <stdint.h>
 #include <atomic>
 #include <map>
+#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
@@ -91,6 +92,8 @@ struct hd_graph {
     int32_t* col = nullptr;
     float* val = nullptr;     // normalised W
     float* dinv = nullptr;    // D^-1/2
+    // what solves find out about the graph, on whatever thread: held for the maps below
+    mutable std::mutex found;
     // SpMM column-slab width of the latest solve per padded batch width (Bp -> S), for hd_graph_tuning
     mutable std::map<int, int> slab_cache;
     // node-range segments of the SpMM: per segment count K, the entry bounds
@@ -100,7 +103,7 @@ struct hd_graph {
     mutable std::map<int, int32_t*> seg_bounds;
     mutable std::map<int, int> seg_cache;
     // entries in the longest row (measured on first use; -1 until then)
-    mutable int32_t max_row = -1;
+    mutable std::atomic<int32_t> max_row{-1};
 };
 
 struct hd_eig {

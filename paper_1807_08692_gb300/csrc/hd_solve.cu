@@ -2060,6 +2060,7 @@ void engine_set_panels(Engine& E, int eff_mode) {
         E.hv = panels_for(E.n, E.Bp, 2);
     }
     // what the products of this solve run with, for hd_graph_tuning
+    std::lock_guard<std::mutex> hold(E.g->found);
     E.g->slab_cache[E.Bp] = E.segK > 1 ? E.vl.S : E.pv.last ? std::min(E.slab, E.pv.w) : E.slab;
 }
 
@@ -2254,6 +2255,7 @@ static int launch_spmm(Engine& E, float c1, float c2, float2* part, const ColSta
 }
 
 static const int32_t* seg_bounds_for(hd_ctx* ctx, const hd_graph* g, int K) {
+    std::lock_guard<std::mutex> hold(g->found);
     auto it = g->seg_bounds.find(K);
     if (it != g->seg_bounds.end()) return it->second;
     int32_t* b = nullptr;
@@ -2264,11 +2266,11 @@ static const int32_t* seg_bounds_for(hd_ctx* ctx, const hd_graph* g, int K) {
     const int64_t w = (g->n + K - 1) / K;
     k_seg_bounds<<<ceil_div(g->n, 256), 256, 0, ctx->stream>>>(g->row_ptr, g->col, g->n, K, w, b);
     ctx->launches++;
-    if (cudaGetLastError() != cudaSuccess) {
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(ctx->stream) != cudaSuccess) {
         cudaFree(b);
         return nullptr;
     }
-    g->seg_bounds[K] = b;
+    g->seg_bounds[K] = b;  // (complete: other contexts' streams may read them)
     return b;
 }
 
@@ -2282,7 +2284,10 @@ int spmm_segments(hd_ctx* ctx, Engine& E) {
         forced = s ? atoi(s) : -1;
     }
     if (forced < 1) return HD_OK;
-    g->seg_cache[E.Bp] = forced;  // reported by hd_graph_tuning
+    {
+        std::lock_guard<std::mutex> hold(g->found);
+        g->seg_cache[E.Bp] = forced;  // reported by hd_graph_tuning
+    }
     if (forced > 1) {
         const int32_t* b = seg_bounds_for(ctx, g, forced);
         if (!b) return hd_fail(ctx, HD_ERR_OOM, "SpMM segment bounds");
