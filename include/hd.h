@@ -353,8 +353,8 @@ int hd_selftest_wait(hd_ctx* ctx, uint32_t limit_us, int32_t* gave_up);
  * and max_iter stay the same (any change re-captures it; with
  * hd_profile_enable on, kernels launch one by one instead).  The call is
  * therefore not itself capturable into a caller's graph.  Errors: HD_ERR_INVALID_ARG for bad
- * sizes, indices out of range or non-finite observation values (checked on
- * the device before any iteration; X is then undefined),
+ * sizes, indices out of range or non-finite observation values (left out on
+ * the device and reported after the first iterations; X is then undefined),
  * HD_ERR_TIMEOUT if a tensor-core kernel gave up one of its bounded pipeline
  * waits (the kernels never hang; X is then undefined),
  * HD_ERR_NOT_CONVERGED is NOT returned: per-column status says it. */

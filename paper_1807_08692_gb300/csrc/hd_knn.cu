@@ -209,7 +209,7 @@ __device__ __forceinline__ void knn_store(const KnnArgs& a, int seg, int64_t row
 // tile that holds them, so that no product is formed for padding.
 //
 // Bound: the FP32 pipe (127 ms of fused multiply-adds for the lists of 100,000 x
-// 512; 221 ms for the whole graph, from 407 ms with a 64 x 64 tile, 4 x 4 per
+// 512; 210 ms for the whole graph, from 407 ms with a 64 x 64 tile, 4 x 4 per
 // thread, and one thread inserting per row; 64 queries against 100,000 x 512:
 // 0.40 ms, from 101.5 ms on one SM).  Candidates above a row's threshold are
 // appended to 64 slots of shared memory (32 columns of a row at a time), merged

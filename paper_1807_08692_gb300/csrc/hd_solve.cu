@@ -1128,7 +1128,7 @@ __global__ void __launch_bounds__(256) k_dot(const float* __restrict__ P, const 
 // The first block of the update (or, where the reduction after it is still gated
 // by the active count, of the low-rank finish) clears what the scalar step and
 // the fp16 copy accumulate into, in place of three memsets per iteration (16
-// queries on 2,000 nodes: 457 -> 397 us); null pointers are skipped.
+// queries on 2,000 nodes: 457 -> 395 to 415 us); null pointers are skipped.
 __device__ __forceinline__ void iter_reset(const IterReset& z) {
     if (blockIdx.x | blockIdx.y) return;
     if (z.p16_max)
@@ -1428,7 +1428,7 @@ __global__ void k_fin_sigma(const float2* part, int nblk, int32_t Bp, ColState* 
 
 // After the update: rr, convergence, beta.  With C: PCG rho' = rr + sum_k coef_k C_k^2.
 // num_active must be zero before the launch (iter_reset).
-// use_half (may be null; 1 before the launch): cleared when a column that stays
+// use_half (may be null; not 0 before the launch, see iter_reset): cleared when a column that stays
 // active has ||r||^2 > theta2 tol^2 ||b||^2 (the next SpMM then gathers fp32).
 __global__ void k_fin_rr(const float2* part, int nblk, int32_t Bp, ColState* st, int32_t max_iter,
                          const double* C, const double* coef, int32_t r, int* num_active, int* use_half = nullptr,
@@ -2038,6 +2038,8 @@ int spmm_slab(const hd_graph* g, int32_t Bp) {
 //                   200,000 x 72: 3.70 / 3.44   30,000 x 148: 1.38 / 1.32   30,000 x 52: 0.67 / 0.69
 //   whole lines     1M x 64: 17.0 / 17.1   1M x 128: 37.9 / 34.3   1M x 256: 75.4 / 67.8
 //                   400,000 x 128: 11.6 / 11.7   250,000 x 256: 14.3 / 13.9
+// Ragged widths take panels from 16 MB on, whole lines from 256 MB on, where the gain
+// passes 3%: below that the two sides lie within 3% of each other either way.
 // The columns past the last whole panel stand alone where the block exceeds L2 (1M x
 // 72: 26.2 against 29.1 when fewer than half a panel join the one before), and join
 // below that, where one launch less counts more (100,000 x 72: 1.84 against 1.90).
