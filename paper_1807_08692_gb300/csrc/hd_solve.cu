@@ -2007,27 +2007,35 @@ VecLaunch vec_launch(hd_ctx* ctx, int64_t n, int32_t Bp, int S) {
         default: { constexpr int SS = 128; __VA_ARGS__; } break;  \
     }
 
+static bool spmm_exceeds_l2(int64_t n, int32_t Bp, int bytes) { return n * Bp * bytes > (int64_t)64 << 20; }
+// One 128-byte line of every node is more than twice what L2 holds: passes that
+// gather a line per entry then find almost none of them there, and a longer
+// stretch of each row at a time is the better use of DRAM.
+static bool spmm_lines_exceed_l2(int64_t n) { return n * 128 > (int64_t)256 << 20; }
+
 // Lanes per row of the SpMM over `cols` columns in groups of `per` (4 fp32 or 8
-// fp16 columns per lane; `big`: the gathered block exceeds what L2 holds).
+// fp16 columns per lane).
 // Whole 128-byte lines, one per row and pass (8 lanes), when the width allows:
 // a 64-column pass over a block larger than L2 reads 1.3 times the DRAM bytes
 // (1M nodes, 64 columns: 1.18 ms against 1.50 ms).  16 lanes when the block fits
-// in L2 (100,000 x 64: 0.082 ms against 0.086 ms), and from 256 columns on, where
+// in L2 (100,000 x 64: 0.082 ms against 0.086 ms), from 256 columns on, where
 // the 128-byte lines of one pass lie 1 KB apart (1M x 256: 6.1 ms against 6.7;
-// panels, see panels_for, take 4.8).
+// panels, see panels_for, take 4.8), and from 2.1M nodes on (16 lanes against 8 at
+// 64 columns, 54 entries a row: 1.5M 2.68 / 2.35 ms, 2M 3.79 / 3.80, 3M 6.04 / 6.76,
+// 5M 10.6 / 12.6).
 // Other widths take the whole row at once up to 16 lanes, else the fewest even
 // parts of at most 16: 100,000 x 40 runs in 0.067 ms with 10 lanes, 0.12 ms in
 // two passes of 9 and 0.174 ms in five of 2.
-static int spmm_lanes(int32_t cols, int per, bool big) {
+static int spmm_lanes(int64_t n, int32_t cols, int per) {
     const int nl = cols / per;
-    if (nl % 8 == 0) return per == 4 && nl % 16 == 0 && (!big || nl >= 64) ? 16 : 8;
+    const bool pass_fits = !spmm_exceeds_l2(n, cols, 16 / per);
+    if (nl % 8 == 0) return per == 4 && nl % 16 == 0 && (pass_fits || nl >= 64 || spmm_lines_exceed_l2(n)) ? 16 : 8;
     return ceil_div(nl, ceil_div(nl, 16));
 }
-static bool spmm_exceeds_l2(int64_t n, int32_t Bp, int bytes) { return n * Bp * bytes > (int64_t)64 << 20; }
 
 // Column-slab width of the SpMM over plain rows (4 x lanes per row).  HD_SLAB caps it.
 int spmm_slab(const hd_graph* g, int32_t Bp) {
-    return getenv("HD_SLAB") ? pick_slab(Bp) : 4 * spmm_lanes(Bp, 4, spmm_exceeds_l2(g->n, Bp, 4));
+    return getenv("HD_SLAB") ? pick_slab(Bp) : 4 * spmm_lanes(g->n, Bp, 4);
 }
 
 // Layout of a gathered n x Bp block with `bytes` per entry: rows, or panels as wide
@@ -2039,7 +2047,11 @@ int spmm_slab(const hd_graph* g, int32_t Bp) {
 //   whole lines     1M x 64: 17.0 / 17.1   1M x 128: 37.9 / 34.3   1M x 256: 75.4 / 67.8
 //                   400,000 x 128: 11.6 / 11.7   250,000 x 256: 14.3 / 13.9
 // Ragged widths take panels from 16 MB on, whole lines from 256 MB on, where the gain
-// passes 3%: below that the two sides lie within 3% of each other either way.
+// passes 3%: below that the two sides lie within 3% of each other either way.  From
+// 2.1M nodes on, blocks of whole 64-column stretches go back to rows, read 256 bytes
+// at a time (products in panels / rows, ms, 54 entries a row: 2M x 128 7.33 / 7.60,
+// 2M x 256 15.0 / 15.3, 3M x 128 12.7 / 12.2, 5M x 128 23.1 / 21.2, 5M x 256 45.3 /
+// 42.5; ragged widths stay: 5M x 40 9.9 / 10.2, 5M x 72 16.0 / 22.3).
 // The columns past the last whole panel stand alone where the block exceeds L2 (1M x
 // 72: 26.2 against 29.1 when fewer than half a panel join the one before), and join
 // below that, where one launch less counts more (100,000 x 72: 1.84 against 1.90).
@@ -2047,6 +2059,7 @@ static Panels panels_for(int64_t n, int32_t Bp, int bytes) {
     const int32_t w = 128 / bytes;
     const int64_t mb = n * Bp * bytes >> 20;
     if (Bp % w ? Bp < w || mb < 16 : Bp <= 2 * w || mb < 256) return panel_rows(n, Bp);
+    if (bytes == 4 && Bp % 64 == 0 && spmm_lines_exceed_l2(n)) return panel_rows(n, Bp);
     const int32_t alone = spmm_exceeds_l2(n, Bp, bytes) ? 4 : w / 2;
     const int32_t last = ((Bp + w - alone) / w - 1) * w;
     return Panels{n, w, last, Bp - last};
@@ -2113,7 +2126,7 @@ static int spmm_launch(hd_ctx* ctx, const hd_graph* g, const float* P, const Pan
 
 int hd_spmm_apply(hd_ctx* ctx, const hd_graph* g, const float* P, float* Q, int32_t ld, int32_t B, float c1,
                   float c2) {
-    return spmm_launch(ctx, g, P, panel_rows(g->n, ld), Q, ld, 4 * spmm_lanes(ld, 4, spmm_exceeds_l2(g->n, ld, 4)), c1, c2, nullptr, nullptr);
+    return spmm_launch(ctx, g, P, panel_rows(g->n, ld), Q, ld, 4 * spmm_lanes(g->n, ld, 4), c1, c2, nullptr, nullptr);
 }
 
 // grid and block of the column reductions: one chunk per block row.  `staged`
@@ -2223,7 +2236,7 @@ static int launch_spmm(Engine& E, float c1, float c2, float2* part, const ColSta
                 const int32_t last = first < cut ? cut : E.Bp;
                 const int L16 = cut && last == E.Bp ? (last - first) / 8
                                 : E.hv.last         ? E.hv.w / 8
-                                                    : spmm_lanes(E.Bp, 8, spmm_exceeds_l2(E.n, E.Bp, 2));
+                                                    : spmm_lanes(E.n, E.Bp, 8);
                 const dim3 gh = spmm_grid(ctx, E.n, last - first, 8, L16, 7);
                 HD_DISPATCH_L(L16, (last - first) / 8, (k_spmm_h<LC, G><<<gh, 128, 0, ctx->stream>>>(
                                        g->row_ptr, g->col, g->val, E.P16, E.hv, E.p16_max, E.P, E.pv, E.Q,
