@@ -2149,18 +2149,27 @@ int hd_spmm_apply(hd_ctx* ctx, const hd_graph* g, const float* P, float* Q, int3
 }
 
 // grid and block of the column reductions: one chunk per block row.  `staged`
-// (k_red_staged) when the thread-per-(g, quad) form would leave the GPU less
-// than half full: it lives off resident warps, about 1,024 threads per SM.
+// (k_red_staged) while the thread-per-(g, quad) form has too few threads to stream:
+// below 192 per SM for the dot product, 168 for the update (which stores as it
+// goes), 320 for the squares.  Thread form / staged, us:
+//   dot      100,000 x 64 (165 per SM) 24.2 / 19.8   200,000 x 36 (185) 24.9 / 25.6
+//            100,000 x 100 (258) 27.3 / 36.9         300,000 x 128 (987) 57.6 / 108
+//   update   100,000 x 64 30.7 / 31.1   200,000 x 36 34 / 47   1M x 36 (926) 131 / 290
+//   squares  100,000 x 128 (330) 19.3 / 18.9         200,000 x 128 (659) 27.3 / 35.9
+// At one or two quads the thread form has 8 or 16 threads per block and short runs of
+// a row: update and squares stay staged at any size (2M x 8 67.6 / 59.6 and 22.4 / 22.4,
+// 5M x 4 135 / 96 and 44 / 37).
 struct RedLaunch {
     dim3 grid;
     unsigned block;
     size_t smem;
     bool staged;
 };
-static RedLaunch red_launch(const Engine& E) {
+static RedLaunch red_launch(const Engine& E, RedOp op) {
     const int nq = E.Bp / 4, qpb = nq < RQ ? nq : RQ;
+    const int per_sm = op == RED_DOT ? 192 : op == RED_UPDATE ? 168 : 320;
     RedLaunch l;
-    l.staged = E.nch * nq * RG < (int64_t)E.ctx->num_sms * 1024;
+    l.staged = E.nch * nq * RG < (int64_t)E.ctx->num_sms * per_sm || (op != RED_DOT && nq <= 2);
     l.grid = dim3((unsigned)E.nch, (unsigned)ceil_div(E.Bp, l.staged ? RS_COLS : 4 * RQ));
     l.block = l.staged ? 256u : (unsigned)(RG * qpb);
     l.smem = (size_t)l.block * 4 * sizeof(float2);
@@ -2184,7 +2193,7 @@ static int launch_staged(Engine& E, const RedLaunch& l, const float* P, const Pa
 static int launch_dot(Engine& E, float2* part, const ColState* st) {
     hd_ctx* ctx = E.ctx;
     HD_PROF(ctx, "dot");
-    const RedLaunch l = red_launch(E);
+    const RedLaunch l = red_launch(E, RED_DOT);
     if (l.staged) return launch_staged<RED_DOT>(E, l, E.P, E.pv, part, st);
     k_dot<<<l.grid, l.block, l.smem, ctx->stream>>>(E.P, E.pv, E.Q, E.n, E.Bp, E.rch, part, st);
     HD_CHECK_LAUNCH(ctx);
@@ -2194,7 +2203,7 @@ static int launch_dot(Engine& E, float2* part, const ColState* st) {
 static int launch_update(Engine& E) {
     hd_ctx* ctx = E.ctx;
     HD_PROF(ctx, "update");
-    const RedLaunch l = red_launch(E);
+    const RedLaunch l = red_launch(E, RED_UPDATE);
     IterReset z;
     z.p16_max = E.use_half ? E.p16_max : nullptr;
     z.Bp = E.Bp;
@@ -2212,7 +2221,7 @@ static int launch_update(Engine& E) {
 static int launch_colsq(Engine& E, const float* V) {
     hd_ctx* ctx = E.ctx;
     HD_PROF(ctx, "colsq");
-    const RedLaunch l = red_launch(E);
+    const RedLaunch l = red_launch(E, RED_SQ);
     if (l.staged) return launch_staged<RED_SQ>(E, l, V, panel_rows(E.n, E.Bp), E.part, nullptr);
     k_colsq<<<l.grid, l.block, l.smem, ctx->stream>>>(V, E.n, E.Bp, E.rch, E.part);
     HD_CHECK_LAUNCH(ctx);

@@ -52,3 +52,14 @@ def test_streams_at_the_copy_rate(n, B):
     gb = n * B * 4 / 1e9
     # two blocks read; four read and two written
     assert t["dot"] < 1.33 * rate * 2 * gb and t["update"] < 1.04 * rate * 6 * gb, (t, rate)
+
+
+@pytest.mark.parametrize("n,B", [(300000, 128), (1000000, 36), (500000, 100)])
+def test_half_full_grids_are_not_staged(n, B):
+    # sizes whose thread form has 700 to 1,000 threads per SM: staged they ran at half this rate
+    import torch
+    import paper_1807_08692_gb300 as hd
+    rate = _copy_us_per_gb(torch)
+    t = _times_us(hd, n, B)
+    gb = n * B * 4 / 1e9
+    assert t["dot"] < 1.8 * rate * 2 * gb and t["update"] < 1.2 * rate * 6 * gb, (t, rate)
