@@ -104,16 +104,16 @@ __device__ __forceinline__ void take64(uint64_t& a0, uint64_t& a1, uint64_t b0, 
 }
 
 // Merge a row's `cnt` buffered candidates (shared memory) into its list of 64
-// keys (global scratch, descending).  Warp-collective; returns the k-th entry,
-// the empty one while there are fewer.
-__device__ __forceinline__ uint64_t knn_flush(uint64_t* list, const uint64_t* buf, int cnt, int k, int lane) {
+// keys (global scratch, descending).  Warp-collective; returns the similarity of
+// the k-th entry, -inf while there are fewer.
+__device__ __forceinline__ float knn_flush(uint64_t* list, const uint64_t* buf, int cnt, int k, int lane) {
     uint64_t a0 = list[lane], a1 = list[lane + 32];
     uint64_t b0 = lane < cnt ? buf[lane] : 0ull, b1 = lane + 32 < cnt ? buf[lane + 32] : 0ull;
     sort64(b0, b1, lane);
     take64(a0, a1, b0, b1, lane);
     list[lane] = a0;
     list[lane + 32] = a1;
-    return __shfl_sync(0xffffffffu, k > 32 ? a1 : a0, (k - 1) & 31);
+    return key_sim(__shfl_sync(0xffffffffu, k > 32 ? a1 : a0, (k - 1) & 31));
 }
 
 // The same for at most 32 candidates held as (similarity bits, id) pairs.
@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(256, 2)
     float* Bs = As + 2 * FK * ALD;                          // [2][FK][BLD]
     uint64_t* bufs = reinterpret_cast<uint64_t*>(Bs + 2 * FK * BLD);  // [BM][KBUF_LD]
     float* tau = reinterpret_cast<float*>(bufs + BM * KBUF_LD);       // [BM]
-    int* tie = reinterpret_cast<int*>(tau + BM);                      // [BM]
-    int* cnt = tie + BM;                                              // [BM]
+    float* kth = tau + BM;                                            // [BM]
+    int* cnt = reinterpret_cast<int*>(kth + BM);                      // [BM]
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, warp = tid >> 5, lane = tid & 31;
     const int ntile = (int)((a.n + BN - 1) / BN), nk = (a.d + FK - 1) / FK, nitem = a.nwork * a.nseg;
     uint64_t* lists = a.lists + (int64_t)blockIdx.x * BM * 64;
@@ -277,8 +277,7 @@ __global__ void __launch_bounds__(256, 2)
             lists[r * 64 + lane + 32] = 0ull;
         }
         if (tid < BM) {
-            tau[tid] = q0 + tid < a.nq ? -INFINITY : INFINITY;  // a row past the last query takes nothing
-            tie[tid] = -1;
+            tau[tid] = kth[tid] = q0 + tid < a.nq ? -INFINITY : INFINITY;  // a row past the last query takes nothing
             cnt[tid] = 0;
         }
         float4 ar[AV], br[2];
@@ -350,10 +349,14 @@ __global__ void __launch_bounds__(256, 2)
                 if (more) stash(b ^ 1);
                 __syncthreads();
             }
-            // ---- candidates of this tile, 32 columns of every row at a time.  The four
+            // ---- candidates of this tile, 32 columns of every row at a time: what lies
+            // above the threshold, which starts at the k-th similarity so far.  The four
             // steps interleave their columns, so a step can meet an id smaller than one
-            // that an earlier step put in the list: what equals the k-th similarity
-            // (tau) enters if its id is below the k-th entry's (tie).
+            // that an earlier step of this tile put in the list; a merge in mid-tile
+            // therefore leaves the threshold just below the new k-th similarity, equals
+            // are taken too and the lists' order decides (a comparison of ids per
+            // candidate instead cost 1 to 5% of the kernel)
+            bool merged = false;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 int most = 0;
@@ -365,28 +368,29 @@ __global__ void __launch_bounds__(256, 2)
                     const float v[2] = {acc[i][2 * j], acc[i][2 * j + 1]};
 #pragma unroll
                     for (int u = 0; u < 2; ++u)
-                        if (v[u] >= th && id0 + u < a.n && !(a.excl && id0 + u == q0 + r) &&
-                            (v[u] > th || id0 + u < tie[r])) {
+                        if (v[u] > th && id0 + u < a.n && !(a.excl && id0 + u == q0 + r)) {
                             const int p = atomicAdd(&cnt[r], 1);
                             bufs[r * KBUF_LD + p] = knn_key(v[u], id0 + u);
                             most = max(most, p + 1);
                         }
                 }
                 if (__syncthreads_or(most > KBUF - 32)) {
+                    merged = true;
                     for (int r = warp; r < BM; r += 8) {
                         const int rc = cnt[r];
                         __syncwarp();
                         if (rc <= KBUF - 32) continue;
-                        const uint64_t kth = knn_flush(lists + r * 64, bufs + r * KBUF_LD, rc, a.k, lane);
+                        const float s = knn_flush(lists + r * 64, bufs + r * KBUF_LD, rc, a.k, lane);
                         if (lane == 0) {
-                            tau[r] = key_sim(kth);
-                            tie[r] = key_id(kth);
+                            kth[r] = s;
+                            tau[r] = nextafterf(s, -INFINITY);
                             cnt[r] = 0;
                         }
                     }
                     __syncthreads();
                 }
             }
+            if (merged && tid < BM) tau[tid] = kth[tid];  // (read again after the next tile's barriers)
         }
         __syncthreads();
         for (int r = warp; r < BM; r += 8) {
