@@ -2317,6 +2317,13 @@ static const int32_t* seg_bounds_for(hd_ctx* ctx, const hd_graph* g, int K) {
     return b;
 }
 
+// Two segments where a row is a quarter or half of a 128-byte line and half of the
+// block still finds room in L2: a product in one pass / in two, ms (54 entries a row)
+//   16 columns   2M 1.13 / 1.10   3M 2.29 / 1.91   5M 4.68 / 3.92
+//    8 columns   3M 1.35 / 1.45   5M 3.61 / 2.80
+// and whole solves, whose late iterations then gather fp32 too, 2M x 16 11.5 / 12.0,
+// 3M x 16 21.5 / 20.4, 5M x 16 43.9 / 40.7, 5M x 8 30.8 / 28.6.  Narrower rows (5M x 4
+// 1.80 / 2.26) and wider ones (5M x 32 5.9 / 6.3) lose.
 int spmm_segments(hd_ctx* ctx, Engine& E) {
     const hd_graph* g = E.g;
     E.segK = 1;
@@ -2326,17 +2333,17 @@ int spmm_segments(hd_ctx* ctx, Engine& E) {
         const char* s = getenv("HD_SEGMENTS");
         forced = s ? atoi(s) : -1;
     }
-    if (forced < 1) return HD_OK;
-    {
-        std::lock_guard<std::mutex> hold(g->found);
-        g->seg_cache[E.Bp] = forced;  // reported by hd_graph_tuning
-    }
-    if (forced > 1) {
-        const int32_t* b = seg_bounds_for(ctx, g, forced);
-        if (!b) return hd_fail(ctx, HD_ERR_OOM, "SpMM segment bounds");
-        E.segK = forced;
+    int K = std::max(forced, 1);
+    if (forced < 1 && (E.Bp == 8 || E.Bp == 16) && E.n * E.Bp * 4 > (int64_t)140 << 20 && !getenv("HD_SLAB")) K = 2;
+    if (K > 1) {
+        const int32_t* b = seg_bounds_for(ctx, g, K);
+        if (!b && forced > 1) return hd_fail(ctx, HD_ERR_OOM, "SpMM segment bounds");
+        if (!b) K = 1;
         E.seg = b;
     }
+    E.segK = K;
+    std::lock_guard<std::mutex> hold(g->found);
+    g->seg_cache[E.Bp] = K;  // reported by hd_graph_tuning
     return HD_OK;
 }
 

@@ -202,7 +202,8 @@ int spmm_slab(const hd_graph* g, int32_t Bp);
 // Layouts of P and P16 for this solve (n, Bp, slab, ts, segK and the eigenpairs set).
 void engine_set_panels(Engine& E, int eff_mode);
 int simt_nchunk(hd_ctx* ctx, int64_t n, int rpad, int Bp);
-// Node-range segments for the SpMM: one pass unless HD_SEGMENTS asks for more;
+// Node-range segments for the SpMM: one pass, or two by the rule beside it, unless
+// HD_SEGMENTS says how many;
 // sets E.segK / E.seg.
 int spmm_segments(hd_ctx* ctx, Engine& E);
 int engine_iteration(Engine& E, int (*after_update)(void*), void* arg);

@@ -41,3 +41,27 @@ def test_shape_on_both_sides_of_the_line(gpu_ctx, monkeypatch, n, widths):
             out.append((X.view(torch.int32), np.array(it)))
         assert np.array_equal(out[0][1], out[1][1]) and bool(torch.equal(out[0][0], out[1][0])), B
     g.close()
+
+
+SEG = 140 << 20   # bytes of an 8- or 16-column block from which its products take two node ranges
+
+
+@pytest.mark.parametrize("n,B,segments", [(SEG // 64, 16, 1), (SEG // 64 + 1, 16, 2), (SEG // 64 + 1, 14, 2), (SEG // 64 + 1, 12, 1),
+                                          (SEG // 32, 8, 1), (SEG // 32 + 1, 8, 2)])
+def test_two_node_ranges(gpu_ctx, monkeypatch, n, B, segments):
+    import torch
+    import paper_1807_08692_gb300 as hd
+    monkeypatch.delenv("HD_SLAB", raising=False)
+    g = _graph(gpu_ctx, n)
+    y = _queries(n, 20, np.random.default_rng(B))
+    k = int(y[0][B])
+    X, it, _, st = hd.query_batch(gpu_ctx, g, None, "paper", y[0][:B + 1], y[1][:k], y[2][:k], 0.9, 1e-5, 100)
+    assert np.all(np.array(st) == 0) and g.tuning(B)[1] == segments
+    # the same columns in a batch of another width, whose sums run in one pass; each residual is below 1e-5 ||y||
+    # and L_a >= I, so the two differ by at most 2e-5 ||y||
+    W, iw, _, sw = hd.query_batch(gpu_ctx, g, None, "paper", *y, 0.9, 1e-5, 100)
+    assert np.all(np.array(sw) == 0) and g.tuning(20)[1] == 1
+    ynorm = torch.tensor([float(np.linalg.norm(y[2][y[0][j]:y[0][j + 1]])) for j in range(B)], device="cuda")
+    assert bool(((X - W[:, :B]).norm(dim=0) <= 2.1e-5 * ynorm).all())
+    assert np.all(np.abs(np.array(it) - np.array(iw)[:B]) <= 1)
+    g.close()
