@@ -453,7 +453,7 @@ extern "C" int hd_temporal_truncated(hd_ctx* ctx, const hd_graph* g, int32_t B, 
         TS_CUDA(cudaMemsetAsync(deg, 0, (size_t)rows * 4, ctx->stream));
     }
     const size_t smem = words <= TS_SMEM_WORDS ? (size_t)words * 4 : 0;
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms, rows / 256));
+    const unsigned grid = (unsigned)std::min<int64_t>(ctx->num_sms, std::max<int64_t>(B, rows / 256));
     static HdDeviceOnce attr;
     TS_TRY(attr.run(ctx->device, [&]() -> int {
         HD_CUDA(ctx, cudaFuncSetAttribute(k_ts_count, cudaFuncAttributeMaxDynamicSharedMemorySize, TS_SMEM_WORDS * 4));

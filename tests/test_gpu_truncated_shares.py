@@ -88,3 +88,27 @@ def test_a_long_shortlist_among_short_ones(gpu_ctx):
 
     # the products of the long one take all of the GPU either way; the vectors are four times as wide
     assert seconds([300000] + [500] * 15) < 2.5 * seconds([300000])
+
+
+def test_short_shortlists_run_side_by_side(gpu_ctx):
+    import torch
+    import paper_1807_08692_gb300 as hd
+    n = 20000
+    g = _graph(gpu_ctx, n, 16)
+    rng = np.random.default_rng(4)
+
+    def seconds(B):
+        ptr, sls, obs = _inputs(n, [100] * B, rng)
+        idx, X = torch.from_numpy(np.concatenate(sls)).cuda(), torch.empty((100, B), device="cuda")
+        best = 1e9
+        for _ in range(12):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            hd.temporal_truncated(gpu_ctx, g, ptr, idx, np.arange(B + 1, dtype=np.int32), obs, np.ones(B, np.float32),
+                                  0.99, 1e-12, 100, X=X)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t0)
+        return best
+
+    # sixteen short chains of loads take the time of one, not of sixteen in a block
+    assert seconds(16) < 1.3 * seconds(1)
