@@ -381,9 +381,10 @@ __global__ void __launch_bounds__(128) k_sort_long(const int32_t* rp, int32_t* c
         }
     }
 }
-int hd_sort_rows(hd_ctx* ctx, const int32_t* rp, int32_t* col, float* val, int64_t n) {
+int hd_sort_rows(hd_ctx* ctx, const int32_t* rp, int32_t* col, float* val, int64_t n, int32_t longest) {
     k_sort_rows<<<ceil_div(n, 4), 128, 0, ctx->stream>>>(rp, col, val, n);
     HD_CHECK_LAUNCH(ctx);
+    if (longest <= SORT_ROW) return HD_OK;
     k_sort_long<<<std::min(ceil_div(n, 128), ctx->num_sms * 8), 128, 0, ctx->stream>>>(rp, col, val, n);
     HD_CHECK_LAUNCH(ctx);
     return HD_OK;

@@ -238,7 +238,8 @@ int hd_graph_from_lists(hd_ctx* ctx, int64_t n, int32_t k, const int32_t* idx_d,
                         float gamma, int sym, hd_graph** out);
 int hd_normalize_graph(hd_ctx* ctx, hd_graph* g);
 // Orders every CSR row by column, equal columns in their given order.
-int hd_sort_rows(hd_ctx* ctx, const int32_t* rp, int32_t* col, float* val, int64_t n);
+// `longest`: entries of the longest row, where the caller knows.
+int hd_sort_rows(hd_ctx* ctx, const int32_t* rp, int32_t* col, float* val, int64_t n, int32_t longest = INT32_MAX);
 int hd_graph_alloc_internal(hd_ctx* ctx, int64_t n, int64_t nnz, hd_graph** out);
 int hd_graph_check(hd_ctx* ctx, const hd_graph* g);
 int hd_eig_alloc(hd_ctx* ctx, int64_t n, int32_t r, int storage, hd_eig** out);

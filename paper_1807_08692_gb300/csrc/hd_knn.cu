@@ -872,9 +872,11 @@ int hd_graph_from_lists(hd_ctx* ctx, int64_t n, int32_t k, const int32_t* idx_d,
     HD_CUDA(ctx, cudaMemcpyAsync(h_len.data(), len, n * 4, cudaMemcpyDeviceToHost, ctx->stream));
     HD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     int64_t acc = 0;
+    int32_t longest = 0;
     for (int64_t i = 0; i < n; ++i) {
         h_ptr[i] = (int32_t)acc;
         acc += h_len[i];
+        longest = std::max(longest, h_len[i]);
     }
     h_ptr[n] = (int32_t)acc;
     if (acc >= (1ll << 31)) return hd_fail(ctx, HD_ERR_INVALID_ARG, "graph too large: nnz=%lld", (long long)acc);
@@ -885,7 +887,7 @@ int hd_graph_from_lists(hd_ctx* ctx, int64_t n, int32_t k, const int32_t* idx_d,
     k_fill<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(idx_d, sim_d, recip, wrev, g->row_ptr, own, cursor, n, k, gamma,
                                                       sym, g->col, g->val);
     HD_CHECK_LAUNCH(ctx);
-    rc = hd_sort_rows(ctx, g->row_ptr, g->col, g->val, n);
+    rc = hd_sort_rows(ctx, g->row_ptr, g->col, g->val, n, longest);
     if (!rc) rc = hd_normalize_graph(ctx, g);
     const int rs = hd_check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "graph", __FILE__, __LINE__);
     if (!rc) rc = rs;

@@ -48,3 +48,20 @@ def test_long_rows_take_no_quadratic_time(gpu_ctx):
     hd.graph_from_csr(gpu_ctx, rp, col, val).close()
     torch.cuda.synchronize()
     assert time.perf_counter() - t0 < 0.2
+
+
+@pytest.mark.parametrize("n", [400, 513, 700])
+def test_a_node_that_every_other_picks(gpu_ctx, n):
+    # the union graph's row of that node is as long as the graph, on both sides of the sort's limit
+    import torch
+    import paper_1807_08692_gb300 as hd
+    rng = np.random.default_rng(n)
+    X = np.zeros((n, 8), np.float32)
+    X[:, 1:] = rng.integers(-1, 2, (n, 7))
+    X[:, 0] = 1.0
+    X[0, 0] = 100.0
+    X[0, 1:] = 0.0
+    rp, col, val, dinv = hd.build_graph(gpu_ctx, torch.from_numpy(X).cuda(), 3, 1.0).export()
+    assert rp[1] - rp[0] == n - 1
+    for i in range(n):
+        assert np.all(np.diff(col[rp[i]:rp[i + 1]]) > 0), i
